@@ -219,12 +219,22 @@ inline uint64_t table_slot_bytes(int k) {
 // Bytes per candidate record (a global position).
 inline uint64_t cand_record_bytes(int) { return 8; }
 
-// The k > 63 halves of launch_round and of the partition pre-pass (compiled
-// in twopaco_kernels_wide.cu).
-int launch_round_wide(const RunView& v, int round, int rounds, cudaStream_t s,
-                      const std::vector<std::pair<uint64_t, uint64_t>>* ranges);
-int launch_partition_count_wide(const RunView& v, cudaStream_t s);
-int launch_class_map_wide(const RunView& v, cudaStream_t s);
+// The parts of launch_round, the partition pre-pass and the class map, one
+// translation unit each (see the head of twopaco_kernels.cu).
+using PartRanges = std::vector<std::pair<uint64_t, uint64_t>>;
+int launch_round_1(const RunView& v, int round, int rounds, cudaStream_t s, const PartRanges* ranges);
+int launch_round_2(const RunView& v, int round, int rounds, cudaStream_t s, const PartRanges* ranges);
+int launch_round_3(const RunView& v, int round, int rounds, cudaStream_t s, const PartRanges* ranges);
+int launch_round_4(const RunView& v, int round, int rounds, cudaStream_t s, const PartRanges* ranges);
+int launch_round_5(const RunView& v, int round, int rounds, cudaStream_t s, const PartRanges* ranges);
+int launch_count_1(const RunView& v, cudaStream_t s);
+int launch_count_2(const RunView& v, cudaStream_t s);
+int launch_count_3(const RunView& v, cudaStream_t s);
+int launch_count_4(const RunView& v, cudaStream_t s);
+int launch_count_5(const RunView& v, cudaStream_t s);
+int launch_map_1(const RunView& v, cudaStream_t s);
+int launch_map_3(const RunView& v, cudaStream_t s);
+int launch_map_5(const RunView& v, cudaStream_t s);
 
 // Digest of a run's input into hdr->input_digest: an order-free sum over the
 // packed words (the bases), the n_seqs + 1 string offsets (the boundaries,

@@ -25,10 +25,13 @@
 #include <type_traits>
 #include <vector>
 
-// This file is compiled twice: on its own (every kernel but the k > 63
-// ones, and the library's entry points), and with TWOPACO_WIDE_ONLY from
-// twopaco_kernels_wide.cu (only the k > 63 instances, launch_round_wide and
-// launch_partition_count_wide), so that the two halves build in parallel.
+// This file is compiled several times, so that its many instances build in
+// parallel: on its own (the kernels that are no template of the k-mer width
+// and the bits per item, and the library's entry points), and with
+// TWOPACO_PART from the small files beside it, for the rounds, the class map
+// and the partition pre-pass of one k-mer width and half of the bits per item:
+//   1, 2  k <= 31, 1-4 and 5-8 bits      3, 4  k <= 63, 1-4 and 5-8 bits
+//   5     k <= 127, the bits a run-time value
 
 namespace twopaco {
 
@@ -43,7 +46,7 @@ extern std::mutex g_prof_mu;
 extern bool g_prof_on;
 extern std::vector<ProfRecord> g_prof;
 extern std::vector<cudaEvent_t> g_event_pool;
-#ifndef TWOPACO_WIDE_ONLY
+#ifndef TWOPACO_PART
 std::atomic<unsigned long long> g_launches{0};
 std::mutex g_prof_mu;
 bool g_prof_on = false;
@@ -205,14 +208,19 @@ __device__ __forceinline__ uint32_t base_at(const uint32_t* __restrict__ packed,
   return (__ldg(packed + (g >> 4)) >> (30u - 2u * (uint32_t)(g & 15))) & 3u;
 }
 
-// 32 bases starting at base g, first base in the two most significant bits.
+// 16 bases starting at base g, first base in the two most significant bits.
+__device__ __forceinline__ uint32_t bases16(const uint32_t* __restrict__ packed, uint64_t g) {
+  const uint32_t* p = packed + (g >> 4);
+  return __funnelshift_l(__ldg(p + 1), __ldg(p), 2u * (uint32_t)(g & 15));
+}
+
+// 32 bases starting at base g, first base in the two most significant bits
+// (the word after the window is read too: the packed input ends in pad words).
 __device__ __forceinline__ uint64_t bases32(const uint32_t* __restrict__ packed, uint64_t g) {
   const uint32_t* p = packed + (g >> 4);
   const uint32_t o2 = 2u * (uint32_t)(g & 15);
-  const uint32_t w0 = __ldg(p), w1 = __ldg(p + 1);
-  uint64_t a = ((uint64_t)w0 << 32) | w1;
-  if (o2) a = (a << o2) | (__ldg(p + 2) >> (32u - o2));
-  return a;
+  const uint32_t w0 = __ldg(p), w1 = __ldg(p + 1), w2 = __ldg(p + 2);
+  return ((uint64_t)__funnelshift_l(w1, w0, o2) << 32) | __funnelshift_l(w2, w1, o2);
 }
 
 // The k-mer starting at base g. KW = 1 for k <= 31 (one 64-bit word), 2 for
@@ -362,34 +370,31 @@ template <int KW>
 struct OccT {
   KeyT<KW> key;    // normalized k-mer
   uint64_t H;      // key_hash(key)
-  uint32_t items;  // filter items this occurrence inserts (bit j = item j)
+  uint32_t j1, j2; // filter items this occurrence inserts (equal but for a palindrome)
   uint32_t tbits;  // pass-2 bits: in-bases 0-3, out-bases 4-7, sentinel 8
   bool sentinel;   // first or last k-mer of its string
   bool rc;         // the string reads the reverse complement of key here
 };
 
+// The (predecessor, successor) item of an occurrence, read in the k-mer's own
+// orientation (jf) and on the other strand (jr = 4 (3 - succ) + (3 - pred)).
+__device__ __forceinline__ uint32_t item_forward(uint32_t pred, uint32_t succ) { return 4u * pred + succ; }
+__device__ __forceinline__ uint32_t item_reverse(uint32_t pred, uint32_t succ) { return 15u - 4u * succ - pred; }
+
+// Pass-2 bits of an item (16: the sentinel item).
+__device__ __forceinline__ uint32_t item_tbits(uint32_t j) {
+  return j == 16u ? 1u << 8 : (1u << (j >> 2)) | (16u << (j & 3u));
+}
+
 // The filter items and pass-2 bits of one occurrence: its (predecessor,
 // successor) pair read in the orientation of the normalized form (both
 // orientations of a palindrome), or the sentinel item and bit.
 __device__ __forceinline__ void occ_bits(uint32_t pred, uint32_t succ, bool use_f, bool use_r, bool sentinel,
-                                         uint32_t* items_out, uint32_t* tbits_out) {
-  if (sentinel) {
-    *items_out = 1u << 16;
-    *tbits_out = 1u << 8;
-    return;
-  }
-  uint32_t items = 0, tb = 0;
-  if (use_f) {
-    items |= 1u << (4 * pred + succ);
-    tb |= (1u << pred) | (16u << succ);
-  }
-  if (use_r) {
-    const uint32_t a = 3u - succ, c = 3u - pred;  // predecessor / successor on the other strand
-    items |= 1u << (4 * a + c);
-    tb |= (1u << a) | (16u << c);
-  }
-  *items_out = items;
-  *tbits_out = tb;
+                                         uint32_t* j1, uint32_t* j2, uint32_t* tbits) {
+  const uint32_t jf = item_forward(pred, succ), jr = item_reverse(pred, succ);
+  *j1 = sentinel ? 16u : (use_f ? jf : jr);
+  *j2 = sentinel ? 16u : (use_r ? jr : jf);
+  *tbits = item_tbits(*j1) | item_tbits(*j2);
 }
 
 template <int KW>
@@ -401,7 +406,7 @@ __device__ __forceinline__ void make_occ(const RunView& v, const KeyT<KW>& f, co
   oc->H = key_hash<KW>(oc->key);
   oc->sentinel = sentinel;
   oc->rc = !use_f;
-  occ_bits(pred, succ, use_f, use_r, sentinel, &oc->items, &oc->tbits);
+  occ_bits(pred, succ, use_f, use_r, sentinel, &oc->j1, &oc->j2, &oc->tbits);
 }
 
 // The occurrence at global position g, read from scratch; false if no k-mer
@@ -439,20 +444,123 @@ __device__ __forceinline__ void read_listed(const RunView& v, uint64_t g, bool s
   make_occ<KW>(v, f, r, pred, succ, sentinel, oc);
 }
 
-// Visit the R consecutive positions p0 .. p0 + R - 1 (p0 < m), rolling the
-// k-mer from each position to the next within a string and reading it from
-// scratch after a string boundary. fn(i, p, valid, occ) runs for every i,
-// with i a compile-time constant once unrolled.
+// A k-mer as 2 KW 32-bit words, w[0] the most significant.
+template <int KW>
+struct Words {
+  uint32_t w[2 * KW];
+};
+
+template <int KW>
+__device__ __forceinline__ Words<KW> to_words(const KeyT<KW>& x) {
+  Words<KW> y;
+  if constexpr (KW == 4) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      y.w[2 * i] = (uint32_t)(x.w[i] >> 32);
+      y.w[2 * i + 1] = (uint32_t)x.w[i];
+    }
+  } else {
+    if constexpr (KW == 2) {
+      y.w[0] = (uint32_t)(x.hi >> 32);
+      y.w[1] = (uint32_t)x.hi;
+    }
+    y.w[2 * KW - 2] = (uint32_t)(x.lo >> 32);
+    y.w[2 * KW - 1] = (uint32_t)x.lo;
+  }
+  return y;
+}
+
+template <int KW>
+__device__ __forceinline__ KeyT<KW> from_words(const Words<KW>& y) {
+  KeyT<KW> x;
+  if constexpr (KW == 4) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x.w[i] = ((uint64_t)y.w[2 * i] << 32) | y.w[2 * i + 1];
+  } else {
+    x.hi = KW == 2 ? ((uint64_t)y.w[0] << 32) | y.w[1] : 0ull;
+    x.lo = ((uint64_t)y.w[2 * KW - 2] << 32) | y.w[2 * KW - 1];
+  }
+  return x;
+}
+
+// Visit the R consecutive positions p0 .. p0 + R - 1, all of them inside one
+// string and none its first or last k-mer. Instead of rolling two k-mers from
+// position to position (a serial chain of 64-bit shifts, masks and inserts of
+// single bases), the forward k-mer and its reverse complement are each one
+// word longer than the k-mer -- the R successor bases appended at their ends --
+// and every position cuts its two k-mers out by funnel shifts of a
+// compile-time distance: one per 32-bit word, and independent of each other.
+// The integer instructions are what bounds every kernel that walks.
 template <int KW, int R, typename F>
-__device__ __forceinline__ void walk(const RunView& v, uint64_t p0, F&& fn) {
+__device__ __forceinline__ void walk_inside(const RunView& v, uint64_t p0, F&& fn) {
+  constexpr int W = 2 * KW;
+  const int k = v.k;
+  const KeyT<KW> f0 = load_kmer<KW>(v.packed, p0, k);
+  const uint32_t next = bases16(v.packed, p0 + (uint64_t)k);
+  const uint32_t before = bases16(v.packed, p0 - 1);  // predecessors of the positions
+  const Words<KW> f = to_words<KW>(f0);
+  const Words<KW> r = to_words<KW>(revcomp<KW>(f0, k));
+  // mask of 2 k bits; only the upper half can hold bits beyond them (the whole of a k <= 31 word)
+  uint32_t mask[W], rx[W + 1];
+#pragma unroll
+  for (int j = 0; j < W; ++j) {
+    const int bits = 2 * k - 32 * (W - 1 - j);  // of word j
+    mask[j] = bits >= 32 ? 0xFFFFFFFFu : (bits <= 0 ? 0u : (1u << bits) - 1u);
+  }
+  // the complements of the successor bases, the first lowest, above the 2 k bits of r
+  const uint32_t t = (uint32_t)(rev_pairs(~(uint64_t)next) >> 32);
+  rx[0] = 0;
+#pragma unroll
+  for (int j = 0; j < W; ++j) rx[j + 1] = r.w[j];
+  const int at = (2 * k) >> 5, sh = (2 * k) & 31;  // rx[W - at] is the word that holds bit 2 k
+#pragma unroll
+  for (int j = 0; j <= W; ++j) {
+    if (j == W - at) rx[j] |= t << sh;
+    if (j == W - at - 1) rx[j] |= __funnelshift_l(t, 0u, sh);
+  }
+  const bool may_be_palindrome = !(k & 1);
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    Words<KW> fi, ri;
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+      fi.w[j] = __funnelshift_l(j + 1 < W ? f.w[j + 1] : next, f.w[j], 2 * i);
+      ri.w[j] = __funnelshift_r(rx[j + 1], rx[j], 2 * i);
+      if (KW == 1 || j < W / 2) {
+        fi.w[j] &= mask[j];
+        ri.w[j] &= mask[j];
+      }
+    }
+    const KeyT<KW> kf = from_words<KW>(fi), kr = from_words<KW>(ri);
+    const bool use_r = v.both && key_less(kr, kf);
+    OccT<KW> oc;
+    oc.key = use_r ? kr : kf;
+    oc.H = key_hash<KW>(oc.key);
+    oc.sentinel = false;
+    oc.rc = use_r;
+    // the item from the bases before and after, or their complements after and before
+    const uint32_t x = (use_r ? ~next : before) >> (30 - 2 * i), y = (use_r ? ~before : next) >> (30 - 2 * i);
+    oc.j1 = oc.j2 = ((x & 3u) << 2) | (y & 3u);
+    if (may_be_palindrome && v.both && !use_r && !key_less(kf, kr))
+      oc.j2 = item_reverse((before >> (30 - 2 * i)) & 3u, (next >> (30 - 2 * i)) & 3u);
+    oc.tbits = item_tbits(oc.j1) | item_tbits(oc.j2);
+    fn(i, p0 + i, true, oc);
+  }
+}
+
+// Visit the R consecutive positions p0 .. p0 + R - 1 (p0 < m), a string (or
+// piece) boundary or the input's end among them: rolling the k-mer from each
+// position to the next within a string and reading it from scratch after a
+// string boundary. b: the bounds at p0.
+template <int KW, int R, typename F>
+__device__ __forceinline__ void walk_edges(const RunView& v, uint64_t p0, Bounds b, F&& fn) {
   static_assert(R >= 1 && R <= 16, "successor bases come from one 32-bit word");
   const int k = v.k;
-  Bounds b = kmer_bounds(v, p0);
   int32_t s_rel = rel(b.start, p0), e_rel = rel(b.end, p0);  // string bounds relative to p0
   const int32_t m_rel = rel(v.m, p0);
   // bases p0 + k .. p0 + k + R - 1: the successor of each position, which is
   // also the base that enters the k-mer when it slides to the next position
-  const uint32_t next = (uint32_t)(bases32(v.packed, p0 + (uint64_t)k) >> 32);
+  const uint32_t next = bases16(v.packed, p0 + (uint64_t)k);
   KeyT<KW> f{}, r{};
   bool fresh = true;
 #pragma unroll
@@ -488,6 +596,16 @@ __device__ __forceinline__ void walk(const RunView& v, uint64_t p0, F&& fn) {
     }
     fn(i, p, valid, oc);
   }
+}
+
+
+// Visit the R consecutive positions p0 .. p0 + R - 1 (p0 < m): fn(i, p, valid,
+// occ) runs for every i, with i a compile-time constant once unrolled.
+template <int KW, int R, typename F>
+__device__ __forceinline__ void walk(const RunView& v, uint64_t p0, F&& fn) {
+  const Bounds b = kmer_bounds(v, p0);
+  if (b.start < p0 && p0 + (uint64_t)(R - 1 + v.k) < b.end) walk_inside<KW, R>(v, p0, fn);
+  else walk_edges<KW, R>(v, p0, b, fn);
 }
 
 __device__ __forceinline__ bool in_round(const RunView& v, uint64_t H, int round) {
@@ -1191,10 +1309,9 @@ __global__ void __launch_bounds__(kBlock) pass1_insert_kernel(RunView v, int rou
           } else {
             const uint64_t G = second_hash(oc.H);
             const ItemPattern pat = item_pattern<HB>(G, v.hashes);
-            const uint32_t j1 = __ffs(oc.items) - 1, j2 = 31 - __clz(oc.items);
-            uint64_t m = item_bits(pat, j1);
-            if (j2 != j1) m |= item_bits(pat, j2);  // a palindrome's two orientations
-            if (BKT) stage_or(v, filter_index(v, oc.H, G), G, j1, j2, m);
+            uint64_t m = item_bits(pat, oc.j1);
+            if (oc.j2 != oc.j1) m |= item_bits(pat, oc.j2);  // a palindrome's two orientations
+            if (BKT) stage_or(v, filter_index(v, oc.H, G), G, oc.j1, oc.j2, m);
             else atomicOr(filter_word(v, oc.H, G), (unsigned long long)m);
             if (DESC) d = make_desc(v, oc.H, G, oc.sentinel);
           }
@@ -1580,10 +1697,9 @@ __global__ void __launch_bounds__(kBlock) pass1_insert_cm_kernel(RunView v, int 
       read_listed<KW>(v, wbase + (e & 511u), (e >> 9) & 1u, &oc);
       const uint64_t G = second_hash(oc.H);
       const ItemPattern pat = item_pattern<HB>(G, v.hashes);
-      const uint32_t j1 = __ffs(oc.items) - 1, j2 = 31 - __clz(oc.items);
-      uint64_t m = item_bits(pat, j1);
-      if (j2 != j1) m |= item_bits(pat, j2);  // a palindrome's two orientations
-      if (BKT) stage_or(v, filter_index(v, oc.H, G), G, j1, j2, m);
+      uint64_t m = item_bits(pat, oc.j1);
+      if (oc.j2 != oc.j1) m |= item_bits(pat, oc.j2);  // a palindrome's two orientations
+      if (BKT) stage_or(v, filter_index(v, oc.H, G), G, oc.j1, oc.j2, m);
       else atomicOr(filter_word(v, oc.H, G), (unsigned long long)m);
     }
     __syncwarp();
@@ -1727,7 +1843,7 @@ __device__ __forceinline__ unsigned long long fused_record(const RunView& v, uin
 
 struct FusedOcc {
   uint64_t key, H, G;
-  uint32_t items, tbits;
+  uint32_t j1, j2, tbits;
   bool sentinel;
 };
 
@@ -1735,7 +1851,7 @@ __device__ __forceinline__ FusedOcc fused_occ(unsigned long long rec) {
   FusedOcc o;
   o.key = rec >> 7;
   o.sentinel = (rec >> 6) & 1u;
-  occ_bits((uint32_t)(rec >> 2) & 3u, (uint32_t)rec & 3u, (rec >> 4) & 1u, (rec >> 5) & 1u, o.sentinel, &o.items,
+  occ_bits((uint32_t)(rec >> 2) & 3u, (uint32_t)rec & 3u, (rec >> 4) & 1u, (rec >> 5) & 1u, o.sentinel, &o.j1, &o.j2,
            &o.tbits);
   o.H = mix64(o.key);  // key_hash of a one-word k-mer
   o.G = second_hash(o.H);
@@ -2047,7 +2163,7 @@ __global__ void __launch_bounds__(kBlock) ord_scatter_kernel(RunView v, int roun
           OccT<KW> oc;
           read_listed<KW>(v, wbase + (e & 511u), sentinel, &oc);
           const uint64_t G = second_hash(oc.H);
-          const uint32_t j1 = __ffs(oc.items) - 1, j2 = 31 - __clz(oc.items);
+          const uint32_t j1 = oc.j1, j2 = oc.j2;
           const uint64_t word = filter_index(v, oc.H, G);
           rec = (word & local_mask) | (((G >> 32) & 0x3FFFFFFFull) << 22) | ((uint64_t)j1 << 52) |
                 ((uint64_t)j2 << 57) | (sentinel ? kOrdSentinel : 0ull);
@@ -2143,9 +2259,8 @@ __global__ void __launch_bounds__(kBlock) ord_or_kernel(RunView v) {
         if constexpr (FUSED) {
           const FusedOcc o = fused_occ(r[u]);
           const ItemPattern pat = item_pattern<HB>(o.G, v.hashes);
-          const uint32_t j1 = __ffs(o.items) - 1, j2 = 31 - __clz(o.items);
-          uint64_t m = item_bits(pat, j1);
-          if (j2 != j1) m |= item_bits(pat, j2);
+          uint64_t m = item_bits(pat, o.j1);
+          if (o.j2 != o.j1) m |= item_bits(pat, o.j2);
           atomicOr(v.filter + filter_index(v, o.H, o.G), (unsigned long long)m);
         } else {
           const uint64_t G = ((r[u] >> 22) & 0x3FFFFFFFull) << 32;  // the bits bit_base reads for u < 6
@@ -3104,7 +3219,7 @@ int done(int n) {
 
 }  // namespace
 
-#ifndef TWOPACO_WIDE_ONLY
+#ifndef TWOPACO_PART
 void count_launches(int n) { g_launches.fetch_add((unsigned long long)n); }
 unsigned long long launches_so_far() { return g_launches.load(); }
 
@@ -3146,54 +3261,30 @@ int launch_pack_finish(const RunView& v, cudaStream_t s) {
   return done(5);
 }
 
-#endif  // TWOPACO_WIDE_ONLY
+#else   // TWOPACO_PART
 
-// Run f with the filter's bits per item as a compile-time constant.
+constexpr int kPartKw = TWOPACO_PART == 5 ? 4 : (TWOPACO_PART <= 2 ? 1 : 2);
+constexpr bool kPartHigh = TWOPACO_PART == 2 || TWOPACO_PART == 4;
+
+// Run f with the filter's bits per item as a compile-time constant (0 at
+// k > 63: a run-time value).
 template <typename F>
-void with_hashes(int h, F&& f) {
-  switch (h) {
-    case 1: f(std::integral_constant<int, 1>{}); break;
-    case 2: f(std::integral_constant<int, 2>{}); break;
-    case 3: f(std::integral_constant<int, 3>{}); break;
-    case 4: f(std::integral_constant<int, 4>{}); break;
-    case 5: f(std::integral_constant<int, 5>{}); break;
-    case 6: f(std::integral_constant<int, 6>{}); break;
-    case 7: f(std::integral_constant<int, 7>{}); break;
-    default: f(std::integral_constant<int, 8>{}); break;
-  }
-}
-
-#ifndef TWOPACO_WIDE_ONLY
-int launch_partition(const RunView& v, int rounds, cudaStream_t s) {
-  if (v.m == 0) return 0;
-  // the filter is clear (pack kernel); the pre-pass uses it, round 0 clears it again
-  if (cudaMemsetAsync(v.bins, 0, (uint64_t)(v.qmask + 1u) * 4, s) != cudaSuccess) return -1;
-  const uint64_t threads = (v.m + kR - 1) / kR;
-  {
-    Timed t("partition_count", s);
-    if (v.k > 63) {
-      if (launch_partition_count_wide(v, s) < 0) return -1;
-    } else {
-      with_hashes(v.hashes, [&](auto hb) {
-        constexpr int HB = decltype(hb)::value;
-        if (v.k <= 31)
-          partition_count_kernel<1, HB><<<grid_for(partition_count_kernel<1, HB>, kBlock, threads), kBlock, 0, s>>>(v);
-        else
-          partition_count_kernel<2, HB><<<grid_for(partition_count_kernel<2, HB>, kBlock, threads), kBlock, 0, s>>>(v);
-      });
+static void with_hashes(int h, F&& f) {
+  if constexpr (kPartKw == 4) {
+    f(std::integral_constant<int, 0>{});
+  } else {
+    constexpr int B = kPartHigh ? 4 : 0;
+    switch (h - B) {
+      case 1: f(std::integral_constant<int, B + 1>{}); break;
+      case 2: f(std::integral_constant<int, B + 2>{}); break;
+      case 3: f(std::integral_constant<int, B + 3>{}); break;
+      default: f(std::integral_constant<int, B + 4>{}); break;
     }
   }
-  uint64_t* prefix = reinterpret_cast<uint64_t*>(v.bins + (v.qmask + 1u));
-  {
-    Timed t("partition_cut", s);
-    partition_cut_kernel<<<1, 1024, 0, s>>>(v, rounds, prefix);
-  }
-  return done(2);
 }
-#endif  // TWOPACO_WIDE_ONLY
 
 template <int KW, bool RD, int HB, int TS>
-int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges* ranges) {
+static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges* ranges) {
   // the pack kernel cleared the filter and the LC bitmap for round 0; the
   // partition pre-pass (rounds > 1) uses the filter before round 0
   if (RD && cudaMemsetAsync(v.filter, 0, v.filter_words64 * 8, s) != cudaSuccess) return -1;
@@ -3358,43 +3449,109 @@ int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges* ranges
   return done(launched);
 }
 
-#ifndef TWOPACO_WIDE_ONLY
-int launch_round(const RunView& v, int round, int rounds, cudaStream_t s, const Ranges* ranges) {
-  if (v.m == 0) return 0;
-  if (v.k > 63) return launch_round_wide(v, round, rounds, s, ranges);
+static int part_round(const RunView& v, int round, int rounds, cudaStream_t s, const Ranges* ranges) {
   int rc = 0;
   with_hashes(v.hashes, [&](auto hb) {
     constexpr int HB = decltype(hb)::value;
-    const int ts = table_slot_kind(v.k);
-    if (ts == 0)
-      rc = rounds > 1 ? round_impl<1, true, HB, 0>(v, round, s, ranges) : round_impl<1, false, HB, 0>(v, round, s, ranges);
-    else if (ts == 1)
-      rc = rounds > 1 ? round_impl<1, true, HB, 1>(v, round, s, ranges) : round_impl<1, false, HB, 1>(v, round, s, ranges);
-    else
-      rc = rounds > 1 ? round_impl<2, true, HB, 2>(v, round, s, ranges) : round_impl<2, false, HB, 2>(v, round, s, ranges);
+    auto go = [&](auto ts) {
+      constexpr int TS = decltype(ts)::value;
+      rc = rounds > 1 ? round_impl<kPartKw, true, HB, TS>(v, round, s, ranges)
+                      : round_impl<kPartKw, false, HB, TS>(v, round, s, ranges);
+    };
+    if constexpr (kPartKw == 1) {
+      if (table_slot_kind(v.k) == 0) go(std::integral_constant<int, 0>{});
+      else go(std::integral_constant<int, 1>{});
+    } else {
+      go(std::integral_constant<int, kPartKw == 2 ? 2 : 3>{});
+    }
   });
   return rc;
 }
 
+static int part_count(const RunView& v, cudaStream_t s) {
+  const uint64_t threads = (v.m + kR - 1) / kR;
+  with_hashes(v.hashes, [&](auto hb) {
+    auto kern = partition_count_kernel<kPartKw, decltype(hb)::value>;
+    kern<<<grid_for(kern, kBlock, threads), kBlock, 0, s>>>(v);
+  });
+  return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
+}
+
+// The parts' entry points, one set per translation unit.
+#define TWOPACO_PART_NAME2(f, p) f##p
+#define TWOPACO_PART_NAME(f, p) TWOPACO_PART_NAME2(f, p)
+int TWOPACO_PART_NAME(launch_round_, TWOPACO_PART)(const RunView& v, int round, int rounds, cudaStream_t s,
+                                                   const Ranges* ranges) {
+  return part_round(v, round, rounds, s, ranges);
+}
+int TWOPACO_PART_NAME(launch_count_, TWOPACO_PART)(const RunView& v, cudaStream_t s) { return part_count(v, s); }
+
+#if TWOPACO_PART == 1 || TWOPACO_PART == 3 || TWOPACO_PART == 5
+// The class map of this k-mer width.
+int TWOPACO_PART_NAME(launch_map_, TWOPACO_PART)(const RunView& v, cudaStream_t s) {
+  Timed t("class_map", s);
+  if constexpr (kPartKw < 4) {
+    if (v.o_regions) {
+      auto kern = class_map_ord_kernel<kPartKw>;
+      kern<<<grid_for(kern, kBlock, v.o_tiles * kBlock), kBlock, 0, s>>>(v);
+      // every tile's first member number, per round
+      const uint64_t chunks = (v.o_tiles + kOrdScanTiles - 1) / kOrdScanTiles;
+      ord_tile_sum_kernel<<<(unsigned)(chunks * v.rounds), kBlock, 0, s>>>(v, chunks);
+      ord_tile_scan_kernel<<<(unsigned)(chunks * v.rounds), kBlock, 0, s>>>(v, chunks);
+      return done(3);
+    }
+  }
+  auto kern = class_map_kernel<kPartKw>;
+  kern<<<grid_for(kern, kBlock, (v.m + kInsertR - 1) / kInsertR), kBlock, 0, s>>>(v);
+  return done(1);
+}
+#endif
+
+#endif  // TWOPACO_PART
+
+#ifndef TWOPACO_PART
+// The part that holds the instances of this run: by k-mer width, then by bits per item.
+int part_of(const RunView& v) {
+  if (v.k > 63) return 5;
+  return (v.k <= 31 ? 1 : 3) + (v.hashes > 4 ? 1 : 0);
+}
+
+int launch_round(const RunView& v, int round, int rounds, cudaStream_t s, const Ranges* ranges) {
+  if (v.m == 0) return 0;
+  switch (part_of(v)) {
+    case 1: return launch_round_1(v, round, rounds, s, ranges);
+    case 2: return launch_round_2(v, round, rounds, s, ranges);
+    case 3: return launch_round_3(v, round, rounds, s, ranges);
+    case 4: return launch_round_4(v, round, rounds, s, ranges);
+    default: return launch_round_5(v, round, rounds, s, ranges);
+  }
+}
+
+int launch_partition(const RunView& v, int rounds, cudaStream_t s) {
+  if (v.m == 0) return 0;
+  // the filter is clear (pack kernel); the pre-pass uses it, round 0 clears it again
+  if (cudaMemsetAsync(v.bins, 0, (uint64_t)(v.qmask + 1u) * 4, s) != cudaSuccess) return -1;
+  {
+    Timed t("partition_count", s);
+    const int part = part_of(v);
+    const int rc = part == 1   ? launch_count_1(v, s)
+                   : part == 2 ? launch_count_2(v, s)
+                   : part == 3 ? launch_count_3(v, s)
+                   : part == 4 ? launch_count_4(v, s)
+                               : launch_count_5(v, s);
+    if (rc < 0) return -1;
+  }
+  uint64_t* prefix = reinterpret_cast<uint64_t*>(v.bins + (v.qmask + 1u));
+  {
+    Timed t("partition_cut", s);
+    partition_cut_kernel<<<1, 1024, 0, s>>>(v, rounds, prefix);
+  }
+  return done(2);
+}
+
 int launch_class_map(const RunView& v, cudaStream_t s) {
   if (!v.cmap || v.m == 0) return 0;
-  if (v.k > 63) return launch_class_map_wide(v, s) < 0 ? -1 : done(1);
-  Timed t("class_map", s);
-  const uint64_t threads = (v.m + kInsertR - 1) / kInsertR;
-  if (v.o_regions) {
-    const unsigned grid = v.k <= 31 ? grid_for(class_map_ord_kernel<1>, kBlock, v.o_tiles * kBlock)
-                                    : grid_for(class_map_ord_kernel<2>, kBlock, v.o_tiles * kBlock);
-    if (v.k <= 31) class_map_ord_kernel<1><<<grid, kBlock, 0, s>>>(v);
-    else class_map_ord_kernel<2><<<grid, kBlock, 0, s>>>(v);
-    // every tile's first member number, per round
-    const uint64_t chunks = (v.o_tiles + kOrdScanTiles - 1) / kOrdScanTiles;
-    ord_tile_sum_kernel<<<(unsigned)(chunks * v.rounds), kBlock, 0, s>>>(v, chunks);
-    ord_tile_scan_kernel<<<(unsigned)(chunks * v.rounds), kBlock, 0, s>>>(v, chunks);
-    return done(3);
-  }
-  if (v.k <= 31) class_map_kernel<1><<<grid_for(class_map_kernel<1>, kBlock, threads), kBlock, 0, s>>>(v);
-  else class_map_kernel<2><<<grid_for(class_map_kernel<2>, kBlock, threads), kBlock, 0, s>>>(v);
-  return done(1);
+  return v.k <= 31 ? launch_map_1(v, s) : (v.k <= 63 ? launch_map_3(v, s) : launch_map_5(v, s));
 }
 
 int launch_emit(const RunView& v, cudaStream_t s, bool again) {
@@ -3434,29 +3591,11 @@ int launch_edges(const DevHeader* hdr_dev, const uint64_t* d_offsets, uint64_t n
   return done(3);
 }
 
-#else
-// k > 63: four-word k-mers, reference slots, the bits per item a run-time value.
-int launch_round_wide(const RunView& v, int round, int rounds, cudaStream_t s, const Ranges* ranges) {
-  return rounds > 1 ? round_impl<4, true, 0, 3>(v, round, s, ranges) : round_impl<4, false, 0, 3>(v, round, s, ranges);
-}
-
-int launch_partition_count_wide(const RunView& v, cudaStream_t s) {
-  const uint64_t threads = (v.m + kR - 1) / kR;
-  partition_count_kernel<4, 0><<<grid_for(partition_count_kernel<4, 0>, kBlock, threads), kBlock, 0, s>>>(v);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
-}
-
-int launch_class_map_wide(const RunView& v, cudaStream_t s) {
-  Timed t("class_map", s);
-  const uint64_t threads = (v.m + kInsertR - 1) / kInsertR;
-  class_map_kernel<4><<<grid_for(class_map_kernel<4>, kBlock, threads), kBlock, 0, s>>>(v);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
-}
-#endif  // TWOPACO_WIDE_ONLY
+#endif  // TWOPACO_PART
 
 }  // namespace twopaco
 
-#ifndef TWOPACO_WIDE_ONLY
+#ifndef TWOPACO_PART
 
 extern "C" unsigned long long twopaco_kernel_launches(void) {
   return twopaco::g_launches.load();
@@ -3506,4 +3645,4 @@ extern "C" int twopaco_profile_kernels(const char** names, unsigned long long* l
   return n;
 }
 
-#endif  // TWOPACO_WIDE_ONLY
+#endif  // TWOPACO_PART

@@ -1,5 +1,3 @@
-// The k > 63 instances of the kernels (four-word k-mers, reference slots):
-// the same source as twopaco_kernels.cu, compiled as a second translation
-// unit so that the two build in parallel.
-#define TWOPACO_WIDE_ONLY 1
+// The instances for k > 63: four-word k-mers, reference slots (see the head of twopaco_kernels.cu).
+#define TWOPACO_PART 5
 #include "twopaco_kernels.cu"
