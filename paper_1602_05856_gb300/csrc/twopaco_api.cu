@@ -309,15 +309,20 @@ RunView make_view(const uint8_t* d_bases, const uint64_t* d_offsets, uint64_t n_
   v.partial = o.partial;
   v.lg_blocks = log2_exact(filter_bits / 256);
   v.qmask = o.partition_bins - 1u;
-  // the pre-pass counts every k-mer up to 2^29 bases, then a 2^-s sample with
-  // s = floor(log2(m / 2^28)), at most 2^-8 (2^-6 at 24 Gbp)
-  int sample_log2 = 0;
-  while (sample_log2 < 8 && (m >> (28 + sample_log2 + 1)) > 0) ++sample_log2;
-  v.part_sample = (1u << sample_log2) - 1u;
-  // from 2^33 bases the pre-pass also walks only every fourth chunk of 65536
-  // positions: the walk, not the counting, is its cost, and the cut needs
-  // the bins' proportions only
-  v.part_chunks = m >= (1ull << 33) ? 3u : 0u;
+  // The pre-pass needs the proportions of the bins, not their counts: the classes
+  // are runs of bins of a hash, so a sample balances them as well. From 2^27 bases
+  // it walks a 2^-c share of the chunks of 65536 positions (at least 2^26
+  // positions, c <= 16), and of what it walks it counts a hash-chosen 2^-s of the
+  // k-mers once that is 2^24 positions and more (at least 2^22 sampled positions,
+  // s <= 8: 64 per bin of the default 65536, a class of ell = 4 to about 0.1%).
+  // Every counted k-mer is a random atomic in a filter beyond L2: on 200 M bases
+  // counting all of them took 4.2 ms of a 13.6 ms build.
+  int chunk_log2 = 0, sample_log2 = 0;
+  while (chunk_log2 < 16 && (m >> (chunk_log2 + 1)) >= (1ull << 26)) ++chunk_log2;
+  while (sample_log2 < 8 && ((m >> chunk_log2) >> (sample_log2 + 1)) >= (1ull << 22)) ++sample_log2;
+  if ((m >> chunk_log2) < (1ull << 24)) sample_log2 = 0;
+  v.part_chunks = (1u << chunk_log2) - 1u;
+  v.part_sample = ((1ull << sample_log2) - 1ull) << std::max(16, log2_exact(o.partition_bins));
   v.hdr = reinterpret_cast<DevHeader*>(base + L.header);
   v.packed = reinterpret_cast<uint32_t*>(base + L.packed);
   v.packed_words = L.packed_words;

@@ -79,8 +79,8 @@ struct RunView {
                             // ([0, m)) or, launched per string, whole tiles of kRangeTile
   int lg_blocks;            // log2(filter_bits / 256)
   uint32_t qmask;           // partition_bins - 1
-  uint32_t part_sample;     // the partition pre-pass counts the k-mers whose H has bits
-                            // 16 .. 16 + log2(part_sample + 1) - 1 all zero (0: every k-mer)
+  uint64_t part_sample;     // the partition pre-pass counts the k-mers whose H has these bits
+                            // (next to the bin's, from bit 16 up) all zero (0: every k-mer)
   uint32_t part_chunks;     // ... and walks the chunks of 65536 positions whose index has these
                             // bits zero (0: every chunk)
   DevHeader* hdr;

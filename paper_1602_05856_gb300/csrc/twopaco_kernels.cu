@@ -2770,7 +2770,7 @@ __global__ void __launch_bounds__(kBlock) partition_count_kernel(RunView v) {
   for (uint64_t p0 = ((uint64_t)blockIdx.x * kBlock + threadIdx.x) * kR; p0 < v.m; p0 += stride) {
     if ((uint32_t)(p0 >> 16) & v.part_chunks) continue;  // a sample of the 64K-position chunks
     walk<KW, kR>(v, p0, [&](int, uint64_t, bool valid, const auto& oc) {
-      if (!valid || ((uint32_t)(oc.H >> 16) & v.part_sample)) return;
+      if (!valid || (oc.H & v.part_sample)) return;
       const uint64_t G = second_hash(oc.H);
       const uint64_t m = item_bits<HB>(G, 17u, v.hashes);
       unsigned long long* w = filter_word(v, oc.H, G);
@@ -2786,46 +2786,60 @@ __global__ void __launch_bounds__(kBlock) partition_count_kernel(RunView v) {
 // leaving one bin for every later class; the last class takes the rest.
 __global__ void __launch_bounds__(1024) partition_cut_kernel(RunView v, int rounds, uint64_t* prefix) {
   const uint32_t q = v.qmask + 1u;
-  __shared__ unsigned long long carry_s;
-  __shared__ unsigned long long wsum[32];
-  if (threadIdx.x == 0) carry_s = 0;
-  __syncthreads();
-  for (uint32_t base = 0; base < q; base += 1024) {
-    const uint32_t i = base + threadIdx.x;
-    unsigned long long x = (i < q) ? v.bins[i] : 0ull, inc = x;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
+  // each thread sums and then scans its own run of bins: one block scan, not one
+  // per 1024 bins; the runs' starts stay in shared memory for the search
+  __shared__ unsigned long long wsum[32], start_s[1025];
+  const uint32_t per = (q + 1023u) / 1024u, i0 = min(q, threadIdx.x * per), i1 = min(q, i0 + per);
+  const bool vec = per % 4 == 0;  // whole 16-byte groups (q is a power of two)
+  unsigned long long x = 0;
+  if (vec) {
+#pragma unroll 8
+    for (uint32_t i = i0; i < i1; i += 4) {
+      const uint4 e = *reinterpret_cast<const uint4*>(v.bins + i);
+      x += (unsigned long long)e.x + e.y + e.z + e.w;
     }
-    if (lane == 31) wsum[wid] = inc;
-    __syncthreads();
-    unsigned long long before = 0, all = 0;
-    for (int w = 0; w < 32; ++w) {
-      before += (w < wid) ? wsum[w] : 0ull;
-      all += wsum[w];
-    }
-    const unsigned long long c0 = carry_s;
-    if (i < q) prefix[i] = c0 + before + inc - x;
-    __syncthreads();
-    if (threadIdx.x == 0) carry_s = c0 + all;
-    __syncthreads();
+  } else {
+    for (uint32_t i = i0; i < i1; ++i) x += v.bins[i];
   }
+  unsigned long long inc = x;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) wsum[wid] = inc;
+  __syncthreads();
+  unsigned long long at = inc - x;
+  for (int w = 0; w < wid; ++w) at += wsum[w];
+  start_s[threadIdx.x] = at;
+  if (threadIdx.x == 1023) start_s[1024] = at + x;
+#pragma unroll 8
+  for (uint32_t i = i0; i < i1; ++i) {
+    prefix[i] = at;
+    at += v.bins[i];
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned long long total = carry_s;
+    const unsigned long long total = start_s[1024];
     prefix[q] = total;
     const unsigned long long L = (unsigned long long)rounds;
     uint32_t j = 0;
+    unsigned long long before = 0;  // prefix[j]
     v.cuts[0] = 0;
     for (int r = 0; r < rounds - 1; ++r) {
-      const uint32_t start = j;
       const uint32_t limit = q - (uint32_t)(rounds - 1 - r);
-      // largest e in [start+1, limit] with (prefix[e] - prefix[start]) * L <= total
-      uint32_t lo = start + 1, hi = limit, best = start + 1;
+      // largest e in [j + 1, limit] with (prefix[e] - prefix[j]) * L <= total (at least
+      // j + 1): first the last run of bins that starts within it, then inside that run
+      uint32_t a = 0, z = 1024;  // run a starts within it (or is j's), run z does not or is past the end
+      while (z - a > 1) {
+        const uint32_t mid = (a + z) / 2;
+        if ((uint64_t)mid * per <= j || (start_s[mid] - before) * L <= total) a = mid; else z = mid;
+      }
+      uint32_t lo = max(j + 1, min(a * per, limit)), hi = min(limit, (a + 1) * per), best = j + 1;
       while (lo <= hi) {
         const uint32_t mid = lo + (hi - lo) / 2;
-        if ((prefix[mid] - prefix[start]) * L <= total) {
+        if ((prefix[mid] - before) * L <= total) {
           best = mid;
           lo = mid + 1;
         } else {
@@ -2833,6 +2847,7 @@ __global__ void __launch_bounds__(1024) partition_cut_kernel(RunView v, int roun
         }
       }
       j = best;
+      before = prefix[j];
       v.cuts[r + 1] = j;
     }
     v.cuts[rounds] = q;
