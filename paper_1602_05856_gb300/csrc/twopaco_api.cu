@@ -109,6 +109,7 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
   L.bitmap_words = (m + 31) / 32;
   L.n_tiles = (L.bitmap_words + kEmitTileWords - 1) / kEmitTileWords;
   L.table_slots = o.table_slots ? next_pow2(o.table_slots) : auto_table_slots(m, rounds);
+  if (L.table_slots < 4) L.table_slots = 4;  // probing reads sectors of four slots
   if (o.partial) L.table_slots = 0;  // no second pass: no table, list or kept slots
   // 32-bit candidate records (31-bit positions and a sentinel flag) below 2^31 bases
   L.narrow = (m < (1ull << 31) && o.wide_layout == 0) ? 1 : 0;
@@ -352,7 +353,10 @@ RunView make_view(const uint8_t* d_bases, const uint64_t* d_offsets, uint64_t n_
   }
   v.cand_cap = L.cand_cap;
   v.lc_bits = reinterpret_cast<uint32_t*>(base + L.lc);
-  v.lc_log2 = L.lc_log2;
+  // linear counting on an eighth of the k-mers, in an eighth of the bits, from 2^20
+  // bits (a million candidates' room) up, and on a 32nd from 2^24
+  v.lc_sample_log2 = L.lc_log2 >= 24 ? 5 : (L.lc_log2 >= 20 ? 3 : 0);
+  v.lc_log2 = L.lc_log2 - v.lc_sample_log2;
   v.seg_count = reinterpret_cast<uint32_t*>(base + L.segs);
   v.bins = rounds > 1 ? reinterpret_cast<uint32_t*>(base + L.bins) : nullptr;
   v.cuts = reinterpret_cast<uint32_t*>(base + L.cuts);
@@ -388,8 +392,6 @@ RunView make_view(const uint8_t* d_bases, const uint64_t* d_offsets, uint64_t n_
     v.o_perm = reinterpret_cast<uint16_t*>(base + L.operm);
     v.o_fused = L.o_fused;
     v.o_tcap = L.o_tcap;
-    // large rounds count distinct candidates on an eighth of the k-mers
-    v.lc_sample_log2 = L.o_rec_cap >= (1ull << 26) ? 3 : 0;
   }
   v.tile_count = reinterpret_cast<uint32_t*>(base + L.tile_count);
   v.tile_prefix = reinterpret_cast<uint64_t*>(base + L.tile_prefix);

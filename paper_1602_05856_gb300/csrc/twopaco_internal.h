@@ -19,10 +19,10 @@ struct DevHeader {
   unsigned long long round_kept;   // candidates after pass 1, current round
   unsigned long long table_slots;  // pass-2 table capacity of the current round
   unsigned long long table_max;    // largest capacity used by any round
-  unsigned long long lc_set;       // linear-counting bits set this round
+  unsigned long long reserved2;
   unsigned int cand_overflow;      // a warp's list segment ran out of room this round
   unsigned int round_listed;       // pass 2 of this round reads the list (else C_temp)
-  unsigned int lc_blocks_done;     // blocks of lc_count finished this round
+  unsigned int reserved;
   unsigned int list_parts;         // pass-2 parts per list segment this round
   unsigned long long emit_ticket;  // next emit tile to claim
   unsigned int overflow;           // the pass-2 table or a boundary list out of room
@@ -151,7 +151,7 @@ struct RunView {
   uint64_t seg_cap;         // records per segment (set per launch)
   uint32_t* lc_bits;        // linear-counting bitmap, 2^lc_log2 bits
   int lc_log2;
-  int lc_sample_log2;       // region-ordered rounds count a 2^-lc_sample_log2 sample of the k-mers
+  int lc_sample_log2;       // linear counting counts a 2^-lc_sample_log2 sample of the k-mers
   uint32_t* bins;           // partition counters (q), rounds > 1
   uint32_t* cuts;           // rounds + 1 class boundaries
   uint8_t* cmap;            // class map, one byte per position (null: rounds walk every position)

@@ -96,11 +96,7 @@ struct Timed {
 // bases) in the first-pass kernels and the partition pre-pass.
 constexpr int kInsertR = 16;
 constexpr int kProbeR = 8;
-// Loads issued one step ahead (measured: the probe's descriptors and the
-// classify's records gain; the second-pass insert's records lose).
-constexpr bool kProbePrefetch = true;
-constexpr bool kInsertPrefetch = false;
-constexpr bool kClassifyPrefetch = true;
+constexpr bool kProbePrefetch = true;  // the probe's descriptors loaded one step ahead
 constexpr int kR = 8;  // partition pre-pass
 
 using Ranges = std::vector<std::pair<uint64_t, uint64_t>>;
@@ -187,16 +183,15 @@ __device__ __forceinline__ uint64_t second_hash(uint64_t H) { return H * 0x9e377
 // Start slot of a k-mer in the pass-2 table (bits above the partition bins).
 __device__ __forceinline__ uint64_t slot_hash(uint64_t H) { return H >> 16; }
 
-// Start slot of a k-mer in a pass-2 table of cap slots (any capacity): bits
-// 16-47 of H scaled to [0, cap) by a multiply-high (Lemire, "Fast random
-// integer generation in an interval", 2019); larger tables take a remainder.
+// Start slot of a k-mer in a pass-2 table of cap slots: bits 16-47 of H scaled
+// to [0, cap) by a multiply-high (Lemire, "Fast random integer generation in an
+// interval", 2019); larger tables take a remainder. Rounded down to a whole
+// sector of N slots (cap is a multiple of N): a probe reads sector by sector.
+template <int N>
 __device__ __forceinline__ uint64_t slot_start(uint64_t H, uint64_t cap) {
-  if (cap <= 0xFFFFFFFFull) return __umulhi((uint32_t)(H >> 16), (uint32_t)cap);
-  return slot_hash(H) % cap;
+  const uint64_t i = cap <= 0xFFFFFFFFull ? __umulhi((uint32_t)(H >> 16), (uint32_t)cap) : slot_hash(H) % cap;
+  return i & ~(uint64_t)(N - 1);
 }
-
-// The slot after i in linear probing, wrapping at cap.
-__device__ __forceinline__ uint64_t next_slot(uint64_t i, uint64_t cap) { return i + 1 == cap ? 0 : i + 1; }
 
 // Reverse the order of the 32 two-bit groups of x.
 __device__ __forceinline__ uint64_t rev_pairs(uint64_t x) {
@@ -809,75 +804,157 @@ __device__ __forceinline__ void cas128(unsigned long long* addr, uint64_t cmp_lo
 
 constexpr uint64_t kNoSlot = ~0ull;
 
+// Slots of a 32-byte sector (four one-word slots, two 16-byte ones): a probe
+// starts at a k-mer's sector and reads a whole sector at a time, so that a
+// k-mer mostly costs one round trip. Slot by slot from any start, the longest
+// of a warp's 32 chains -- six to eight slots at a load of 0.4 -- cost one each,
+// and the rest of the warp its instructions. Tables hold whole sectors.
+template <int TS>
+struct SectorOf {
+  static constexpr int kSlots = TS == 0 ? 4 : (TS == 2 ? 1 : 2);
+  unsigned long long key[kSlots];   // the slot's word (TS 0), key (1), low key word (2) or reference (3)
+  unsigned long long more[kSlots];  // its mask (1, 3) or high key word (2)
+  unsigned int mask;                // TS 2: its mask
+
+  __device__ __forceinline__ void load(const void* table, uint64_t first) {  // first: a multiple of kSlots
+    const ulonglong2* p = reinterpret_cast<const ulonglong2*>(static_cast<const char*>(table) + first * (32 / kSlots));
+    const ulonglong2 a = __ldcg(p), b = __ldcg(p + 1);
+    if constexpr (TS == 0) {
+      key[0] = a.x; key[1] = a.y; key[2] = b.x; key[3] = b.y;
+    } else if constexpr (TS == 2) {
+      key[0] = a.x; more[0] = a.y;
+      mask = (unsigned int)b.x;
+    } else {
+      key[0] = a.x; more[0] = a.y;
+      key[1] = b.x; more[1] = b.y;
+    }
+  }
+};
+
+// Insert into the one-word slots T[0 .. cap), probing from the sector at i (a
+// multiple of 4 below cap): the key's slot, or kNoSlot if every slot was tried
+// (the table is full). Bits already present are not written again. A word is
+// key << 9 | mask bits; never all ones for a key < 2^54.
+__device__ __forceinline__ uint64_t word_insert(unsigned long long* T, uint64_t cap, uint64_t i, uint64_t key,
+                                                uint32_t bits) {
+  for (uint64_t seen = 0; seen < cap; seen += 4) {
+    SectorOf<0> q;
+    q.load(T, i);
+    for (;;) {  // again only after another k-mer took the empty slot
+      unsigned long long cur = 0;
+      int at = 4;  // the first slot that is empty or the key's
+#pragma unroll
+      for (int k = 3; k >= 0; --k)
+        if (q.key[k] == kEmpty || (q.key[k] >> kMaskBits) == key) {
+          cur = q.key[k];
+          at = k;
+        }
+      if (at == 4) break;
+      unsigned long long* s = T + i + at;
+      if (cur == kEmpty) {
+        cur = atomicCAS(s, kEmpty, (key << kMaskBits) | bits);
+        if (cur == kEmpty) return i + at;
+      }
+      if ((cur >> kMaskBits) == key) {
+        if ((cur & bits) != bits) atomicOr(s, (unsigned long long)bits);
+        return i + at;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (k == at) q.key[k] = cur;
+    }
+    i = i + 4 == cap ? 0 : i + 4;
+  }
+  return kNoSlot;
+}
+
+// Mask of key in the one-word slots T[0 .. cap), or -1 if absent.
+__device__ __forceinline__ int word_find(const unsigned long long* T, uint64_t cap, uint64_t i, uint64_t key) {
+  for (uint64_t seen = 0; seen < cap; seen += 4) {
+    SectorOf<0> q;
+    q.load(T, i);
+    unsigned long long cur = 0;
+    bool hit = false;
+#pragma unroll
+    for (int k = 3; k >= 0; --k)
+      if (q.key[k] == kEmpty || (q.key[k] >> kMaskBits) == key) {
+        cur = q.key[k];
+        hit = true;
+      }
+    if (hit) return cur == kEmpty ? -1 : (int)(cur & ((1u << kMaskBits) - 1u));
+    i = i + 4 == cap ? 0 : i + 4;
+  }
+  return -1;
+}
+
 // Insert (key, bits) into a table of cap TS-kind slots (table_slot_kind),
-// probing from slot start (< cap); the key's slot, or kNoSlot if every slot
-// was tried (the table is full). Bits already present are not written again.
+// probing from the sector at start (below cap); the key's slot, or kNoSlot if
+// every slot was tried (the table is full). Bits already present are not
+// written again.
 template <int TS>
 __device__ __forceinline__ uint64_t table_insert(const RunView& v, uint64_t cap, const Key& key,
                                              uint64_t start, uint32_t bits) {
-  uint64_t i = start;
-  for (uint64_t probe = 0; probe < cap; ++probe, i = next_slot(i, cap)) {
-    if (TS == 0) {
-      // one word: key << 9 | mask bits; never all ones for a key < 2^54. A
-      // plain load first: most candidates meet their k-mer already in the
-      // table, and a random load costs less than a random atomic
-      unsigned long long* s = static_cast<unsigned long long*>(v.table) + i;
-      unsigned long long cur = __ldcg(s);
-      if (cur == kEmpty) {
-        cur = atomicCAS(s, kEmpty, (key.lo << kMaskBits) | bits);
-        if (cur == kEmpty) return i;
+  if constexpr (TS == 0) {
+    return word_insert(static_cast<unsigned long long*>(v.table), cap, start, key.lo, bits);
+  } else {
+    constexpr uint64_t N = SectorOf<TS>::kSlots;
+    uint64_t base = start;
+    for (uint64_t seen = 0; seen < cap; seen += N) {
+      SectorOf<TS> q;
+      if constexpr (TS == 1) q.load(v.table, base);  // TS 2: the CAS itself is the first look
+#pragma unroll
+      for (uint64_t k = 0; k < N; ++k) {
+        if constexpr (TS == 1) {
+          Slot1* s = static_cast<Slot1*>(v.table) + base + k;
+          unsigned long long cur = q.key[k];
+          uint32_t have = (uint32_t)q.more[k];
+          if (cur == kEmpty) {
+            cur = atomicCAS(&s->key, kEmpty, (unsigned long long)key.lo);
+            if (cur == kEmpty) cur = key.lo;
+            have = 0;
+          }
+          if (cur != key.lo) continue;
+          if ((have & bits) != bits) atomicOr(&s->mask, bits);
+        } else {
+          Slot2* s = static_cast<Slot2*>(v.table) + base;
+          uint64_t ol, oh;
+          cas128(&s->w0, kEmpty, kEmpty, key.lo, key.hi, &ol, &oh);
+          if (!((ol == kEmpty && oh == kEmpty) || (ol == key.lo && oh == key.hi))) continue;
+          if ((__ldcg(&s->mask) & bits) != bits) atomicOr(&s->mask, bits);
+        }
+        return base + k;
       }
-      if ((cur >> kMaskBits) != key.lo) continue;
-      if ((cur & bits) != bits) atomicOr(s, (unsigned long long)bits);
-      return i;
-    } else if (TS == 1) {
-      Slot1* s = static_cast<Slot1*>(v.table) + i;
-      const ulonglong2 w = __ldcg(reinterpret_cast<const ulonglong2*>(s));
-      unsigned long long cur = w.x;
-      uint32_t have = (uint32_t)w.y;
-      if (cur == kEmpty) {
-        cur = atomicCAS(&s->key, kEmpty, (unsigned long long)key.lo);
-        if (cur == kEmpty) cur = key.lo;
-        have = 0;
-      }
-      if (cur != key.lo) continue;
-      if ((have & bits) != bits) atomicOr(&s->mask, bits);
-      return i;
-    } else {
-      Slot2* s = static_cast<Slot2*>(v.table) + i;
-      uint64_t ol, oh;
-      cas128(&s->w0, kEmpty, kEmpty, key.lo, key.hi, &ol, &oh);
-      const bool mine = (ol == kEmpty && oh == kEmpty) || (ol == key.lo && oh == key.hi);
-      if (!mine) continue;
-      if ((__ldcg(&s->mask) & bits) != bits) atomicOr(&s->mask, bits);
-      return i;
+      base = base + N == cap ? 0 : base + N;
     }
+    return kNoSlot;
   }
-  return kNoSlot;
 }
 
 // Mask of key, or -1 if absent.
 template <int TS>
 __device__ __forceinline__ int table_find(const RunView& v, uint64_t cap, const Key& key, uint64_t start) {
-  uint64_t i = start;
-  for (uint64_t probe = 0; probe < cap; ++probe, i = next_slot(i, cap)) {
-    if (TS == 0) {
-      const unsigned long long cur = __ldcg(static_cast<const unsigned long long*>(v.table) + i);
-      if (cur == kEmpty) return -1;
-      if ((cur >> kMaskBits) == key.lo) return (int)(cur & ((1u << kMaskBits) - 1u));
-    } else if (TS == 1) {
-      const Slot1* s = static_cast<const Slot1*>(v.table) + i;
-      const ulonglong2 w = __ldcg(reinterpret_cast<const ulonglong2*>(s));
-      if (w.x == key.lo) return (int)(unsigned int)w.y;
-      if (w.x == kEmpty) return -1;
-    } else {
-      const Slot2* s = static_cast<const Slot2*>(v.table) + i;
-      const ulonglong2 w = __ldcg(reinterpret_cast<const ulonglong2*>(&s->w0));
-      if (w.x == key.lo && w.y == key.hi) return (int)__ldcg(&s->mask);
-      if (w.x == kEmpty && w.y == kEmpty) return -1;
+  if constexpr (TS == 0) {
+    return word_find(static_cast<const unsigned long long*>(v.table), cap, start, key.lo);
+  } else {
+    constexpr uint64_t N = SectorOf<TS>::kSlots;
+    uint64_t base = start;
+    for (uint64_t seen = 0; seen < cap; seen += N) {
+      SectorOf<TS> q;
+      q.load(v.table, base);
+#pragma unroll
+      for (uint64_t k = 0; k < N; ++k) {
+        if constexpr (TS == 1) {
+          if (q.key[k] == key.lo) return (int)(uint32_t)q.more[k];
+          if (q.key[k] == kEmpty) return -1;
+        } else {
+          if (q.key[0] == key.lo && q.more[0] == key.hi) return (int)q.mask;
+          if (q.key[0] == kEmpty && q.more[0] == kEmpty) return -1;
+        }
+      }
+      base = base + N == cap ? 0 : base + N;
     }
+    return -1;
   }
-  return -1;
 }
 
 // Slots of k-mers of 64 to 127 bases (kind 3): instead of the key, a
@@ -901,35 +978,45 @@ __device__ __forceinline__ bool ref_holds(const RunView& v, uint64_t ref, const 
 }
 
 __device__ __forceinline__ uint64_t table_insert_ref(const RunView& v, uint64_t cap, const Key4& key,
-                                                     uint64_t H, uint32_t bits, uint64_t g, bool rc) {
+                                                     uint64_t H, uint64_t start, uint32_t bits, uint64_t g,
+                                                     bool rc) {
   const uint64_t tag = H >> 49;
   const unsigned long long mine = (tag << 49) | ((uint64_t)rc << 48) | (g + 1);
-  uint64_t i = slot_start(H, cap);
-  for (uint64_t probe = 0; probe < cap; ++probe, i = next_slot(i, cap)) {
-    Slot3* s = static_cast<Slot3*>(v.table) + i;
-    unsigned long long cur = __ldcg(&s->ref);
-    if (cur == 0) {
-      cur = atomicCAS(&s->ref, 0ull, mine);
+  uint64_t base = start;
+  for (uint64_t seen = 0; seen < cap; seen += 2) {
+    SectorOf<3> q;
+    q.load(v.table, base);
+#pragma unroll
+    for (uint64_t k = 0; k < 2; ++k) {
+      Slot3* s = static_cast<Slot3*>(v.table) + base + k;
+      unsigned long long cur = q.key[k];
+      uint32_t have = (uint32_t)q.more[k];
       if (cur == 0) {
-        atomicOr(&s->mask, bits);
-        return i;
+        cur = atomicCAS(&s->ref, 0ull, mine);
+        have = 0;
+        if (cur == 0) cur = mine;  // claimed
       }
+      if (cur != mine && ((cur >> 49) != tag || !ref_holds(v, cur, key))) continue;
+      if ((have & bits) != bits) atomicOr(&s->mask, bits);
+      return base + k;
     }
-    if ((cur >> 49) != tag || !ref_holds(v, cur, key)) continue;
-    if ((__ldcg(&s->mask) & bits) != bits) atomicOr(&s->mask, bits);
-    return i;
+    base = base + 2 == cap ? 0 : base + 2;
   }
   return kNoSlot;
 }
 
 __device__ __forceinline__ int table_find_ref(const RunView& v, uint64_t cap, const Key4& key, uint64_t H) {
   const uint64_t tag = H >> 49;
-  uint64_t i = slot_start(H, cap);
-  for (uint64_t probe = 0; probe < cap; ++probe, i = next_slot(i, cap)) {
-    const Slot3* s = static_cast<const Slot3*>(v.table) + i;
-    const unsigned long long cur = __ldcg(&s->ref);
-    if (cur == 0) return -1;
-    if ((cur >> 49) == tag && ref_holds(v, cur, key)) return (int)__ldcg(&s->mask);
+  uint64_t base = slot_start<2>(H, cap);
+  for (uint64_t seen = 0; seen < cap; seen += 2) {
+    SectorOf<3> q;
+    q.load(v.table, base);
+#pragma unroll
+    for (uint64_t k = 0; k < 2; ++k) {
+      if (q.key[k] == 0) return -1;
+      if ((q.key[k] >> 49) == tag && ref_holds(v, q.key[k], key)) return (int)(uint32_t)q.more[k];
+    }
+    base = base + 2 == cap ? 0 : base + 2;
   }
   return -1;
 }
@@ -938,14 +1025,14 @@ __device__ __forceinline__ int table_find_ref(const RunView& v, uint64_t cap, co
 template <int KW, int TS>
 __device__ __forceinline__ uint64_t insert_occurrence(const RunView& v, uint64_t cap, const OccT<KW>& oc,
                                                       uint64_t g) {
-  if constexpr (TS == 3) return table_insert_ref(v, cap, oc.key, oc.H, oc.tbits, g, oc.rc);
-  else return table_insert<TS>(v, cap, oc.key, slot_start(oc.H, cap), oc.tbits);
+  if constexpr (TS == 3) return table_insert_ref(v, cap, oc.key, oc.H, slot_start<2>(oc.H, cap), oc.tbits, g, oc.rc);
+  else return table_insert<TS>(v, cap, oc.key, slot_start<SectorOf<TS>::kSlots>(oc.H, cap), oc.tbits);
 }
 
 template <int KW, int TS>
 __device__ __forceinline__ int find_occurrence(const RunView& v, uint64_t cap, const OccT<KW>& oc) {
   if constexpr (TS == 3) return table_find_ref(v, cap, oc.key, oc.H);
-  else return table_find<TS>(v, cap, oc.key, slot_start(oc.H, cap));
+  else return table_find<TS>(v, cap, oc.key, slot_start<SectorOf<TS>::kSlots>(oc.H, cap));
 }
 
 // Mask held by slot i (a slot that table_insert returned).
@@ -1010,23 +1097,62 @@ __device__ __forceinline__ void block_add(unsigned long long x, unsigned long lo
   __syncthreads();
 }
 
+// Linear counting (Whang, Vander-Zanden & Taylor 1990) of the distinct
+// candidates, on the 2^-lc_sample_log2 of the k-mers that a few bits of their
+// hash choose: sets the bit of a candidate whose k-mer hashes to h (table_setup
+// counts the bits). Every k-mer counted (no sample) cost one random atomic per
+// candidate; an atomic that returns whether the bit was new, to save the count,
+// made the probe wait (181 -> 193 us).
+__device__ __forceinline__ void lc_mark(const RunView& v, uint64_t h) {
+  if ((uint32_t)(h >> 24) & ((1u << v.lc_sample_log2) - 1u)) return;
+  const uint64_t x = h >> (64 - v.lc_log2);
+  atomicOr(v.lc_bits + (x >> 5), 1u << (x & 31));
+}
+
+constexpr uint64_t kLcMul = 0xff51afd7ed558ccdull;
+
+// OR the bits of a row of positions into a bitmap: lane by lane ascending
+// positions g (lanes without one: g = ~0, set = false), bit g set where `set`.
+// The lanes of one bitmap word are combined into one atomic.
+__device__ __forceinline__ void or_row(uint32_t* bitmap, uint64_t g, bool set) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t w = g >> 5;
+  const uint64_t prev = __shfl_up_sync(0xffffffffu, w, 1);
+  const bool head = lane == 0 || w != prev;
+  const uint32_t later = __ballot_sync(0xffffffffu, head) & (0xFFFFFFFEu << lane);  // heads after this lane
+  const int end = later ? __ffs(later) - 1 : 32;
+  uint32_t bits = set ? 1u << (g & 31) : 0u;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_down_sync(0xffffffffu, bits, o);
+    if (lane + o < end) bits |= y;
+  }
+  if (head && bits) atomicOr(bitmap + w, bits);
+}
+
 // ---------------------------------------------------------------------------
 // Kernels
 // ---------------------------------------------------------------------------
 
-// Four ASCII bytes -> four 2-bit codes (first byte in bits 7-6); *bad gets
-// 0xFF in every byte that is not one of ACGTacgt.
-__device__ __forceinline__ uint32_t pack4(uint32_t x, uint32_t* bad, uint32_t* is_n) {
+// Four ASCII bytes -> four 2-bit codes in the result's top byte (first byte in
+// bits 31-30); *diff gets nonzero bytes exactly where a byte is not one of
+// ACGTacgt. Bits 2-1 of a letter tell a, c, t, g = 0x61, 0x63, 0x74, 0x67 apart
+// (0, 1, 2, 3); a byte permute turns them into the letter they stand for, which
+// the byte must be, and one multiply gathers the four codes (no two of its
+// partial products share a bit). The pack is bound by its instructions: with four byte
+// compares and four shifts per word it ran at 54% issue and a third of the
+// memory bandwidth.
+__device__ __forceinline__ uint32_t pack4(uint32_t x, uint32_t* diff) {
   const uint32_t low = x | 0x20202020u;
-  const uint32_t ok = __vcmpeq4(low, 0x61616161u) | __vcmpeq4(low, 0x63636363u) |
-                      __vcmpeq4(low, 0x67676767u) | __vcmpeq4(low, 0x74747474u);
-  *bad = ~ok;
-  *is_n = __vcmpeq4(low, 0x6e6e6e6eu);
-  // a=0x61 c=0x63 g=0x67 t=0x74: bits 2-1 are 00 01 11 10; fold to 0 1 2 3
   const uint32_t t = (low >> 1) & 0x03030303u;
-  const uint32_t c = t ^ ((t >> 1) & 0x01010101u);
-  return ((c & 3u) << 6) | (((c >> 8) & 3u) << 4) | (((c >> 16) & 3u) << 2) | ((c >> 24) & 3u);
+  const uint32_t sel = __byte_perm(t | (t >> 4), 0u, 0x4420);  // the four t as nibbles
+  *diff = low ^ __byte_perm(0x67746361u, 0u, sel);             // g t c a
+  const uint32_t c = t ^ ((t >> 1) & 0x01010101u);             // a c t g = 0 1 2 3 -> 0 1 3 2
+  return c * 0x40100401u;
 }
+
+// 0xFF in every byte that is an N (either case).
+__device__ __forceinline__ uint32_t is_n_bytes(uint32_t x) { return __vcmpeq4(x | 0x20202020u, 0x6e6e6e6eu); }
 
 // Bit j of the result: the top bit of byte j of e (for a __vcmpeq4 mask:
 // byte j matched).
@@ -1045,26 +1171,32 @@ __device__ __forceinline__ uint32_t pack16(const RunView& v, uint64_t g, uint4 q
   const bool split = v.nmask != nullptr;
   if (full) {
     const uint32_t part[4] = {q.x, q.y, q.z, q.w};
+    uint32_t code[4], diff[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      uint32_t bad, is_n;
-      out |= pack4(part[c], &bad, &is_n) << (24 - 8 * c);
-      if (split) {
-        bad &= ~is_n;
-        nb |= byte_bits(is_n) << (4 * c);
+    for (int c = 0; c < 4; ++c) code[c] = pack4(part[c], &diff[c]);
+    out = __byte_perm(__byte_perm(code[3], code[2], 0x0073), __byte_perm(code[1], code[0], 0x0073), 0x5410);
+    if (diff[0] | diff[1] | diff[2] | diff[3]) {  // a byte that is no base: rare
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        uint32_t bad = diff[c];
+        if (split) {
+          const uint32_t is_n = is_n_bytes(part[c]);
+          bad &= ~is_n;
+          nb |= byte_bits(is_n) << (4 * c);
+        }
+        if (bad && *bad_at == ~0ull) *bad_at = g + 4 * c + (__ffs(bad) - 1) / 8;
       }
-      if (bad && *bad_at == ~0ull) *bad_at = g + 4 * c + (__ffs(bad) - 1) / 8;
     }
   } else if (g < v.m) {
     for (int i = 0; i < 16 && g + i < v.m; ++i) {
       const uint32_t c = v.bases[g + i];
-      uint32_t bad, is_n;
-      const uint32_t code = pack4(c | 0x61616100u, &bad, &is_n) >> 6;  // pad bytes are 'a'
-      if (split && (is_n & 0xFFu)) {
-        bad = 0;
+      uint32_t diff;
+      const uint32_t code = pack4(c | 0x61616100u, &diff) >> 30;  // pad bytes are 'a'
+      if (split && (is_n_bytes(c) & 0xFFu)) {
+        diff = 0;
         nb |= 1u << i;
       }
-      if ((bad & 0xFFu) && *bad_at == ~0ull) *bad_at = g + i;
+      if ((diff & 0xFFu) && *bad_at == ~0ull) *bad_at = g + i;
       out |= code << (30 - 2 * i);
     }
   }
@@ -1351,7 +1483,7 @@ __global__ void __launch_bounds__(kBlock, 3) pass1_probe_kernel(RunView v, int r
   constexpr int kR = kProbeR;
   const uint64_t stride = (uint64_t)gridDim.x * kBlock * kR;
   constexpr int kLanesPerWord = 32 / kR;
-  unsigned long long kept = 0, valid_n = 0;
+  uint32_t kept = 0, valid_n = 0;  // per thread: below 2^32
   const uint32_t warp_id = (blockIdx.x * kBlock + threadIdx.x) >> 5;
   uint64_t* seg = v.cands + (uint64_t)warp_id * v.seg_cap;  // wide records
   uint32_t* seg32 = reinterpret_cast<uint32_t*>(v.cands) + (uint64_t)warp_id * v.seg_cap;
@@ -1382,10 +1514,7 @@ __global__ void __launch_bounds__(kBlock, 3) pass1_probe_kernel(RunView v, int r
         const uint32_t pres = present_items<HB>(G[i], word[i], v.hashes);
         if ((pres >> 16) || __popc(pres & 0xFFFFu) >= 2) keep_bits |= 1u << i;
       }
-      if (((keep_bits >> i) & 1u) && !v.partial) {
-        const uint64_t idx = (G[i] * 0xff51afd7ed558ccdull) >> (64 - v.lc_log2);
-        atomicOr(v.lc_bits + (idx >> 5), 1u << (idx & 31));
-      }
+      if (((keep_bits >> i) & 1u) && !v.partial) lc_mark(v, G[i] * kLcMul);
     }
     // C_temp: kLanesPerWord lanes make up one 32-bit word
     uint32_t wv = keep_bits << (kR * (lane % kLanesPerWord));
@@ -1431,9 +1560,9 @@ __global__ void __launch_bounds__(kBlock, 3) pass1_probe_kernel(RunView v, int r
     v.seg_count[warp_id] = (uint32_t)(seg_used < v.seg_cap ? seg_used : v.seg_cap);
     if (seg_used > v.seg_cap) v.hdr->cand_overflow = 1;
   }
-  block_add(kept, &v.hdr->pass1_kept);
-  block_add(kept, v.partial ? &v.hdr->pass2_kept : &v.hdr->round_kept);
-  if (round == v.count_round) block_add(valid_n, &v.hdr->positions);
+  block_add((unsigned long long)kept, &v.hdr->pass1_kept);
+  block_add((unsigned long long)kept, v.partial ? &v.hdr->pass2_kept : &v.hdr->round_kept);
+  if (round == v.count_round) block_add((unsigned long long)valid_n, &v.hdr->positions);
 }
 
 // The probe loop from descriptors (same decisions and outputs as
@@ -1450,7 +1579,7 @@ __global__ void __launch_bounds__(kBlock) pass1_probe_desc_kernel(RunView v, int
   const int lane = threadIdx.x & 31;
   const uint32_t below = (1u << lane) - 1u;
   const uint64_t stride = (uint64_t)gridDim.x * kBlock * kRows;
-  unsigned long long kept = 0, valid_n = 0;
+  uint32_t kept = 0, valid_n = 0;  // per thread: below 2^32
   const uint32_t warp_id = (blockIdx.x * kBlock + threadIdx.x) >> 5;
   uint64_t* seg = v.cands + (uint64_t)warp_id * v.seg_cap;
   uint32_t* seg32 = reinterpret_cast<uint32_t*>(v.cands) + (uint64_t)warp_id * v.seg_cap;
@@ -1505,8 +1634,7 @@ __global__ void __launch_bounds__(kBlock) pass1_probe_desc_kernel(RunView v, int
         continue;
       }
       if (keep) {
-        const uint64_t idx = ((d[q] & ~(kDescActive | kDescSentinel)) * 0xff51afd7ed558ccdull) >> (64 - v.lc_log2);
-        atomicOr(v.lc_bits + (idx >> 5), 1u << (idx & 31));
+        lc_mark(v, (d[q] & ~(kDescActive | kDescSentinel)) * kLcMul);
         const uint64_t at = seg_used + __popc(row & below);
         if (at < v.seg_cap) {
           const uint64_t p = wbase + 32 * q + lane;
@@ -1530,9 +1658,9 @@ __global__ void __launch_bounds__(kBlock) pass1_probe_desc_kernel(RunView v, int
     v.seg_count[warp_id] = (uint32_t)(seg_used < v.seg_cap ? seg_used : v.seg_cap);
     if (seg_used > v.seg_cap) v.hdr->cand_overflow = 1;
   }
-  block_add(kept, &v.hdr->pass1_kept);
-  block_add(kept, v.partial ? &v.hdr->pass2_kept : &v.hdr->round_kept);
-  if (round == v.count_round) block_add(valid_n, &v.hdr->positions);
+  block_add((unsigned long long)kept, &v.hdr->pass1_kept);
+  block_add((unsigned long long)kept, v.partial ? &v.hdr->pass2_kept : &v.hdr->round_kept);
+  if (round == v.count_round) block_add((unsigned long long)valid_n, &v.hdr->positions);
 }
 
 // ---------------------------------------------------------------------------
@@ -1718,7 +1846,7 @@ __global__ void __launch_bounds__(kBlock) pass1_probe_cm_kernel(RunView v, int r
   uint16_t* idx = idx_s[wid];
   uint32_t* keep_w = keep_s[wid];
   const uint32_t below = (1u << lane) - 1u;
-  unsigned long long kept = 0, valid_n = 0;
+  uint32_t kept = 0, valid_n = 0;  // per thread: below 2^32
   const uint32_t warp_id = (blockIdx.x * kBlock + threadIdx.x) >> 5;
   uint64_t* seg = v.cands + (uint64_t)warp_id * v.seg_cap;
   uint32_t* seg32 = reinterpret_cast<uint32_t*>(v.cands) + (uint64_t)warp_id * v.seg_cap;
@@ -1761,8 +1889,7 @@ __global__ void __launch_bounds__(kBlock) pass1_probe_cm_kernel(RunView v, int r
       }
       const uint32_t row = __ballot_sync(0xffffffffu, keep);
       if (keep) {
-        const uint64_t x = (G * 0xff51afd7ed558ccdull) >> (64 - v.lc_log2);
-        atomicOr(v.lc_bits + (x >> 5), 1u << (x & 31));
+        lc_mark(v, G * kLcMul);
         const uint64_t at = seg_used + __popc(row & below);
         if (at < v.seg_cap) {
           if (v.narrow) seg32[at] = (uint32_t)g | (sentinel << 31);
@@ -1788,9 +1915,9 @@ __global__ void __launch_bounds__(kBlock) pass1_probe_cm_kernel(RunView v, int r
     v.seg_count[warp_id] = (uint32_t)(seg_used < v.seg_cap ? seg_used : v.seg_cap);
     if (seg_used > v.seg_cap) v.hdr->cand_overflow = 1;
   }
-  block_add(kept, &v.hdr->pass1_kept);
-  block_add(kept, v.partial ? &v.hdr->pass2_kept : &v.hdr->round_kept);
-  if (round == v.count_round) block_add(valid_n, &v.hdr->positions);
+  block_add((unsigned long long)kept, &v.hdr->pass1_kept);
+  block_add((unsigned long long)kept, v.partial ? &v.hdr->pass2_kept : &v.hdr->round_kept);
+  if (round == v.count_round) block_add((unsigned long long)valid_n, &v.hdr->positions);
 }
 
 // ---------------------------------------------------------------------------
@@ -2329,11 +2456,7 @@ __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
         }
         if (keep && !v.partial) {  // linear counting over a 2^-lc_sample_log2 sample of the k-mers
           const uint64_t id = (word_index << 30) | ((r >> 22) & 0x3FFFFFFFull);
-          const uint64_t h = id * 0xff51afd7ed558ccdull;
-          if (((uint32_t)(h >> 24) & ((1u << v.lc_sample_log2) - 1u)) == 0) {
-            const uint64_t x = h >> (64 - v.lc_log2);
-            atomicOr(v.lc_bits + (x >> 5), 1u << (x & 31));
-          }
+          lc_mark(v, id * kLcMul);
         }
       }
       const uint32_t row = __ballot_sync(0xffffffffu, keep);
@@ -2522,48 +2645,49 @@ constexpr double kTableLoadWord = 2.5, kTableLoad = 2.0;
 constexpr unsigned long long kPartRecords = 128, kMaxParts = 4096;
 
 // Size the pass-2 table of this round: 2.5 or 2 times the number of distinct
-// candidate k-mers, estimated by linear counting (Whang, Vander-Zanden &
-// Taylor 1990) from the bits the probe set (at least 1024 slots, a multiple
-// of 32, not rounded to a power of two), capped by the workspace. A saturated bitmap falls back to
-// twice the number of candidate positions. The estimate only sets the table's
-// size; an undersized table is detected and reported, never silently wrong.
-// Every block counts its share of the bitmap; the last block to finish sizes
-// the table.
-__global__ void __launch_bounds__(kBlock) table_setup_kernel(RunView v) {
-  if (v.o_fused && ordered_round(v)) {  // the round's table was the fused one: nothing left to size or clear
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+// candidate k-mers, as the probe's linear counting estimates it (at least 1024
+// slots, a multiple of 32, not rounded to a power of two), capped by the
+// workspace. A saturated bitmap falls back to the number of candidate
+// positions. The estimate only sets the table's size; an undersized table is
+// detected and reported, never silently wrong. One block: the sampled bitmap is
+// at most 1 MiB, and a grid that counts it and hands the sum to its last block
+// took 10-13 us of every round.
+__global__ void __launch_bounds__(1024) table_setup_kernel(RunView v) {
+  __shared__ unsigned int part[32];
+  DevHeader* h = v.hdr;
+  if (v.o_fused && ordered_round(v)) {  // the round's table was the fused one: nothing to size or clear
+    if (threadIdx.x == 0) {
       const unsigned long long used = (unsigned long long)v.o_tcap * v.o_regions;
-      v.hdr->table_slots = 0;
-      if (used > v.hdr->table_max) v.hdr->table_max = used;
-      v.hdr->cand_overflow = 0;
-      v.hdr->round_kept = 0;
-      v.hdr->lc_set = 0;
-      v.hdr->lc_blocks_done = 0;
+      h->cand_overflow = 0;
+      h->round_kept = 0;
+      h->table_slots = 0;
+      if (used > h->table_max) h->table_max = used;
     }
     return;
   }
-  const uint64_t words = (1ull << v.lc_log2) / 32;
-  const uint64_t stride = (uint64_t)gridDim.x * kBlock;
-  unsigned long long c = 0;
-  for (uint64_t i = (uint64_t)blockIdx.x * kBlock + threadIdx.x; i < words; i += stride)
-    c += __popc(__ldcg(v.lc_bits + i));
-  block_add(c, &v.hdr->lc_set);
-  __shared__ bool last;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    last = atomicAdd(&v.hdr->lc_blocks_done, 1u) == gridDim.x - 1;
+  unsigned int c = 0;
+  const uint32_t quads = 1u << (v.lc_log2 - 7);  // of four words; lc_log2 >= 16
+#pragma unroll 8
+  for (uint32_t i = threadIdx.x; i < quads; i += 1024) {
+    const uint4 q = __ldcg(reinterpret_cast<const uint4*>(v.lc_bits) + i);
+    c += __popc(q.x) + __popc(q.y) + __popc(q.z) + __popc(q.w);
   }
+  c = warp_sum(c);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
   __syncthreads();
-  if (!last || threadIdx.x != 0) return;
-  __threadfence();
-  const unsigned long long kept = *(volatile unsigned long long*)&v.hdr->round_kept;
-  const unsigned long long set = *(volatile unsigned long long*)&v.hdr->lc_set;
+  if (threadIdx.x != 0) return;
+  unsigned long long set = 0;
+  for (int w = 0; w < 32; ++w) set += part[w];
+  const unsigned long long kept = h->round_kept;
+  const unsigned int overflowed = h->cand_overflow;
+  h->cand_overflow = 0;
+  h->round_kept = 0;
   const double M = (double)(1ull << v.lc_log2);
   unsigned long long distinct = kept;
   if ((double)set < M - M / 1024.0) {  // at least 1/1024 of the bits still clear: about 7 per bit
-    // a region-ordered round counted a 2^-s sample of the k-mers: scale it up,
-    // with eight standard deviations of the sample's size to spare
-    const int sl = (v.o_regions && *(volatile unsigned int*)&v.hdr->ord_ok) ? v.lc_sample_log2 : 0;
+    // a 2^-s sample of the k-mers was counted: scale it up, with eight standard
+    // deviations of the sample's size to spare
+    const int sl = v.lc_sample_log2;
     const double f = (double)(1u << sl);
     const double est = -M * log1p(-(double)set / M) * f;
     const unsigned long long e = (unsigned long long)(est * 1.1 + (sl ? 8.0 * sqrt(est * f) : 0.0)) + 64ull;
@@ -2574,16 +2698,12 @@ __global__ void __launch_bounds__(kBlock) table_setup_kernel(RunView v) {
   if (cap < 1024ull) cap = 1024ull;
   cap = (cap + 31) / 32 * 32;  // any capacity works (slot_start); whole 32-slot groups
   if (cap > v.table_max_slots) cap = v.table_max_slots;
-  v.hdr->table_slots = cap;
-  if (cap > v.hdr->table_max) v.hdr->table_max = cap;
-  v.hdr->round_listed = *(volatile unsigned int*)&v.hdr->cand_overflow ? 0u : 1u;
+  h->table_slots = cap;
+  if (cap > h->table_max) h->table_max = cap;
+  h->round_listed = overflowed ? 0u : 1u;
   // pass 2 cuts every list segment into parts of about kPartRecords records
-  unsigned long long parts = (kept / v.n_segments + kPartRecords) / kPartRecords;
-  v.hdr->list_parts = (unsigned int)(parts < kMaxParts ? parts : kMaxParts);
-  v.hdr->cand_overflow = 0;
-  v.hdr->round_kept = 0;
-  v.hdr->lc_set = 0;
-  v.hdr->lc_blocks_done = 0;
+  const unsigned long long parts = (kept / v.n_segments + kPartRecords) / kPartRecords;
+  h->list_parts = (unsigned int)(parts < kMaxParts ? parts : kMaxParts);
 }
 
 template <int TS>
@@ -2624,53 +2744,26 @@ __device__ __forceinline__ uint64_t list_at(const RunView& v, uint64_t i, bool* 
 // Pass-2 work over the candidate list. Every list segment is cut into
 // list_parts parts (interleaved 32-record rows), and the launched warps take
 // the (segment, part) pairs in turn, so that the work spreads evenly over a
-// grid that is resident all at once. fn(i) runs for list index i.
-template <typename F>
-__device__ __forceinline__ void for_listed(const RunView& v, F&& fn) {
+// grid that is resident all at once. A warp takes U rows of its part at a time:
+// fn(first + row0, row, n - row0) gets the list index and the distance (in
+// records) of the rows -- row u holds the records u * row .. u * row + 31 from
+// there, as far as they lie below the third argument.
+template <int U, typename F>
+__device__ __forceinline__ void for_rows(const RunView& v, F&& fn) {
   // 32-bit arithmetic: at most kMaxSegments segments of at most kMaxParts parts
   const uint32_t parts = *(volatile unsigned int*)&v.hdr->list_parts;
   const uint32_t pairs = v.n_segments * parts;
   const uint32_t warps = gridDim.x * (kBlock / 32);
-  const uint32_t lane = threadIdx.x & 31;
-  for (uint32_t w = (blockIdx.x * kBlock + threadIdx.x) >> 5; w < pairs; w += warps) {
-    const uint32_t sgm = w / parts, part = w - sgm * parts;
-    const uint32_t n = __ldcg(v.seg_count + sgm);
-    const uint64_t first = (uint64_t)sgm * v.seg_cap;
-    for (uint32_t j = part * 32 + lane; j < n; j += 32 * parts) fn(first + j);
-  }
-}
-
-// for_listed that reads each record one ahead: fn(i, g, sentinel, slot)
-// gets list index i with its position (and with SLOT its kept table slot)
-// already loaded, while the lane's next record is in flight.
-template <bool SLOT, typename F>
-__device__ __forceinline__ void for_listed_ahead(const RunView& v, bool last_use, F&& fn) {
-  const uint32_t parts = *(volatile unsigned int*)&v.hdr->list_parts;
-  const uint32_t pairs = v.n_segments * parts;
-  const uint32_t warps = gridDim.x * (kBlock / 32);
-  const uint32_t lane = threadIdx.x & 31;
   const uint32_t row = 32 * parts;
   for (uint32_t w = (blockIdx.x * kBlock + threadIdx.x) >> 5; w < pairs; w += warps) {
     const uint32_t sgm = w / parts, part = w - sgm * parts;
     const uint32_t n = __ldcg(v.seg_count + sgm);
     const uint64_t first = (uint64_t)sgm * v.seg_cap;
-    uint32_t j = part * 32 + lane;
-    bool sent = false;
-    uint64_t g = j < n ? list_at(v, first + j, &sent, last_use) : 0;
-    uint32_t slot = (SLOT && j < n) ? __ldcs(v.cand_slot + first + j) : 0u;
-    while (j < n) {
-      const uint32_t jn = j + row;
-      bool sent_n = false;
-      const uint64_t gn = jn < n ? list_at(v, first + jn, &sent_n, last_use) : 0;
-      const uint32_t slot_n = (SLOT && jn < n) ? __ldcs(v.cand_slot + first + jn) : 0u;
-      fn(first + j, g, sent, slot);
-      j = jn;
-      g = gn;
-      sent = sent_n;
-      slot = slot_n;
-    }
+    for (uint64_t r0 = part * 32; r0 < n; r0 += (uint64_t)U * row) fn(first + r0, row, (uint32_t)(n - r0));
   }
 }
+
+constexpr int kClassifyAhead = 2;  // rows of the list in flight per warp
 
 // Algorithm 1, insert loop, second pass: every candidate ORs its in/out bases
 // (or the sentinel bit) into the exact table entry of its k-mer. Reads the
@@ -2681,22 +2774,17 @@ __global__ void __launch_bounds__(kBlock) pass2_insert_kernel(RunView v) {
   if (v.o_fused && ordered_round(v)) return;  // the fused records took this round's pass 2
   const uint64_t cap = *(volatile unsigned long long*)&v.hdr->table_slots;
   if (*(volatile unsigned int*)&v.hdr->round_listed) {
-    auto insert_one = [&](uint64_t i, uint64_t g, bool sent, uint32_t) {
+    const uint32_t lane = threadIdx.x & 31;
+    for_rows<1>(v, [&](uint64_t i0, uint32_t, uint32_t left) {
+      if (lane >= left) return;
+      bool sent;
+      const uint64_t g = list_at(v, i0 + lane, &sent, false);
       OccT<KW> oc;
       read_listed<KW>(v, g, sent, &oc);
       const uint64_t slot = insert_occurrence<KW, TS>(v, cap, oc, g);
       if (slot == kNoSlot) v.hdr->overflow = 1;
-      if (v.cand_slot) v.cand_slot[i] = slot == kNoSlot ? 0xFFFFFFFFu : (uint32_t)slot;
-    };
-    if (kInsertPrefetch) {
-      for_listed_ahead<false>(v, false, insert_one);
-    } else {
-      for_listed(v, [&](uint64_t i) {
-        bool sent;
-        const uint64_t g = list_at(v, i, &sent, false);
-        insert_one(i, g, sent, 0u);
-      });
-    }
+      if (v.cand_slot) v.cand_slot[i0 + lane] = slot == kNoSlot ? 0xFFFFFFFFu : (uint32_t)slot;
+    });
     return;
   }
   const uint64_t stride = (uint64_t)gridDim.x * kBlock;
@@ -2710,49 +2798,62 @@ __global__ void __launch_bounds__(kBlock) pass2_insert_kernel(RunView v) {
 
 // Algorithm 1, probe loop, second pass: a candidate is a junction iff its
 // k-mer is a sentinel or has more than one distinct in- or out-base. Sets
-// the junction's bit of C_final (cleared before the first round). A listed
-// candidate reads its mask from the slot the insert loop kept (or looks its
-// k-mer up when no slots were kept).
+// the junction's bit of C_final (cleared before the first round; a row's bits
+// in one atomic per bitmap word). A listed candidate reads its mask from the
+// slot the insert loop kept (or looks its k-mer up when no slots were kept).
 template <int KW, int TS>
 __global__ void __launch_bounds__(kBlock) pass2_classify_kernel(RunView v) {
   if (v.o_fused && ordered_round(v)) return;  // the fused records took this round's pass 2
   const uint64_t cap = *(volatile unsigned long long*)&v.hdr->table_slots;
   unsigned long long found = 0;
-  auto mark = [&](uint64_t g, int mk) {
-    if (mk < 0) v.hdr->overflow = 1;
-    if (mk < 0 || is_junction_mask(mk)) {
-      atomicOr(v.cfinal + (g >> 5), 1u << (g & 31));
-      ++found;
-    }
-  };
   if (*(volatile unsigned int*)&v.hdr->round_listed) {
-    auto classify_one = [&](uint64_t i, uint64_t g, bool sent, uint32_t slot) {
-      if (v.cand_slot) {
-        mark(g, slot == 0xFFFFFFFFu ? -1 : table_mask<TS>(v, slot));
-      } else {
-        OccT<KW> oc;
-        read_listed<KW>(v, g, sent, &oc);
-        mark(g, find_occurrence<KW, TS>(v, cap, oc));
+    constexpr int U = kClassifyAhead;
+    const uint32_t lane = threadIdx.x & 31;
+    for_rows<U>(v, [&](uint64_t i0, uint32_t row, uint32_t left) {
+      uint64_t g[U];
+      uint32_t slot[U];
+      bool sent[U];
+      int mk[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const bool ok = u * row + lane < left;
+        const uint64_t i = i0 + (uint64_t)u * row + lane;
+        g[u] = ok ? list_at(v, i, &sent[u], true) : ~0ull;
+        slot[u] = (ok && v.cand_slot) ? __ldcs(v.cand_slot + i) : 0xFFFFFFFFu;
       }
-    };
-    if (kClassifyPrefetch && v.cand_slot) {
-      for_listed_ahead<true>(v, true, classify_one);
-    } else if (kClassifyPrefetch) {
-      for_listed_ahead<false>(v, true, classify_one);
-    } else {
-      for_listed(v, [&](uint64_t i) {
-        bool sent;
-        const uint64_t g = list_at(v, i, &sent, true);
-        classify_one(i, g, sent, v.cand_slot ? __ldcs(v.cand_slot + i) : 0u);
-      });
-    }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        mk[u] = -1;
+        if (v.cand_slot) {
+          if (slot[u] != 0xFFFFFFFFu) mk[u] = table_mask<TS>(v, slot[u]);
+        } else if (g[u] != ~0ull) {
+          OccT<KW> oc;
+          read_listed<KW>(v, g[u], sent[u], &oc);
+          mk[u] = find_occurrence<KW, TS>(v, cap, oc);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (u * row >= left) break;  // the same for every lane
+        const bool ok = g[u] != ~0ull;
+        if (ok && mk[u] < 0) v.hdr->overflow = 1;
+        const bool junction = ok && (mk[u] < 0 || is_junction_mask(mk[u]));
+        found += junction;
+        or_row(v.cfinal, g[u], junction);
+      }
+    });
   } else {
     const uint64_t stride = (uint64_t)gridDim.x * kBlock;
     for (uint64_t g = v.p_begin + (uint64_t)blockIdx.x * kBlock + threadIdx.x; g < v.p_end; g += stride) {
       if (!((__ldg(v.ctemp + (g >> 5)) >> (g & 31)) & 1u)) continue;
       OccT<KW> oc;
       if (!read_occurrence<KW>(v, g, &oc)) continue;
-      mark(g, find_occurrence<KW, TS>(v, cap, oc));
+      const int mk = find_occurrence<KW, TS>(v, cap, oc);
+      if (mk < 0) v.hdr->overflow = 1;
+      if (mk < 0 || is_junction_mask(mk)) {
+        atomicOr(v.cfinal + (g >> 5), 1u << (g & 31));
+        ++found;
+      }
     }
   }
   block_add(found, &v.hdr->pass2_kept);
@@ -2895,41 +2996,64 @@ __global__ void __launch_bounds__(kBlock) emit_kernel(RunView v) {
     c = warp_sum(c);
     if (lane == 0) warp_s[wid] = c;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t tot = 0;
+    if (wid == 0) {
+      uint32_t tot = 0, mine = 0;
+#pragma unroll
       for (int w = 0; w < kBlock / 32; ++w) {
         const uint32_t x = warp_s[w];
-        warp_s[w] = tot;
+        if (lane == w) mine = tot;
         tot += x;
       }
-      total_s = tot;
+      __syncwarp();
+      if (lane < kBlock / 32) warp_s[lane] = mine;
+      // the look-back, 32 tiles at a time: a lane per tile, down to the nearest
+      // one that has published its prefix (one tile at a time, the last tiles of
+      // a short run walked hundreds of round trips: 30 us for 35 M positions, 25
+      // so; 128 tiles at a time waited for more of them and took 33)
       unsigned long long prefix = 0;
-      if (tile == 0) {
-        status[0] = kFlagPrefix | tot;
-      } else {
-        status[tile] = kFlagAgg | tot;
-        uint64_t j = tile - 1;
-        uint32_t spins = 0;
-        for (;;) {
-          const unsigned long long st = status[j];
-          if (st & kFlagPrefix) {
-            prefix += st & kValMask;
-            break;
-          }
-          if (st & kFlagAgg) {
-            prefix += st & kValMask;
-            --j;  // tile 0 only ever holds a prefix, so j stays >= 0
-            continue;
-          }
+      if (lane == 0) {
+        if (tile == 0) status[0] = kFlagPrefix | tot;
+        else status[tile] = kFlagAgg | tot;
+      }
+      uint32_t spins = 0;
+      for (int64_t j = (int64_t)tile - 1; j >= 0;) {
+        const int64_t i = j - lane;
+        unsigned long long st = kFlagPrefix;  // before tile 0: an empty prefix
+        if (i >= 0) st = status[i];
+        const uint32_t done_m = __ballot_sync(0xffffffffu, (st & kFlagPrefix) != 0);
+        const uint32_t none_m = __ballot_sync(0xffffffffu, st == 0);
+        const int p = done_m ? __ffs(done_m) - 1 : 31;  // the nearest prefix ends the walk
+        if (none_m & ((2u << p) - 1u)) {  // a tile up to there has not published yet
           if (++spins > kSpinLimit) {
-            v.hdr->timeout = 1;
+            if (lane == 0) v.hdr->timeout = 1;
             break;
           }
           __nanosleep(32);
+          continue;
         }
-        status[tile] = kFlagPrefix | (prefix + tot);
+        unsigned long long x = lane <= p ? st & kValMask : 0ull;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        prefix += x;
+        if (done_m) break;
+        j -= 32;
       }
-      prefix_s = prefix;
+      if (lane == 0) {
+        if (tile) status[tile] = kFlagPrefix | (prefix + tot);
+        total_s = tot;
+        prefix_s = prefix;
+      }
+    } else if (wid == 1 && lane < 2) {
+      // meanwhile, the strings that start in this tile (the last tile also takes t = n_seqs)
+      const uint64_t g = lane == 0 ? tile_base * 32
+                                   : (tile + 1 == v.n_tiles ? ~0ull : (tile_base + kEmitTileWords) * 32);
+      uint64_t lo = 0, hi = (uint64_t)v.n_seqs + 1;  // first t in [0, n_seqs + 1) with offsets[t] >= g
+      while (lo < hi) {
+        const uint64_t mid = (lo + hi) >> 1;
+        if (__ldg(v.offsets + mid) < g) lo = mid + 1; else hi = mid;
+      }
+      if (lane == 0) t_lo_s = lo;
+      else t_hi_s = lo;
     }
     __syncthreads();
     // batch by batch: every lane expands its word into the warp's stage at its
@@ -2968,20 +3092,6 @@ __global__ void __launch_bounds__(kBlock) emit_kernel(RunView v) {
     }
     // out_offsets[t] (junctions before string t) for the strings that start in
     // this tile; the last tile also takes t = n_seqs (start m: the total)
-    if (threadIdx.x == 0) {
-      const uint64_t g_lo = tile_base * 32;
-      const uint64_t g_hi = tile + 1 == v.n_tiles ? ~0ull : (tile_base + kEmitTileWords) * 32;
-      auto lower = [&](uint64_t g) {  // first t in [0, n_seqs + 1) with offsets[t] >= g
-        uint64_t lo = 0, hi = (uint64_t)v.n_seqs + 1;
-        while (lo < hi) {
-          const uint64_t mid = (lo + hi) >> 1;
-          if (__ldg(v.offsets + mid) < g) lo = mid + 1; else hi = mid;
-        }
-        return lo;
-      };
-      t_lo_s = lower(g_lo);
-      t_hi_s = lower(g_hi);
-    }
     __syncthreads();
     for (uint64_t t = t_lo_s + threadIdx.x; t < t_hi_s; t += kBlock) {
       const uint64_t g = __ldg(v.offsets + t), w = g >> 5, j = w - tile_base;
@@ -3431,7 +3541,7 @@ static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges*
   if (v.partial) return done(launched);  // the partially compacted graph: no second pass
   {
     Timed t("table_setup", s);
-    table_setup_kernel<<<grid_for(table_setup_kernel, kBlock, (1ull << v.lc_log2) / 32), kBlock, 0, s>>>(pv);
+    table_setup_kernel<<<1, 1024, 0, s>>>(pv);
   }
   {
     Timed t("table_clear", s);
