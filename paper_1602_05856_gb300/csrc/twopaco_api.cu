@@ -81,8 +81,7 @@ struct Layout {
   uint32_t o_tcap;     // fused: table slots per region
   int o_lg_region_words;
   uint64_t o_rec_cap, o_tiles;
-  uint64_t rplane, othist, owcount, ocsum, ocpre, obtot, ostart, ofill, orecs, odec, ometa, otcount, otbase, otsum,
-      operm;
+  uint64_t olist, ofirst, othist, ocsum, ocpre, obtot, ostart, ofill, orecs, odec, ometa;
   uint64_t bucket_cap, bucket_chunk;
   uint64_t n_chunks, run_cap;
   uint64_t total;
@@ -141,17 +140,33 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
   L.cand_cap = o.candidate_records ? o.candidate_records
                                    : (per_round / 2 > (1u << 16) ? per_round / 2 : (1u << 16));
   if (o.partial) L.cand_cap = 0;
-  // region-ordered first pass: class-map rounds (k <= 63, h <= 6, one launch
-  // per loop) with at most kOrdMaxRegions regions of at most 2^22 words and
-  // at most kOrdMaxHist (round, region) counters; automatically for filters of
-  // 1 GiB and more (far beyond L2), or for any filter when asked
+  // region-bucketed first-pass inserts of a one-round run: a filter beyond L2 (over
+  // 64 MiB) with at least 16 ORs of a chunk on every 32-byte filter sector on
+  // average, or any filter when asked
+  const bool beyond_l2 = filter_bits / 8 > (64ull << 20);
+  const uint64_t per_chunk = std::min<uint64_t>(per_round, 1ull << 31) * 4 / 5;
+  const bool want_bkt =
+      o.bucket_inserts == 1 || (o.bucket_inserts == 0 && beyond_l2 && per_chunk >= 16 * (filter_bits / 256));
+  // region-ordered first pass: k <= 63, h <= 6, one launch per loop, at most
+  // kOrdMaxRegions regions of at most 2^22 words and at most kOrdMaxHist
+  // (round, region) counters; rounds automatically for filters of 1 GiB and more,
+  // and in one round wherever bucketed inserts are wanted
   L.o_regions = 0;
   {
     const uint64_t fwords = filter_bits / 64;
-    const uint64_t rw = std::max<uint64_t>(1, std::min<uint64_t>(1ull << kRegionWordsLog2, fwords / 64));
-    const uint64_t R = fwords / rw;
-    const bool want = o.ordered_first_pass == 1 || (o.ordered_first_pass == 0 && filter_bits / 8 >= (1ull << 30));
-    if (want && rounds > 1 && rounds <= kMaxMapRounds && k <= 63 && o.hashes <= 6 && !o.per_string_launches &&
+    // as many regions as a byte can number, so that a region, the next one (read
+    // ahead) and a part of the table are well inside L2, of at most 2^22 words (32
+    // MiB) each; fewer where the counters of many rounds, or table parts of at least
+    // 1024 slots (k <= 27), want it
+    const uint64_t r_min = std::max<uint64_t>(1, fwords >> kRegionWordsLog2);
+    uint64_t R = std::max<uint64_t>(r_min, std::min<uint64_t>(kOrdMaxRegions, fwords));
+    while (R > r_min && R * (uint64_t)rounds > kOrdMaxHist) R /= 2;
+    while (R > r_min && k <= 27 && !o.partial && L.table_slots / R < 1024) R /= 2;
+    const uint64_t rw = fwords / R;
+    const bool auto_rounds = filter_bits / 8 >= (1ull << 30);
+    const bool want = rounds > 1 ? o.ordered_first_pass == 1 || (o.ordered_first_pass == 0 && auto_rounds)
+                                 : want_bkt && o.ordered_first_pass != 2;
+    if (want && rounds <= kMaxMapRounds && k <= 63 && o.hashes <= 6 && !o.per_string_launches &&
         m > 0 && R <= kOrdMaxRegions && R * (uint64_t)rounds <= kOrdMaxHist) {
       L.o_regions = (uint32_t)R;
       L.o_lg_region_words = log2_exact(rw);
@@ -195,27 +210,20 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
   // of bit bases, flags) when they fit -- under 2^31 bases, h <= 6, b <= 2^37
   // class map: one byte per position for 2 .. kMaxMapRounds rounds (then the
   // rounds need no descriptors: each visits only its class's positions)
-  L.use_cmap = (rounds > 1 && rounds <= kMaxMapRounds) ? 1 : 0;
+  // (the sorted tiles of the ordered first pass take its place)
+  L.use_cmap = (rounds > 1 && rounds <= kMaxMapRounds && !L.o_regions) ? 1 : 0;
   L.cmap = at;
   if (L.use_cmap) at += align_up(m + 64);
-  L.use_desc = (L.narrow && o.hashes <= 6 && filter_bits <= (1ull << 37) && !L.use_cmap) ? 1 : 0;
+  L.use_desc = (L.narrow && o.hashes <= 6 && filter_bits <= (1ull << 37) && !L.use_cmap && !L.o_regions) ? 1 : 0;
   L.desc = at;
   if (L.use_desc) at += align_up((m + 16) * 8);
-  // region buckets for the first-pass inserts: filters beyond L2 (over 64 MiB),
-  // or any filter when asked; regions of up to 2^22 words (32 MiB), at most
-  // kMaxRegions of them; records carry up to 6 bits per item
+  // region buckets for the first-pass inserts alone (where the ordered first pass
+  // does not go): regions of up to 2^22 words (32 MiB), at most kMaxRegions of
+  // them; records carry up to 6 bits per item
   const uint64_t fwords = filter_bits / 64;
-  const bool want_bkt = o.bucket_inserts == 1 || (o.bucket_inserts == 0 && filter_bits / 8 > (64ull << 20));
   uint64_t region_words = std::min<uint64_t>(1ull << kRegionWordsLog2, fwords / 4);
   L.n_regions = 0;
-  // automatically only where it measured faster: when a chunk's records put at
-  // least 16 ORs on every 32-byte filter sector on average (on a 24 Gbp input
-  // with a 2^36-bit filter, about 7 per sector, the cold misses of every region
-  // cost more than the direct ORs; on 310 Mbp with 2^30 bits, 77 per sector, the
-  // buckets win)
-  const uint64_t per_chunk = std::min<uint64_t>(per_round, 1ull << 31) * 4 / 5;
-  const bool dense = per_chunk >= 16 * (filter_bits / 256);
-  if (want_bkt && (o.bucket_inserts == 1 || dense) && o.hashes <= 6 && m > 0 && region_words >= 1 &&
+  if (want_bkt && !L.o_regions && o.hashes <= 6 && m > 0 && region_words >= 1 &&
       fwords / region_words <= kMaxRegions) {
     L.n_regions = (uint32_t)(fwords / region_words);
     L.n_sub = 1;
@@ -229,22 +237,20 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
     const uint64_t chunk = L.bucket_cap * buckets / 5 * 4 * (uint64_t)rounds;
     L.bucket_chunk = std::max<uint64_t>(kRangeTile, chunk / kRangeTile * kRangeTile);
   }
-  if (L.o_regions) L.n_regions = 0;  // the ordered first pass applies the inserts by region itself
   L.bfill = at;
   if (L.n_regions) at += align_up(((uint64_t)L.n_regions * L.n_sub + 1) * 128);
   L.brecs = at;
   if (L.n_regions) at += align_up(L.bucket_cap * L.n_regions * L.n_sub * 8);
-  L.rplane = L.othist = L.owcount = L.ocsum = L.ocpre = L.obtot = L.ostart = L.ofill = L.orecs = L.odec = L.ometa = at;
-  L.otcount = L.otbase = L.otsum = L.operm = at;
+  L.olist = L.ofirst = L.othist = L.ocsum = L.ocpre = L.obtot = L.ostart = L.ofill = L.orecs = L.odec = L.ometa = at;
   if (L.o_regions) {
     const uint64_t R = L.o_regions;
-    L.rplane = at;
-    at += align_up(m + 64);
+    L.olist = at;
+    at += align_up(L.o_tiles * kOrdTile * 2);
+    L.ofirst = at;
+    at += align_up(L.o_tiles * ((uint64_t)rounds + 1) * 2);
     const uint64_t chunks = (L.o_tiles + kOrdScanTiles - 1) / kOrdScanTiles;
     L.othist = at;
     at += align_up(L.o_tiles * rounds * R * 2);
-    L.owcount = at;
-    at += align_up((uint64_t)rounds * L.o_tiles * 8 * 2);
     L.ocsum = at;
     at += align_up(chunks * R * 4);
     L.ocpre = at;
@@ -262,14 +268,6 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
     at += align_up((L.o_rec_cap + 31) / 32 * 4 * (L.o_fused ? 2 : 1));
     L.ometa = at;
     at += align_up(L.o_tiles * R * 4);
-    L.otcount = at;
-    at += align_up((uint64_t)rounds * L.o_tiles * 4);
-    L.otbase = at;
-    at += align_up((uint64_t)rounds * L.o_tiles * 8);
-    L.otsum = at;
-    at += align_up((uint64_t)rounds * ((L.o_tiles + kOrdScanTiles - 1) / kOrdScanTiles) * 8);
-    L.operm = at;
-    at += align_up(L.o_rec_cap * 2);
   }
   // N splitting: N mask and boundary bitmap (one bit per base), per-chunk
   // boundary counts, the sorted boundaries and their ranks
@@ -373,9 +371,9 @@ RunView make_view(const uint8_t* d_bases, const uint64_t* d_offsets, uint64_t n_
   v.o_regions = L.o_regions;
   if (L.o_regions) {
     v.o_lg_region_words = L.o_lg_region_words;
-    v.rplane = reinterpret_cast<uint8_t*>(base + L.rplane);
+    v.o_list = reinterpret_cast<uint16_t*>(base + L.olist);
+    v.o_first = reinterpret_cast<uint16_t*>(base + L.ofirst);
     v.o_thist = reinterpret_cast<uint16_t*>(base + L.othist);
-    v.o_wcount = reinterpret_cast<uint16_t*>(base + L.owcount);
     v.o_csum = reinterpret_cast<uint32_t*>(base + L.ocsum);
     v.o_cpre = reinterpret_cast<unsigned long long*>(base + L.ocpre);
     v.o_btot = reinterpret_cast<unsigned long long*>(base + L.obtot);
@@ -386,10 +384,6 @@ RunView make_view(const uint8_t* d_bases, const uint64_t* d_offsets, uint64_t n_
     v.o_dec = reinterpret_cast<uint32_t*>(base + L.odec);
     v.o_meta = reinterpret_cast<uint32_t*>(base + L.ometa);
     v.o_tiles = L.o_tiles;
-    v.o_tcount = reinterpret_cast<uint32_t*>(base + L.otcount);
-    v.o_tbase = reinterpret_cast<unsigned long long*>(base + L.otbase);
-    v.o_tsum = reinterpret_cast<unsigned long long*>(base + L.otsum);
-    v.o_perm = reinterpret_cast<uint16_t*>(base + L.operm);
     v.o_fused = L.o_fused;
     v.o_tcap = L.o_tcap;
   }

@@ -116,17 +116,15 @@ struct RunView {
   uint64_t* bucket_recs;    // n_regions * n_sub buckets of bucket_cap records
   uint64_t bucket_cap;
   uint64_t bucket_chunk;    // positions per scatter-and-apply chunk (a multiple of kRangeTile)
-  // region-ordered first pass (o_regions > 0; class-map rounds): the class map
-  // also records every position's filter region (rplane) and counts the
-  // positions of every tile per (class, region) pair and per (class, warp
-  // chunk); a round then writes one 8-byte record per position of its class
-  // into the bucket of its region, applies the ORs and the probes bucket by
-  // bucket, and gathers the decisions back in position order
+  // region-ordered first pass (o_regions > 0): the positions of every tile sorted
+  // by class and filter region; a round then writes one 8-byte record per position
+  // of its class into the bucket of its region, applies the ORs and the probes
+  // bucket by bucket, and gathers the decisions back in position order
   uint32_t o_regions;       // filter regions (buckets), at most kOrdMaxRegions
   int o_lg_region_words;    // log2 of the 64-bit words per region (at most 22)
-  uint8_t* rplane;          // region of every position's k-mer, one byte per position
+  uint16_t* o_list;         // every tile's positions sorted by class and region (kOrdTile per tile)
+  uint16_t* o_first;        // per tile: the first list entry of every class, then the end (rounds + 1)
   uint16_t* o_thist;        // per tile, class and region: its positions (tile-major)
-  uint16_t* o_wcount;       // per class, tile and warp chunk of kOrdTile / 8 positions: its positions
   uint32_t* o_csum;         // per chunk of kOrdScanTiles tiles and bucket: the round's members
   unsigned long long* o_cpre;  // per chunk and bucket: the round's members in the chunks before
   unsigned long long* o_btot;  // per bucket: the round's members
@@ -138,10 +136,6 @@ struct RunView {
                             // junctions) per 32 slots
   uint32_t* o_meta;         // per tile and bucket: where the tile's records start in the bucket
   uint64_t o_tiles;         // tiles of kOrdTile positions: ceil(m / kOrdTile)
-  uint32_t* o_tcount;       // positions of every class in every tile (rounds x o_tiles)
-  unsigned long long* o_tbase;  // members of the round in the tiles before (rounds x o_tiles)
-  unsigned long long* o_tsum;   // members of the round per scan chunk of tiles
-  uint16_t* o_perm;         // per member of the round: its rank within its tile's room
   int o_fused;              // k <= 27, not partial: pass 2 runs on the records (fused records)
   uint32_t o_tcap;          // fused: table slots per bucket (region), the table is o_regions x o_tcap slots
   int use_desc;             // the insert leaves descriptors and the probe reads them
@@ -176,12 +170,11 @@ constexpr uint32_t kMinBuckets = 256;      // buckets of bucketed inserts, at le
 constexpr uint32_t kMaxBuckets = 1024;
 constexpr int kRegionWordsLog2 = 22;       // 32 MiB regions (words of 8 bytes)
 constexpr uint32_t kCmWindowPositions = 512;  // positions per class-map window (one warp's)
-constexpr int kOrdTileWindows = 32;        // region-ordered first pass: windows per tile
-constexpr uint64_t kOrdTile = (uint64_t)kOrdTileWindows * kCmWindowPositions;  // 16384 positions
+constexpr uint64_t kOrdTile = 16384;       // region-ordered first pass: positions per tile
 constexpr uint32_t kOrdMaxRegions = 256;   // buckets (filter regions), at most
 constexpr uint32_t kOrdMaxHist = 4096;     // rounds x regions, at most
 constexpr uint32_t kOrdFillStride = 32;    // bucket fill counters 128 bytes apart
-constexpr uint32_t kOrdScanTiles = 1024;   // tiles per block of the member-number scan
+constexpr uint32_t kOrdScanTiles = 128;    // tiles per block of the scans over tiles
 
 // Kernel launch helpers (twopaco_kernels.cu). Each returns the number of
 // kernels it launched, or -1 after a launch error.

@@ -1711,57 +1711,114 @@ __global__ void __launch_bounds__(kBlock) class_map_kernel(RunView v) {
   }
 }
 
-// The class map of a run with the region-ordered first pass, a tile of
-// kOrdTile positions per block: also the region plane (the filter region of
-// every position's k-mer) and, per tile, its positions of every (class,
-// region) pair (o_thist, tile-major) and of every (class, warp chunk of
-// kOrdTile / 8 positions) (o_wcount, class-major) and of every class
-// (o_tcount, class-major).
+// The sorted tiles of a run with the region-ordered first pass, instead of a
+// class map: every tile of kOrdTile positions lists the positions that have a
+// k-mer, sorted by (class, filter region) -- 16 bits each, bits 0-13 the
+// position within the tile, kOrdEntrySentinel for the first or last k-mer of a
+// string -- with the count of every (class, region) pair (o_thist) and the first
+// entry of every class (o_first). A round then reads exactly its members, in
+// the order of the buckets their records go to: the scatter needs no
+// compaction, no rank per member and no staging to write whole runs, and the
+// gather reads the decisions of a run as consecutive bits. (With a class byte
+// and a region byte per position instead, every round read 2 bytes of every
+// position and compacted, ranked and staged its members: scatter and gather
+// took 10.6 + 7.1 ps per position of a 6 Gbp build of four rounds.)
+//
+// A block sorts a tile in shared memory: the walk counts the pairs with
+// atomics that return each position's rank, a scan gives every pair its place.
+constexpr int kSortBlock = 512;
+constexpr uint32_t kOrdEntryPos = 0x3FFFu, kOrdEntrySentinel = 0x4000u;
+constexpr uint32_t kSortNone = 0xFFFFFFFFu;
+// per position its pair, rank and sentinel flag, then the sorted list, then the counts
+constexpr size_t kSortBytes = (size_t)kOrdTile * 6 + (size_t)kOrdMaxHist * 4;
+
 template <int KW>
-__global__ void __launch_bounds__(kBlock) class_map_ord_kernel(RunView v) {
-  constexpr int kChunks = (int)(kOrdTile / ((uint64_t)kBlock * kInsertR));  // 4
-  constexpr int kWarpChunks = kBlock / 32;                                   // 8
+__global__ void __launch_bounds__(kSortBlock, 2) class_sort_kernel(RunView v) {
+  extern __shared__ __align__(16) unsigned char sort_dyn_s[];
+  uint32_t* ent = reinterpret_cast<uint32_t*>(sort_dyn_s);            // kOrdTile
+  uint16_t* list = reinterpret_cast<uint16_t*>(ent + kOrdTile);       // kOrdTile
+  uint32_t* hist = reinterpret_cast<uint32_t*>(list + kOrdTile);      // L * R
   __shared__ uint32_t cuts_s[kMaxMapRounds + 1];
-  __shared__ uint32_t thist_s[kOrdMaxHist];
-  __shared__ uint32_t wcnt_s[kWarpChunks * kMaxMapRounds];
-  for (int i = threadIdx.x; i <= v.rounds; i += kBlock) cuts_s[i] = v.cuts[i];
+  __shared__ uint32_t warp_s[kSortBlock / 32];
+  constexpr int kUnits = (int)(kOrdTile / kInsertR);  // walks of 16 positions per tile
   const uint32_t R = v.o_regions, L = (uint32_t)v.rounds, nh = L * R;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (L > 1)
+    for (uint32_t i = threadIdx.x; i <= L; i += kSortBlock) cuts_s[i] = v.cuts[i];
+  // regions are runs of blocks (four words each): the top bits of H give them directly
+  const bool by_block = v.o_lg_region_words >= 2;
+  const int rshift = by_block ? 64 - v.lg_blocks + v.o_lg_region_words - 2 : 0;  // 64: one region
   for (uint64_t t = blockIdx.x; t < v.o_tiles; t += gridDim.x) {
-    for (uint32_t i = threadIdx.x; i < nh; i += kBlock) thist_s[i] = 0;
-    for (uint32_t i = threadIdx.x; i < kWarpChunks * L; i += kBlock) wcnt_s[i] = 0;
+    for (uint32_t i = threadIdx.x; i < nh; i += kSortBlock) hist[i] = 0;
     __syncthreads();
-    for (int c = 0; c < kChunks; ++c) {
-      const uint64_t p0 = t * kOrdTile + ((uint64_t)c * kBlock + threadIdx.x) * kInsertR;
-      if (p0 >= v.m) break;
-      // the warp chunk of these positions: kOrdTile / 8 = 2048 positions, 128 threads' worth
-      const uint32_t wc = (uint32_t)((((uint64_t)c * kBlock + threadIdx.x) * kInsertR) / (kOrdTile / kWarpChunks));
-      uint32_t w[4] = {0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u};
-      uint32_t r[4] = {0u, 0u, 0u, 0u};
+    for (int unit = threadIdx.x; unit < kUnits; unit += kSortBlock) {
+      const uint64_t p0 = t * kOrdTile + (uint64_t)unit * kInsertR;
+      if (p0 >= v.m) {
+#pragma unroll
+        for (int i = 0; i < kInsertR; ++i) ent[i * kUnits + unit] = kSortNone;
+        continue;
+      }
       walk<KW, kInsertR>(v, p0, [&](int i, uint64_t, bool valid, const auto& oc) {
-        if (!valid) return;
-        const uint32_t cls = class_of_bin(cuts_s, v.rounds, (uint32_t)oc.H & v.qmask);
-        w[i >> 2] = (w[i >> 2] & ~(0xFFu << (8 * (i & 3)))) | ((cls | (oc.sentinel ? kCmSentinel : 0u)) << (8 * (i & 3)));
-        const uint32_t reg = ord_region(v, oc.H, second_hash(oc.H));
-        r[i >> 2] |= reg << (8 * (i & 3));
-        atomicAdd(thist_s + cls * R + reg, 1u);
-        atomicAdd(wcnt_s + wc * L + cls, 1u);
+        uint32_t e = kSortNone;
+        if (valid) {
+          const uint32_t cls = L > 1 ? class_of_bin(cuts_s, (int)L, (uint32_t)oc.H & v.qmask) : 0u;
+          const uint32_t reg = by_block ? (rshift < 64 ? (uint32_t)(oc.H >> rshift) : 0u)
+                                        : ord_region(v, oc.H, second_hash(oc.H));
+          const uint32_t bin = cls * R + reg;
+          e = (bin << 16) | atomicAdd(hist + bin, 1u) | (oc.sentinel ? kOrdEntrySentinel : 0u);
+        }
+        ent[i * kUnits + unit] = e;  // bin < 2^12, rank < 2^14
       });
-      *reinterpret_cast<uint4*>(v.cmap + p0) = make_uint4(w[0], w[1], w[2], w[3]);
-      *reinterpret_cast<uint4*>(v.rplane + p0) = make_uint4(r[0], r[1], r[2], r[3]);
     }
     __syncthreads();
-    // at most kOrdTile = 16384 positions per tile: every count fits 16 bits
-    uint16_t* th = v.o_thist + t * nh;
-    for (uint32_t i = threadIdx.x; i < nh; i += kBlock) th[i] = (uint16_t)thist_s[i];
-    for (uint32_t i = threadIdx.x; i < kWarpChunks * L; i += kBlock) {
-      const uint32_t cls = i % L, wc = i / L;
-      v.o_wcount[((uint64_t)cls * v.o_tiles + t) * kWarpChunks + wc] = (uint16_t)wcnt_s[i];
+    // exclusive scan of the counts (nh <= 4096: at most 8 per thread), which go out first
+    uint32_t total;
+    {
+      const uint32_t per = (nh + kSortBlock - 1) / kSortBlock;
+      const uint32_t i0 = min(nh, threadIdx.x * per), i1 = min(nh, i0 + per);
+      uint16_t* th = v.o_thist + t * nh;
+      uint32_t sum = 0;
+      for (uint32_t i = i0; i < i1; ++i) {
+        const uint32_t c = hist[i];
+        th[i] = (uint16_t)c;  // at most kOrdTile = 16384
+        sum += c;
+      }
+      uint32_t inc = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      if (lane == 31) warp_s[wid] = inc;
+      __syncthreads();
+      uint32_t before = 0;
+      total = 0;
+#pragma unroll
+      for (int w = 0; w < kSortBlock / 32; ++w) {
+        before += w < wid ? warp_s[w] : 0u;
+        total += warp_s[w];
+      }
+      uint32_t at = before + inc - sum;
+      uint16_t* first = v.o_first + t * (L + 1);
+      for (uint32_t i = i0; i < i1; ++i) {
+        const uint32_t c = hist[i];
+        hist[i] = at;
+        if (i % R == 0) first[i / R] = (uint16_t)at;
+        at += c;
+      }
+      if (threadIdx.x == 0) first[L] = (uint16_t)total;
     }
-    for (uint32_t cls = threadIdx.x; cls < L; cls += kBlock) {
-      uint32_t tot = 0;
-      for (int wc = 0; wc < kWarpChunks; ++wc) tot += wcnt_s[wc * L + cls];
-      v.o_tcount[(uint64_t)cls * v.o_tiles + t] = tot;
+    __syncthreads();
+    for (int e0 = threadIdx.x; e0 < (int)kOrdTile; e0 += kSortBlock) {
+      const uint32_t e = ent[e0];
+      if (e == kSortNone) continue;
+      const uint32_t pos = (uint32_t)(e0 & (kUnits - 1)) * kInsertR + (uint32_t)(e0 / kUnits);
+      list[hist[e >> 16] + (e & 0x3FFFu)] = (uint16_t)(pos | (e & kOrdEntrySentinel));
     }
+    __syncthreads();
+    uint4* out = reinterpret_cast<uint4*>(v.o_list + t * kOrdTile);
+    const uint4* in = reinterpret_cast<const uint4*>(list);
+    for (uint32_t i = threadIdx.x; i < (total + 7) / 8; i += kSortBlock) out[i] = in[i];
     __syncthreads();
   }
 }
@@ -1811,7 +1868,6 @@ __device__ __forceinline__ bool ordered_round(const RunView& v) {
 template <int KW, int HB, bool BKT = false>
 __global__ void __launch_bounds__(kBlock) pass1_insert_cm_kernel(RunView v, int round) {
   __shared__ uint16_t idx_s[kBlock / 32][kCmWindow];
-  if (ordered_round(v)) return;  // the region-ordered kernels take this round
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   uint16_t* idx = idx_s[wid];
   const uint64_t stride = (uint64_t)gridDim.x * kBlock * 16;
@@ -1841,7 +1897,6 @@ template <int KW, int HB>
 __global__ void __launch_bounds__(kBlock) pass1_probe_cm_kernel(RunView v, int round) {
   __shared__ uint16_t idx_s[kBlock / 32][kCmWindow];
   __shared__ uint32_t keep_s[kBlock / 32][kCmWindow / 32];
-  if (ordered_round(v)) return;  // the region-ordered kernels take this round
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   uint16_t* idx = idx_s[wid];
   uint32_t* keep_w = keep_s[wid];
@@ -1929,16 +1984,13 @@ __global__ void __launch_bounds__(kBlock) pass1_probe_cm_kernel(RunView v, int r
 // then the probes bucket by bucket -- so that the random accesses of a region
 // all hit L2 -- and gathers the probe's decisions back in position order.
 //
-// Buckets: the class map counted the positions of every (class, region)
-// pair per tile, so a round's buckets are laid out exactly (each a multiple
-// of 32 slots). Tiles: kOrdTile consecutive positions, each warp of the block
-// taking kOrdTile / 8 of them (kOrdTileWindows / 8 windows). A tile's records
-// for a bucket are consecutive in the bucket, in tile order: a scan over the
-// tiles' counts gives every tile its room in every bucket (o_meta). The
-// members of a round are numbered in position order (o_tbase holds every
-// tile's first number); o_perm[member] is the member's rank within its
-// tile's room, so that the gather finds the member's decision bit at
-// o_start[bucket] + room + rank.
+// Buckets: the sorted tiles (class_sort_kernel) hold the count of every
+// (class, region) pair per tile, so a round's buckets are laid out exactly
+// (each a multiple of 32 slots). A tile's records for a bucket are consecutive
+// in the bucket, in tile order and in the order of the tile's list: a scan over
+// the tiles' counts gives every tile its room in every bucket (o_meta), and a
+// member's slot is its bucket's start plus its tile's room plus its index
+// within its run of the list.
 //
 // A record: bits 0-21 the word within its region, 22-51 the bits 32-61 of G
 // (the bit bases of up to 6 bits per item), 52-56 and 57-61 the items (two
@@ -1946,7 +1998,6 @@ __global__ void __launch_bounds__(kBlock) pass1_probe_cm_kernel(RunView v, int r
 // the records (k <= 27) a record holds the occurrence instead (fused_record).
 // ---------------------------------------------------------------------------
 
-constexpr int kOrdWarpWindows = kOrdTileWindows / (kBlock / 32);  // windows per warp and tile
 constexpr uint32_t kOrdPiece = 4096;  // records per apply or probe work item (a multiple of 32)
 constexpr unsigned long long kOrdSentinel = 1ull << 62;
 
@@ -1957,10 +2008,14 @@ constexpr unsigned long long kOrdSentinel = 1ull << 62;
 // palindrome), 2-3 and 0-1 the predecessor and successor bases -- and the
 // kernels that apply it recompute H, G, the filter word and the items.
 __device__ __forceinline__ unsigned long long fused_record(const RunView& v, uint64_t g, bool sentinel) {
-  const Key f = load_kmer<1>(v.packed, g, v.k);
+  // one window of 32 bases from the predecessor on holds it all (k + 2 <= 29)
+  const uint64_t x = sentinel ? bases32(v.packed, g) >> 2 : bases32(v.packed, g - 1);
+  Key f;
+  f.hi = 0;
+  f.lo = (x << 2) >> (64 - 2 * v.k);
   const Key r = v.both ? revcomp<1>(f, v.k) : f;
-  const uint32_t pred = sentinel ? 0u : base_at(v.packed, g - 1);
-  const uint32_t succ = sentinel ? 0u : base_at(v.packed, g + v.k);
+  const uint32_t pred = sentinel ? 0u : (uint32_t)(x >> 62);
+  const uint32_t succ = sentinel ? 0u : (uint32_t)(x >> (60 - 2 * v.k)) & 3u;
   const bool use_f = !v.both || !key_less(r, f);
   const bool use_r = v.both && !key_less(f, r);
   const uint64_t key = use_f ? f.lo : r.lo;
@@ -1988,7 +2043,10 @@ __device__ __forceinline__ FusedOcc fused_occ(unsigned long long rec) {
 // The fused pass-2 table: bucket b owns the o_tcap one-word slots (key << 9 |
 // mask) from b * o_tcap, so that its inserts and lookups stay in L2 beside
 // the filter region; a k-mer starts at bits 16-47 of H scaled to o_tcap
-// (Lemire's multiply-high) and probes linearly within the region.
+// (Lemire's multiply-high) and probes linearly within the part. Slot by slot,
+// unlike the direct table: the whole reserve is the table, at a load of a few
+// percent, so that the first slot mostly decides (a sector at a time took the
+// probe of 6 Gbp from 7.6 to 11.4 ps per position).
 __device__ __forceinline__ bool fused_table_insert(const RunView& v, uint32_t b, uint64_t key, uint64_t H,
                                                    uint32_t tbits) {
   const uint32_t cap = v.o_tcap;
@@ -2020,118 +2078,6 @@ __device__ __forceinline__ int fused_table_find(const RunView& v, uint32_t b, ui
   return -1;
 }
 
-// A lane's 16 positions of the window at wbase: their class and region bytes.
-__device__ __forceinline__ void ord_lane_bytes(const RunView& v, uint64_t wbase, uint4* cls, uint4* reg) {
-  const uint64_t p0 = wbase + 16 * (uint64_t)(threadIdx.x & 31);
-  *cls = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
-  *reg = make_uint4(0u, 0u, 0u, 0u);
-  if (p0 < v.m) {
-    *cls = __ldcg(reinterpret_cast<const uint4*>(v.cmap + p0));
-    *reg = __ldcg(reinterpret_cast<const uint4*>(v.rplane + p0));
-  }
-}
-
-// Bit i: the lane's position i is of this round's class (act), a sentinel
-// (sent), has a k-mer (val).
-__device__ __forceinline__ void ord_lane_bits(const uint4& q, int round, uint32_t* act, uint32_t* sent,
-                                              uint32_t* val) {
-  const uint32_t part[4] = {q.x, q.y, q.z, q.w};
-  const uint32_t want = (uint32_t)round * 0x01010101u;
-  uint32_t a = 0, s = 0, l = 0;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    a |= byte_bits(__vcmpeq4(part[c] & 0xBFBFBFBFu, want)) << (4 * c);
-    s |= byte_bits(part[c] << 1) << (4 * c);
-    l |= byte_bits(~part[c]) << (4 * c);
-  }
-  *act = a;
-  *sent = s;
-  *val = l;
-}
-
-__device__ __forceinline__ uint32_t uint4_byte(const uint4& q, uint32_t i) {
-  const uint32_t w = i < 8 ? (i < 4 ? q.x : q.y) : (i < 12 ? q.z : q.w);
-  return (w >> (8 * (i & 3))) & 0xFFu;
-}
-
-// compact_window with the region of every listed position in reg[0 .. n).
-__device__ __forceinline__ uint32_t compact_window_ord(const RunView& v, uint64_t wbase, int round, uint16_t* idx,
-                                                       uint8_t* reg) {
-  const int lane = threadIdx.x & 31;
-  uint4 q, rq;
-  ord_lane_bytes(v, wbase, &q, &rq);
-  uint32_t act, sent, val;
-  ord_lane_bits(q, round, &act, &sent, &val);
-  const uint32_t n = __popc(act);
-  uint32_t inc = n;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += y;
-  }
-  uint32_t at = inc - n;
-  while (act) {
-    const uint32_t i = __ffs(act) - 1;
-    act &= act - 1;
-    idx[at] = (uint16_t)((16 * lane + i) | (((sent >> i) & 1u) << 9));
-    reg[at] = (uint8_t)uint4_byte(rq, i);
-    ++at;
-  }
-  __syncwarp();
-  return __shfl_sync(0xffffffffu, inc, 31);
-}
-
-// Members of every (round, tile): thread blocks of the scan below take
-// kOrdScanTiles tiles of one round each.
-
-// o_tsum[round * chunks + c] = members of the round in tiles [c * 1024, (c + 1) * 1024).
-__global__ void __launch_bounds__(kBlock) ord_tile_sum_kernel(RunView v, uint64_t chunks) {
-  const uint64_t r = blockIdx.x / chunks, c = blockIdx.x % chunks;
-  const uint32_t* cnt = v.o_tcount + r * v.o_tiles;
-  unsigned long long s = 0;
-  for (uint64_t t = c * kOrdScanTiles + threadIdx.x; t < min((c + 1) * kOrdScanTiles, v.o_tiles); t += kBlock)
-    s += cnt[t];
-  __shared__ unsigned long long part[kBlock / 32];
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long t = 0;
-    for (int w = 0; w < kBlock / 32; ++w) t += part[w];
-    v.o_tsum[blockIdx.x] = t;
-  }
-}
-
-// o_tbase[round * tiles + t] = members of the round in tiles before t.
-__global__ void __launch_bounds__(kBlock) ord_tile_scan_kernel(RunView v, uint64_t chunks) {
-  const uint64_t r = blockIdx.x / chunks, c = blockIdx.x % chunks;
-  unsigned long long before = 0;
-  for (uint64_t i = threadIdx.x; i < c; i += kBlock) before += v.o_tsum[r * chunks + i];
-  __shared__ unsigned long long part[kBlock / 32];
-  __shared__ unsigned long long carry_s;
-  before = warp_sum(before);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = before;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long t = 0;
-    for (int w = 0; w < kBlock / 32; ++w) t += part[w];
-    carry_s = t;
-  }
-  __syncthreads();
-  const uint32_t* cnt = v.o_tcount + r * v.o_tiles;
-  unsigned long long* base = v.o_tbase + r * v.o_tiles;
-  for (uint64_t t0 = c * kOrdScanTiles; t0 < min((c + 1) * kOrdScanTiles, v.o_tiles); t0 += kBlock) {
-    const uint64_t t = t0 + threadIdx.x;
-    const uint32_t x = t < v.o_tiles ? cnt[t] : 0u;
-    uint32_t tot;
-    const uint32_t ex = block_exclusive_scan(x, &tot);
-    if (t < v.o_tiles) base[t] = carry_s + ex;
-    __syncthreads();
-    if (threadIdx.x == 0) carry_s += tot;
-    __syncthreads();
-  }
-}
-
 // Exclusive scan of x over the block (blockDim.x == kBlock), 64-bit.
 __device__ __forceinline__ unsigned long long block_exclusive_scan64(unsigned long long x, unsigned long long* total) {
   __shared__ unsigned long long warp_tot[kBlock / 32];
@@ -2159,16 +2105,32 @@ __device__ __forceinline__ unsigned long long block_exclusive_scan64(unsigned lo
 // The rooms of a round's tiles in its buckets, in tile order: o_meta[t * R + b]
 // = the round's members of bucket b in the tiles before t. Three steps over
 // chunks of kOrdScanTiles tiles: the chunks' sums, their prefix per bucket
-// (with every bucket's total, o_btot), then every tile's room.
+// (with every bucket's total, o_btot), then every tile's room. The counts of
+// kRoomAhead tiles are loaded before any of them is used: one after the other
+// they were a chain of L2 round trips per thread.
+constexpr int kRoomAhead = 8;
+static_assert(kOrdScanTiles % kRoomAhead == 0, "whole groups of tiles");
+
+template <typename F>
+__device__ __forceinline__ void for_tile_counts(const RunView& v, int round, F&& fn) {
+  const uint32_t R = v.o_regions, nh = (uint32_t)v.rounds * R;
+  const uint64_t t0 = (uint64_t)blockIdx.x * kOrdScanTiles, t1 = min(t0 + kOrdScanTiles, v.o_tiles);
+  const uint16_t* th = v.o_thist + (uint64_t)round * R + threadIdx.x;
+  for (uint64_t t = t0; t < t1; t += kRoomAhead) {
+    uint32_t c[kRoomAhead];
+#pragma unroll
+    for (int u = 0; u < kRoomAhead; ++u) c[u] = t + u < t1 ? __ldg(th + (t + u) * nh) : 0u;
+#pragma unroll
+    for (int u = 0; u < kRoomAhead; ++u)
+      if (t + u < t1) fn(t + u, c[u]);
+  }
+}
+
 __global__ void __launch_bounds__(kBlock) ord_room_sum_kernel(RunView v, int round) {
-  const uint32_t R = v.o_regions, b = threadIdx.x, nh = (uint32_t)v.rounds * R;
-  if (b >= R) return;
-  const uint64_t c = blockIdx.x, t1 = min((c + 1) * kOrdScanTiles, v.o_tiles);
-  const uint16_t* th = v.o_thist + (uint64_t)round * R + b;
+  if (threadIdx.x >= v.o_regions) return;
   uint32_t s = 0;
-#pragma unroll 8
-  for (uint64_t t = c * kOrdScanTiles; t < t1; ++t) s += th[t * nh];
-  v.o_csum[c * R + b] = s;
+  for_tile_counts(v, round, [&](uint64_t, uint32_t c) { s += c; });
+  v.o_csum[(uint64_t)blockIdx.x * v.o_regions + threadIdx.x] = s;
 }
 
 __global__ void __launch_bounds__(kBlock) ord_room_prefix_kernel(RunView v, uint64_t chunks) {
@@ -2190,34 +2152,32 @@ __global__ void __launch_bounds__(kBlock) ord_room_prefix_kernel(RunView v, uint
 }
 
 __global__ void __launch_bounds__(kBlock) ord_room_scan_kernel(RunView v, int round) {
-  const uint32_t R = v.o_regions, b = threadIdx.x, nh = (uint32_t)v.rounds * R;
-  if (b >= R) return;
-  const uint64_t c = blockIdx.x, t1 = min((c + 1) * kOrdScanTiles, v.o_tiles);
-  const uint16_t* th = v.o_thist + (uint64_t)round * R + b;
-  unsigned long long run = v.o_cpre[c * R + b];
-  for (uint64_t t = c * kOrdScanTiles; t < t1; ++t) {
-    v.o_meta[t * R + b] = (uint32_t)run;  // within a bucket below 2^32 (the setup checks)
-    run += th[t * nh];
-  }
+  const uint32_t R = v.o_regions;
+  if (threadIdx.x >= R) return;
+  unsigned long long run = v.o_cpre[(uint64_t)blockIdx.x * R + threadIdx.x];
+  for_tile_counts(v, round, [&](uint64_t t, uint32_t c) {
+    v.o_meta[t * R + threadIdx.x] = (uint32_t)run;  // within a bucket below 2^32 (the setup checks)
+    run += c;
+  });
 }
 
 // Before a round's scatter: the buckets' starts (each a multiple of 32), the
 // work tickets cleared, and whether the round's records fit (else the direct
 // kernels take the round). One block.
 __global__ void __launch_bounds__(kBlock) ord_setup_kernel(RunView v, int round) {
-  const uint32_t R = v.o_regions;
-  for (uint32_t b = threadIdx.x; b < R; b += kBlock) v.o_fill[(uint64_t)b * kOrdFillStride] = (uint32_t)v.o_btot[b];
+  static_assert(kOrdMaxRegions <= kBlock, "one thread per bucket");
+  const uint32_t R = v.o_regions, b = threadIdx.x;
+  const unsigned long long n = b < R ? v.o_btot[b] : 0ull;
+  unsigned long long total;
+  const unsigned long long start = block_exclusive_scan64((n + 31) & ~31ull, &total);
+  if (b < R) {
+    v.o_fill[(uint64_t)b * kOrdFillStride] = (uint32_t)n;
+    v.o_start[b] = start;
+  }
+  const int fits = __syncthreads_and(n < (1ull << 32));  // slots within a bucket are 32-bit
   if (threadIdx.x == 0) {
-    uint64_t at = 0;
-    bool fits = true;
-    for (uint32_t b = 0; b < R; ++b) {
-      v.o_start[b] = at;
-      const uint64_t n = v.o_btot[b];
-      fits = fits && n < (1ull << 32);  // slots within a bucket are 32-bit
-      at += (n + 31) & ~31ull;
-    }
-    v.o_start[R] = at;
-    v.hdr->ord_ok = (fits && at <= v.o_rec_cap) ? 1u : 0u;
+    v.o_start[R] = total;
+    v.hdr->ord_ok = (fits && total <= v.o_rec_cap) ? 1u : 0u;
     v.hdr->ord_rounds += v.hdr->ord_ok;
     v.hdr->ord_ticket[0] = 0;
     v.hdr->ord_ticket[1] = 0;
@@ -2225,94 +2185,78 @@ __global__ void __launch_bounds__(kBlock) ord_setup_kernel(RunView v, int round)
   }
 }
 
-// Records a tile stages in shared memory, sorted by bucket, before writing
-// them out run by run (a tile with more members writes them one by one).
-constexpr uint32_t kOrdStage = 4352;  // four blocks of 256 threads per SM (228 KB of shared memory)
-constexpr size_t kOrdStageBytes = (size_t)kOrdStage * 9;  // the records, then their buckets
+// A tile's members of a round, in the order of the tile's list (by bucket): the
+// list from `list` on, `n` members; member i is in bucket bucket_s[i], at slot
+// delta_s[bucket] + i of the round's records.
+struct TileMembers {
+  const uint16_t* list;
+  uint32_t n;
+};
+
+// Load a tile's members (called by the whole block; ends with a barrier). The
+// members' buckets are filled in by R / kBlock-th of the threads each, run by run.
+__device__ __forceinline__ TileMembers ord_tile(const RunView& v, uint64_t t, int round, const uint64_t* start_s,
+                                                unsigned long long* delta_s, uint32_t* run_s, uint8_t* bucket_s) {
+  const uint32_t R = v.o_regions, L = (uint32_t)v.rounds, b = threadIdx.x;
+  const uint32_t count = b < R ? v.o_thist[(t * L + round) * R + b] : 0u;
+  const uint32_t room = b < R ? __ldg(v.o_meta + t * R + b) : 0u;
+  TileMembers tm;
+  const uint16_t* first = v.o_first + t * (L + 1);
+  tm.list = v.o_list + t * kOrdTile + first[round];
+  const uint32_t off = block_exclusive_scan(count, &tm.n);
+  if (b < R) {
+    delta_s[b] = start_s[b] + room - off;
+    run_s[b] = off | (count << 16);  // both at most kOrdTile = 2^14
+  }
+  __syncthreads();
+  // R is a power of two of at most kBlock: kBlock / R threads per run
+  const uint32_t r = threadIdx.x & (R - 1u), x = run_s[r], end = (x & 0xFFFFu) + (x >> 16);
+  for (uint32_t i = (x & 0xFFFFu) + threadIdx.x / R; i < end; i += kBlock / R) bucket_s[i] = (uint8_t)r;
+  __syncthreads();
+  return tm;
+}
 
 // Algorithm 1, insert loop, first pass, over this round's class: one record
-// per position into the bucket of its filter region (tiles grid-strided).
+// per member into the bucket of its filter region (tiles grid-strided). The
+// members come in bucket order, so that consecutive threads write consecutive
+// records of a run. A few members per thread are in flight at a time.
 template <int KW, int HB, bool FUSED>
 __global__ void __launch_bounds__(kBlock) ord_scatter_kernel(RunView v, int round) {
-  extern __shared__ __align__(16) unsigned char ord_dyn_s[];
-  unsigned long long* stage_rec = reinterpret_cast<unsigned long long*>(ord_dyn_s);
-  uint8_t* stage_b = ord_dyn_s + (size_t)kOrdStage * 8;
-  __shared__ uint16_t idx_s[kBlock / 32][kCmWindow];
-  __shared__ uint8_t reg_s[kBlock / 32][kCmWindow];
-  __shared__ uint32_t cur_s[kOrdMaxRegions];   // members per bucket, then the next rank
-  __shared__ uint32_t room_s[kOrdMaxRegions];  // where the tile's room starts in every bucket
-  __shared__ uint32_t off_s[kOrdMaxRegions];   // where every bucket's run starts in the stage
-  __shared__ unsigned long long start_s[kOrdMaxRegions];
-  __shared__ uint32_t wcnt_s[kBlock / 32];
+  __shared__ uint8_t bucket_s[kOrdTile];
+  __shared__ unsigned long long delta_s[kOrdMaxRegions];
+  __shared__ uint64_t start_s[kOrdMaxRegions];
+  __shared__ uint32_t run_s[kOrdMaxRegions];
   if (!ordered_round(v)) return;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const uint32_t R = v.o_regions;
-  for (uint32_t b = threadIdx.x; b < R; b += kBlock) start_s[b] = v.o_start[b];
+  for (uint32_t b = threadIdx.x; b < v.o_regions; b += kBlock) start_s[b] = v.o_start[b];
   const uint64_t local_mask = (1ull << v.o_lg_region_words) - 1ull;
-  const unsigned long long* tbase = v.o_tbase + (uint64_t)round * v.o_tiles;
-  const uint64_t n_tiles = (v.p_end - v.p_begin + kOrdTile - 1) / kOrdTile;
-  for (uint64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    const uint64_t tpos = v.p_begin + t * kOrdTile;
-    // the tile's members per bucket (o_thist) and per warp chunk (o_wcount),
-    // and its rooms (o_meta)
-    const uint32_t mine = threadIdx.x < R ? v.o_thist[(t * v.rounds + round) * R + threadIdx.x] : 0u;
-    uint32_t total;
-    const uint32_t off = block_exclusive_scan(mine, &total);
-    if (threadIdx.x < R) {
-      room_s[threadIdx.x] = __ldg(v.o_meta + t * R + threadIdx.x);
-      off_s[threadIdx.x] = off;
-      cur_s[threadIdx.x] = 0;
-    }
-    if (threadIdx.x == 0) {
-      const uint16_t* wcnt = v.o_wcount + ((uint64_t)round * v.o_tiles + t) * (kBlock / 32);
-      uint32_t run = 0;
-      for (int w = 0; w < kBlock / 32; ++w) {
-        wcnt_s[w] = run;
-        run += wcnt[w];
-      }
-    }
-    __syncthreads();
-    const bool staged = total <= kOrdStage;
-    uint64_t mi = tbase[t] + wcnt_s[wid];  // number of the warp's next member
-    for (int q = 0; q < kOrdWarpWindows; ++q) {
-      const uint64_t wbase = tpos + (uint64_t)(wid * kOrdWarpWindows + q) * kCmWindow;
-      if (wbase >= v.p_end) break;
-      const uint32_t n = compact_window_ord(v, wbase, round, idx_s[wid], reg_s[wid]);
-      for (uint32_t j = lane; j < n; j += 32) {
-        const uint32_t e = idx_s[wid][j], b = reg_s[wid][j];
-        const uint32_t rank = atomicAdd(&cur_s[b], 1u);
-        v.o_perm[mi + j] = (uint16_t)rank;
-        const bool sentinel = (e >> 9) & 1u;
+  for (uint64_t t = blockIdx.x; t < v.o_tiles; t += gridDim.x) {
+    const TileMembers tm = ord_tile(v, t, round, start_s, delta_s, run_s, bucket_s);
+    constexpr int U = KW == 1 ? 4 : 2;
+    for (uint32_t i0 = threadIdx.x; i0 < tm.n; i0 += U * kBlock) {
+      uint32_t e[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) e[u] = i0 + u * kBlock < tm.n ? __ldcs(tm.list + i0 + u * kBlock) : 0u;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t i = i0 + u * kBlock;
+        if (i >= tm.n) break;
+        const bool sentinel = e[u] & kOrdEntrySentinel;
+        const uint64_t g = t * kOrdTile + (e[u] & kOrdEntryPos);
         unsigned long long rec;
         if constexpr (FUSED) {
-          rec = fused_record(v, wbase + (e & 511u), sentinel);
+          rec = fused_record(v, g, sentinel);
         } else {
           OccT<KW> oc;
-          read_listed<KW>(v, wbase + (e & 511u), sentinel, &oc);
+          read_listed<KW>(v, g, sentinel, &oc);
           const uint64_t G = second_hash(oc.H);
-          const uint32_t j1 = oc.j1, j2 = oc.j2;
           const uint64_t word = filter_index(v, oc.H, G);
-          rec = (word & local_mask) | (((G >> 32) & 0x3FFFFFFFull) << 22) | ((uint64_t)j1 << 52) |
-                ((uint64_t)j2 << 57) | (sentinel ? kOrdSentinel : 0ull);
+          rec = (word & local_mask) | (((G >> 32) & 0x3FFFFFFFull) << 22) | ((uint64_t)oc.j1 << 52) |
+                ((uint64_t)oc.j2 << 57) | (sentinel ? kOrdSentinel : 0ull);
         }
-        if (staged) {
-          stage_rec[off_s[b] + rank] = rec;
-          stage_b[off_s[b] + rank] = (uint8_t)b;
-        } else {
-          v.o_recs[start_s[b] + room_s[b] + rank] = rec;
-        }
+        v.o_recs[delta_s[bucket_s[i]] + i] = rec;
       }
-      mi += n;
-      __syncwarp();
     }
-    __syncthreads();
-    if (staged) {  // consecutive threads on consecutive records of a run
-      for (uint32_t i = threadIdx.x; i < total; i += kBlock) {
-        const uint32_t b = stage_b[i];
-        v.o_recs[start_s[b] + room_s[b] + (i - off_s[b])] = stage_rec[i];
-      }
-      __syncthreads();
-    }
+    __syncthreads();  // the shared arrays serve the next tile
   }
 }
 
@@ -2320,15 +2264,12 @@ __global__ void __launch_bounds__(kBlock) ord_scatter_kernel(RunView v, int roun
 // that the blocks in flight work on one or two regions at a time. first_s[b]:
 // the first item of bucket b (first_s[R]: the number of items).
 __device__ __forceinline__ void ord_items(const RunView& v, uint32_t* first_s) {
-  if (threadIdx.x == 0) {
-    uint32_t acc = 0;
-    for (uint32_t b = 0; b < v.o_regions; ++b) {
-      first_s[b] = acc;
-      const uint64_t n = __ldcg(v.o_fill + (uint64_t)b * kOrdFillStride);
-      acc += (uint32_t)((n + kOrdPiece - 1) / kOrdPiece);
-    }
-    first_s[v.o_regions] = acc;
-  }
+  const uint32_t b = threadIdx.x;  // at most kBlock buckets
+  const uint64_t n = b < v.o_regions ? __ldcg(v.o_fill + (uint64_t)b * kOrdFillStride) : 0ull;
+  uint32_t total;
+  const uint32_t first = block_exclusive_scan((uint32_t)((n + kOrdPiece - 1) / kOrdPiece), &total);
+  if (b < v.o_regions) first_s[b] = first;
+  if (b == 0) first_s[v.o_regions] = total;
   __syncthreads();
 }
 
@@ -2430,38 +2371,52 @@ __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
     const uint64_t start = __ldg(v.o_start + b);  // a multiple of 32, as is i0
     const uint64_t* recs = v.o_recs + start;
     const uint64_t region = (uint64_t)b << v.o_lg_region_words;
-    for (uint64_t w0 = i0 + 32 * wid; w0 < i1; w0 += kBlock) {
-      const uint64_t i = w0 + lane;
-      bool keep = false;
-      if (FUSED && i < i1) {  // the decision, and the candidate's edges into the region's table
-        const FusedOcc o = fused_occ(__ldcs(recs + i));
-        if (o.sentinel) {
-          keep = true;
+    // U chunks of 32 records per warp and step: their records, then their filter
+    // words, all in flight at once
+    constexpr int U = FUSED ? 2 : 4;
+    for (uint64_t w0 = i0 + 32 * wid; w0 < i1; w0 += U * kBlock) {
+      unsigned long long rec[U], word[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint64_t i = w0 + (uint64_t)u * kBlock + lane;
+        rec[u] = i < i1 ? __ldcs(recs + i) : ~0ull;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        word[u] = 0;
+        if (rec[u] == ~0ull) continue;
+        if constexpr (FUSED) {
+          const FusedOcc o = fused_occ(rec[u]);
+          if (!o.sentinel) word[u] = __ldcg(v.filter + filter_index(v, o.H, o.G));
         } else {
-          const uint64_t word = __ldcg(v.filter + filter_index(v, o.H, o.G));
-          const uint32_t pres = present_items<HB>(o.G, word, v.hashes);
-          keep = (pres >> 16) || __popc(pres & 0xFFFFu) >= 2;
-        }
-        if (keep && !fused_table_insert(v, b, o.key, o.H, o.tbits)) v.hdr->overflow = 1;
-      } else if (i < i1) {
-        const uint64_t r = __ldcs(recs + i);
-        const uint64_t word_index = region | (r & 0x3FFFFFull);
-        if (r & kOrdSentinel) {
-          keep = true;
-        } else {
-          const uint64_t G = ((r >> 22) & 0x3FFFFFFFull) << 32;
-          const uint64_t word = __ldcg(v.filter + word_index);
-          const uint32_t pres = present_items<HB>(G, word, v.hashes);
-          keep = (pres >> 16) || __popc(pres & 0xFFFFu) >= 2;
-        }
-        if (keep && !v.partial) {  // linear counting over a 2^-lc_sample_log2 sample of the k-mers
-          const uint64_t id = (word_index << 30) | ((r >> 22) & 0x3FFFFFFFull);
-          lc_mark(v, id * kLcMul);
+          if (!(rec[u] & kOrdSentinel)) word[u] = __ldcg(v.filter + (region | (rec[u] & 0x3FFFFFull)));
         }
       }
-      const uint32_t row = __ballot_sync(0xffffffffu, keep);
-      // fused: word pairs, the candidates' bits then the junctions' (ord_classify)
-      if (lane == 0) v.o_dec[((start + w0) >> 5) << (FUSED ? 1 : 0)] = row;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint64_t c = w0 + (uint64_t)u * kBlock;
+        if (c >= i1) break;  // the same for the whole warp
+        bool keep = false;
+        if (rec[u] != ~0ull) {
+          if constexpr (FUSED) {  // the decision, and the candidate's edges into the region's table
+            const FusedOcc o = fused_occ(rec[u]);
+            const uint32_t pres = present_items<HB>(o.G, word[u], v.hashes);
+            keep = o.sentinel || (pres >> 16) || __popc(pres & 0xFFFFu) >= 2;
+            if (keep && !fused_table_insert(v, b, o.key, o.H, o.tbits)) v.hdr->overflow = 1;
+          } else {
+            const uint64_t G = ((rec[u] >> 22) & 0x3FFFFFFFull) << 32;
+            const uint32_t pres = present_items<HB>(G, word[u], v.hashes);
+            keep = (rec[u] & kOrdSentinel) || (pres >> 16) || __popc(pres & 0xFFFFu) >= 2;
+            if (keep && !v.partial) {
+              const uint64_t id = ((region | (rec[u] & 0x3FFFFFull)) << 30) | ((rec[u] >> 22) & 0x3FFFFFFFull);
+              lc_mark(v, id * kLcMul);
+            }
+          }
+        }
+        const uint32_t row = __ballot_sync(0xffffffffu, keep);
+        // fused: word pairs, the candidates' bits then the junctions' (ord_classify)
+        if (lane == 0) v.o_dec[((start + c) >> 5) << (FUSED ? 1 : 0)] = row;
+      }
     }
   }
 }
@@ -2521,120 +2476,182 @@ __global__ void __launch_bounds__(kBlock) ord_classify_kernel(RunView v) {
   }
 }
 
-// The probe loop's outputs in position order: every member of the round's
-// class takes its decision from its record's slot (its tile's room in its
-// bucket plus its rank, o_perm); C_temp words, the candidate list segment of
-// the warp and the counts are as pass1_probe_cm_kernel writes them (with
-// fused records: C_temp words, and the junction bits ORed into C_final
-// instead of a list). Every
-// lane takes its own 16 positions of a window (at most 40 registers: six
-// blocks per SM).
-__global__ void __launch_bounds__(kBlock, 6) ord_gather_kernel(RunView v, int round) {
-  __shared__ uint32_t room_s[kOrdMaxRegions];
-  __shared__ unsigned long long start_s[kOrdMaxRegions];
-  __shared__ uint32_t wcnt_s[kBlock / 32];
-  if (!ordered_round(v)) return;
+// What a tile's decisions leave behind, called by the whole block with the
+// tile's candidate, junction (fused) and sentinel bits in shared memory: the
+// tile's words of C_temp, its junctions (fused) or, partial, its candidates in
+// C_final -- a tile has one block and rounds own disjoint positions, so no
+// atomic -- or its candidates in the warp's segment of the pass-2 list, in
+// position order. Clears the bits for the next tile.
+constexpr uint32_t kOrdTileWords = (uint32_t)(kOrdTile / 32);
+
+struct TileOut {
+  unsigned long long kept, junctions;
+  uint64_t seg_used;
+};
+
+__device__ __forceinline__ void ord_tile_out(const RunView& v, uint64_t t, bool fused, uint32_t* keep_s, uint32_t* jun_s,
+                                             uint32_t* sent_s, TileOut* o) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const uint32_t R = v.o_regions;
-  for (uint32_t b = threadIdx.x; b < R; b += kBlock) start_s[b] = v.o_start[b];
-  unsigned long long kept = 0, valid_n = 0, junctions = 0;
   const uint32_t warp_id = (blockIdx.x * kBlock + threadIdx.x) >> 5;
-  uint64_t* seg = v.cands + (uint64_t)warp_id * v.seg_cap;
-  uint32_t* seg32 = reinterpret_cast<uint32_t*>(v.cands) + (uint64_t)warp_id * v.seg_cap;
-  uint64_t seg_used = 0;
-  const unsigned long long* tbase = v.o_tbase + (uint64_t)round * v.o_tiles;
-  const uint64_t n_tiles = (v.p_end - v.p_begin + kOrdTile - 1) / kOrdTile;
-  for (uint64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    const uint64_t tpos = v.p_begin + t * kOrdTile;
-    for (uint32_t b = threadIdx.x; b < R; b += kBlock) room_s[b] = __ldg(v.o_meta + t * R + b);
-    if (threadIdx.x == 0) {
-      const uint16_t* wcnt = v.o_wcount + ((uint64_t)round * v.o_tiles + t) * (kBlock / 32);
-      uint32_t run = 0;
-      for (int w = 0; w < kBlock / 32; ++w) {
-        wcnt_s[w] = run;
-        run += wcnt[w];
+  constexpr uint32_t kPer = kOrdTileWords / (kBlock / 32);  // words per warp
+  for (uint32_t w0 = wid * kPer; w0 < (wid + 1) * kPer; w0 += 32) {
+    const uint64_t w = t * kOrdTileWords + w0 + lane;
+    const uint32_t keep = keep_s[w0 + lane], jun = jun_s[w0 + lane], sent = sent_s[w0 + lane];
+    keep_s[w0 + lane] = 0;
+    jun_s[w0 + lane] = 0;
+    sent_s[w0 + lane] = 0;
+    if (w < v.bitmap_words) {
+      v.ctemp[w] = keep;
+      const uint32_t add = v.partial ? keep : jun;
+      if (add) v.cfinal[w] |= add;
+    }
+    const uint32_t n = __popc(keep);
+    o->kept += n;
+    o->junctions += __popc(jun);
+    if (v.partial || fused) continue;
+    uint32_t inc = n;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+      if (lane >= d) inc += y;
+    }
+    uint64_t at = o->seg_used + inc - n;
+    for (uint32_t x = keep; x; x &= x - 1, ++at) {
+      const uint32_t i = __ffs(x) - 1;
+      const uint64_t g = w * 32 + i;
+      if (at < v.seg_cap) {
+        const uint32_t sentinel = (sent >> i) & 1u;
+        if (v.narrow) (reinterpret_cast<uint32_t*>(v.cands) + (uint64_t)warp_id * v.seg_cap)[at] = (uint32_t)g | (sentinel << 31);
+        else (v.cands + (uint64_t)warp_id * v.seg_cap)[at] = g | ((uint64_t)sentinel << 63);
+      }
+    }
+    o->seg_used += __shfl_sync(0xffffffffu, inc, 31);
+  }
+}
+
+// The counts and the list segment's length after a block's last tile.
+__device__ __forceinline__ void ord_counts_out(const RunView& v, bool fused, const TileOut& o) {
+  const uint32_t warp_id = (blockIdx.x * kBlock + threadIdx.x) >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    v.seg_count[warp_id] = (uint32_t)(o.seg_used < v.seg_cap ? o.seg_used : v.seg_cap);
+    if (o.seg_used > v.seg_cap) v.hdr->cand_overflow = 1;
+  }
+  block_add(o.kept, &v.hdr->pass1_kept);
+  block_add(o.kept, v.partial ? &v.hdr->pass2_kept : &v.hdr->round_kept);
+  if (fused) block_add(o.junctions, &v.hdr->pass2_kept);
+}
+
+// k-mer positions of a tile: the end of its last class.
+__device__ __forceinline__ uint32_t ord_tile_positions(const RunView& v, uint64_t t) {
+  return v.o_first[t * ((uint32_t)v.rounds + 1u) + (uint32_t)v.rounds];
+}
+
+// The probe loop's outputs in position order: every member of the round's
+// class takes its decision from its record's slot -- the members of a run read
+// consecutive bits -- and sets its bits of the tile in shared memory; then the
+// tile's words, list entries and counts go out (ord_tile_out).
+__global__ void __launch_bounds__(kBlock) ord_gather_kernel(RunView v, int round) {
+  __shared__ uint8_t bucket_s[kOrdTile];
+  __shared__ unsigned long long delta_s[kOrdMaxRegions];
+  __shared__ uint64_t start_s[kOrdMaxRegions];
+  __shared__ uint32_t run_s[kOrdMaxRegions];
+  __shared__ uint32_t keep_s[kOrdTileWords], jun_s[kOrdTileWords], sent_s[kOrdTileWords];
+  if (!ordered_round(v)) return;
+  for (uint32_t b = threadIdx.x; b < v.o_regions; b += kBlock) start_s[b] = v.o_start[b];
+  for (uint32_t i = threadIdx.x; i < kOrdTileWords; i += kBlock) keep_s[i] = jun_s[i] = sent_s[i] = 0;
+  const bool fused = v.o_fused, listed = !fused && !v.partial;
+  TileOut o{0, 0, 0};
+  unsigned long long valid_n = 0;
+  for (uint64_t t = blockIdx.x; t < v.o_tiles; t += gridDim.x) {
+    const TileMembers tm = ord_tile(v, t, round, start_s, delta_s, run_s, bucket_s);
+    if (threadIdx.x == 0) valid_n += ord_tile_positions(v, t);
+    constexpr int U = 4;
+    for (uint32_t i0 = threadIdx.x; i0 < tm.n; i0 += U * kBlock) {
+      uint2 d[U];
+      uint32_t e[U], bit[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t i = i0 + u * kBlock;
+        d[u] = make_uint2(0u, 0u);
+        if (i >= tm.n) continue;
+        e[u] = __ldcs(tm.list + i);
+        const uint64_t s = delta_s[bucket_s[i]] + i;
+        bit[u] = (uint32_t)s & 31u;
+        if (fused) d[u] = __ldg(reinterpret_cast<const uint2*>(v.o_dec) + (s >> 5));  // candidates, junctions
+        else d[u].x = __ldg(v.o_dec + (s >> 5));
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (i0 + u * kBlock >= tm.n || !((d[u].x >> bit[u]) & 1u)) continue;  // a junction is a candidate
+        const uint32_t pos = e[u] & kOrdEntryPos, m = 1u << (pos & 31u);
+        atomicOr(keep_s + (pos >> 5), m);
+        if ((d[u].y >> bit[u]) & 1u) atomicOr(jun_s + (pos >> 5), m);
+        if (listed && (e[u] & kOrdEntrySentinel)) atomicOr(sent_s + (pos >> 5), m);
       }
     }
     __syncthreads();
-    uint64_t mi = tbase[t] + wcnt_s[wid];  // number of the warp's next member
-    for (int q = 0; q < kOrdWarpWindows; ++q) {
-      const uint64_t wbase = tpos + (uint64_t)(wid * kOrdWarpWindows + q) * kCmWindow;
-      if (wbase >= v.p_end) break;
-      uint4 cq, rq;
-      ord_lane_bytes(v, wbase, &cq, &rq);
-      uint32_t act, sent, val;
-      ord_lane_bits(cq, round, &act, &sent, &val);
-      valid_n += __popc(val);
-      const uint32_t n = __popc(act);
-      uint32_t inc = n;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-      }
-      uint64_t at = mi + inc - n;  // number of the lane's first member
-      uint32_t keep = 0, jun = 0;
-      for (uint32_t a = act; a; a &= a - 1, ++at) {
-        const uint32_t i = __ffs(a) - 1, b = uint4_byte(rq, i);
-        const uint64_t s = start_s[b] + room_s[b] + __ldg(v.o_perm + at);
-        if (v.o_fused) {  // the candidate and junction words of the slot, in one load
-          const uint2 d = __ldg(reinterpret_cast<const uint2*>(v.o_dec) + (s >> 5));
-          keep |= ((d.x >> (s & 31)) & 1u) << i;
-          jun |= ((d.y >> (s & 31)) & 1u) << i;
-        } else {
-          keep |= ((__ldg(v.o_dec + (s >> 5)) >> (s & 31)) & 1u) << i;
-        }
-      }
-      mi += __shfl_sync(0xffffffffu, inc, 31);
-      // C_temp (and, fused, C_final): lanes 2i and 2i + 1 hold the halves of the window's word i
-      const uint32_t hi = __shfl_down_sync(0xffffffffu, keep, 1);
-      const uint32_t jhi = __shfl_down_sync(0xffffffffu, jun, 1);
-      if (!(lane & 1)) {
-        const uint64_t w = (wbase >> 5) + (lane >> 1);
-        const uint32_t word = keep | (hi << 16);
-        if (w < v.bitmap_words) {
-          v.ctemp[w] = word;
-          // rounds own disjoint positions; one writer per word
-          if (v.partial) {
-            v.cfinal[w] |= word;
-          } else if (v.o_fused) {
-            const uint32_t jw = jun | (jhi << 16);
-            if (jw) atomicOr(v.cfinal + w, jw);  // no wait on the word's other rounds' bits
-          }
-        }
-      }
-      const uint32_t kc = __popc(keep);
-      kept += kc;
-      junctions += __popc(jun);
-      if (v.partial || v.o_fused) continue;
-      uint32_t kinc = kc;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, kinc, o);
-        if (lane >= o) kinc += y;
-      }
-      uint64_t o = seg_used + kinc - kc;
-      for (uint32_t k = keep; k; k &= k - 1, ++o) {
-        const uint32_t i = __ffs(k) - 1;
-        const uint64_t g = wbase + 16 * (uint64_t)lane + i;
-        const uint32_t sentinel = (sent >> i) & 1u;
-        if (o < v.seg_cap) {
-          if (v.narrow) seg32[o] = (uint32_t)g | (sentinel << 31);
-          else seg[o] = g | ((uint64_t)sentinel << 63);
-        }
-      }
-      seg_used += __shfl_sync(0xffffffffu, kinc, 31);
+    ord_tile_out(v, t, fused, keep_s, jun_s, sent_s, &o);
+    __syncthreads();  // the shared arrays serve the next tile
+  }
+  ord_counts_out(v, fused, o);
+  if (round == v.count_round) block_add((unsigned long long)valid_n, &v.hdr->positions);
+}
+
+// The insert and the probe of a round whose records do not fit their room,
+// directly on the filter, over the round's members of every tile's list.
+template <int KW, int HB>
+__global__ void __launch_bounds__(kBlock) list_insert_kernel(RunView v, int round) {
+  if (ordered_round(v)) return;  // the region-ordered kernels took this round
+  for (uint64_t t = blockIdx.x; t < v.o_tiles; t += gridDim.x) {
+    const uint16_t* first = v.o_first + t * ((uint32_t)v.rounds + 1u);
+    const uint32_t a = first[round], b = first[round + 1];
+    for (uint32_t i = a + threadIdx.x; i < b; i += kBlock) {
+      const uint32_t e = v.o_list[t * kOrdTile + i];
+      OccT<KW> oc;
+      read_listed<KW>(v, t * kOrdTile + (e & kOrdEntryPos), e & kOrdEntrySentinel, &oc);
+      const uint64_t G = second_hash(oc.H);
+      const ItemPattern pat = item_pattern<HB>(G, v.hashes);
+      uint64_t m = item_bits(pat, oc.j1);
+      if (oc.j2 != oc.j1) m |= item_bits(pat, oc.j2);  // a palindrome's two orientations
+      atomicOr(filter_word(v, oc.H, G), (unsigned long long)m);
     }
-    __syncthreads();  // room_s and wcnt_s serve the next tile
   }
-  if (lane == 0) {
-    v.seg_count[warp_id] = (uint32_t)(seg_used < v.seg_cap ? seg_used : v.seg_cap);
-    if (seg_used > v.seg_cap) v.hdr->cand_overflow = 1;
+}
+
+template <int KW, int HB>
+__global__ void __launch_bounds__(kBlock) list_probe_kernel(RunView v, int round) {
+  __shared__ uint32_t keep_s[kOrdTileWords], jun_s[kOrdTileWords], sent_s[kOrdTileWords];
+  if (ordered_round(v)) return;  // the region-ordered kernels took this round
+  for (uint32_t i = threadIdx.x; i < kOrdTileWords; i += kBlock) keep_s[i] = jun_s[i] = sent_s[i] = 0;
+  __syncthreads();
+  TileOut o{0, 0, 0};
+  unsigned long long valid_n = 0;
+  for (uint64_t t = blockIdx.x; t < v.o_tiles; t += gridDim.x) {
+    const uint16_t* first = v.o_first + t * ((uint32_t)v.rounds + 1u);
+    const uint32_t a = first[round], b = first[round + 1];
+    if (threadIdx.x == 0) valid_n += ord_tile_positions(v, t);
+    for (uint32_t i = a + threadIdx.x; i < b; i += kBlock) {
+      const uint32_t e = v.o_list[t * kOrdTile + i], pos = e & kOrdEntryPos;
+      const bool sentinel = e & kOrdEntrySentinel;
+      OccT<KW> oc;
+      read_listed<KW>(v, t * kOrdTile + pos, sentinel, &oc);
+      const uint64_t G = second_hash(oc.H);
+      bool keep = sentinel;
+      if (!sentinel) {
+        const uint32_t pres = present_items<HB>(G, __ldcg(filter_word(v, oc.H, G)), v.hashes);
+        keep = (pres >> 16) || __popc(pres & 0xFFFFu) >= 2;
+      }
+      if (!keep) continue;
+      atomicOr(keep_s + (pos >> 5), 1u << (pos & 31u));
+      if (sentinel) atomicOr(sent_s + (pos >> 5), 1u << (pos & 31u));
+      if (!v.partial) lc_mark(v, G * kLcMul);
+    }
+    __syncthreads();
+    ord_tile_out(v, t, false, keep_s, jun_s, sent_s, &o);
+    __syncthreads();
   }
-  block_add(kept, &v.hdr->pass1_kept);
-  block_add(kept, v.partial ? &v.hdr->pass2_kept : &v.hdr->round_kept);
-  if (v.o_fused) block_add(junctions, &v.hdr->pass2_kept);
-  if (round == v.count_round) block_add(valid_n, &v.hdr->positions);
+  ord_counts_out(v, false, o);
+  if (round == v.count_round) block_add((unsigned long long)valid_n, &v.hdr->positions);
 }
 
 // Table slots per estimated distinct candidate: 2.5 for one-word slots
@@ -3408,6 +3425,64 @@ static void with_hashes(int h, F&& f) {
   }
 }
 
+// A round's first pass in filter-region order (and, fused, its second pass):
+// launches every kernel of it; *pv gets the list segments. Kernels launched, or -1.
+template <int KW, int HB>
+static int ordered_round_impl(const RunView& v, int round, cudaStream_t s, RunView* pv) {
+  const bool fused = KW == 1 && v.o_fused;
+  {
+    Timed t("ord_rooms", s);
+    const uint64_t chunks = (v.o_tiles + kOrdScanTiles - 1) / kOrdScanTiles;
+    ord_room_sum_kernel<<<(unsigned)chunks, kBlock, 0, s>>>(v, round);
+    ord_room_prefix_kernel<<<v.o_regions, kBlock, 0, s>>>(v, chunks);
+    ord_room_scan_kernel<<<(unsigned)chunks, kBlock, 0, s>>>(v, round);
+    ord_setup_kernel<<<1, kBlock, 0, s>>>(v, round);
+  }
+  {
+    Timed t("ord_scatter", s);
+    auto kern = ord_scatter_kernel<KW, HB, false>;
+    if constexpr (KW == 1)
+      if (fused) kern = ord_scatter_kernel<KW, HB, true>;
+    kern<<<grid_for(kern, kBlock, v.o_tiles * kBlock, v.blocks_per_sm), kBlock, 0, s>>>(v, round);
+  }
+  {
+    Timed t("ord_or", s);
+    auto kern = fused ? ord_or_kernel<HB, true> : ord_or_kernel<HB, false>;
+    kern<<<grid_for(kern, kBlock, ~0ull >> 1), kBlock, 0, s>>>(v);
+  }
+  {
+    Timed t("list_insert", s);
+    auto kern = list_insert_kernel<KW, HB>;
+    kern<<<grid_for(kern, kBlock, v.o_tiles * kBlock, v.blocks_per_sm), kBlock, 0, s>>>(v, round);
+  }
+  // one candidate-list segment per warp of the gather (and of the direct probe)
+  unsigned grid = std::min(grid_for(ord_gather_kernel, kBlock, v.o_tiles * kBlock, v.blocks_per_sm),
+                           grid_for(list_probe_kernel<KW, HB>, kBlock, v.o_tiles * kBlock, v.blocks_per_sm));
+  grid = std::min(grid, (unsigned)(kMaxSegments / (kBlock / 32)));
+  pv->n_segments = grid * (kBlock / 32);
+  pv->seg_cap = (v.narrow ? 2 * v.cand_cap : v.cand_cap) / pv->n_segments;
+  if (fused && cudaMemsetAsync(v.table, 0xFF, (uint64_t)v.o_tcap * v.o_regions * 8, s) != cudaSuccess)
+    return -1;  // every fused table slot empty (all ones)
+  {
+    Timed t("ord_probe", s);
+    auto kern = fused ? ord_probe_kernel<HB, true> : ord_probe_kernel<HB, false>;
+    kern<<<grid_for(kern, kBlock, ~0ull >> 1), kBlock, 0, s>>>(v);
+  }
+  if (fused) {
+    Timed t("ord_classify", s);
+    ord_classify_kernel<<<grid_for(ord_classify_kernel, kBlock, ~0ull >> 1), kBlock, 0, s>>>(v);
+  }
+  {
+    Timed t("ord_gather", s);
+    ord_gather_kernel<<<grid, kBlock, 0, s>>>(*pv, round);
+  }
+  {
+    Timed t("list_probe", s);
+    list_probe_kernel<KW, HB><<<grid, kBlock, 0, s>>>(*pv, round);
+  }
+  return fused ? 11 : 10;
+}
+
 template <int KW, bool RD, int HB, int TS>
 static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges* ranges) {
   // the pack kernel cleared the filter and the LC bitmap for round 0; the
@@ -3415,8 +3490,10 @@ static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges*
   if (RD && cudaMemsetAsync(v.filter, 0, v.filter_words64 * 8, s) != cudaSuccess) return -1;
   if (round > 0 && cudaMemsetAsync(v.lc_bits, 0, (1ull << v.lc_log2) / 8, s) != cudaSuccess) return -1;
   constexpr bool kDescOk = HB <= 6;
-  const bool cm = RD && v.cmap != nullptr;  // rounds visit only their class's positions
-  const bool desc = !cm && kDescOk && v.use_desc;
+  constexpr bool kOrdOk = HB >= 1 && HB <= 6 && KW <= 2;  // a record carries the bit bases of up to 6 bits per item
+  const bool ord = kOrdOk && v.o_regions > 0;  // region-ordered first pass, over the sorted tiles
+  const bool cm = RD && v.cmap != nullptr;     // rounds visit only their class's positions
+  const bool desc = !cm && !ord && kDescOk && v.use_desc;
   // every loop over all positions at once, or once per string (ranges)
   const Ranges whole{{v.p_begin, v.p_end}};
   const Ranges& rs = ranges ? *ranges : whole;
@@ -3427,39 +3504,19 @@ static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges*
     return x;
   };
   int launched = 0;
-  // filters beyond L2: the region-ordered first pass (class-map rounds), or
+  RunView pv = v;
   // region buckets for the inserts alone, chunk by chunk
   constexpr bool kBktOk = HB <= 6;  // a record carries the bit bases of up to 6 bits per item
   constexpr int HBO = kBktOk ? HB : 1;
   const bool bkt = kBktOk && v.n_regions > 0;
-  const bool ord = kBktOk && cm && v.o_regions > 0 && !ranges;
-  const bool fused = ord && v.o_fused;
-  if (ord) {
-    {
-      Timed t("ord_scatter", s);
-      const uint64_t chunks = (v.o_tiles + kOrdScanTiles - 1) / kOrdScanTiles;
-      ord_room_sum_kernel<<<(unsigned)chunks, kBlock, 0, s>>>(v, round);
-      ord_room_prefix_kernel<<<v.o_regions, kBlock, 0, s>>>(v, chunks);
-      ord_room_scan_kernel<<<(unsigned)chunks, kBlock, 0, s>>>(v, round);
-      ord_setup_kernel<<<1, kBlock, 0, s>>>(v, round);
-      const uint64_t tiles = (v.p_end - v.p_begin + kOrdTile - 1) / kOrdTile;
-      auto kern = ord_scatter_kernel<KW, HBO, false>;
-      if constexpr (KW == 1)
-        if (fused) kern = ord_scatter_kernel<KW, HBO, true>;
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOrdStageBytes) !=
-          cudaSuccess)
-        return -1;
-      kern<<<grid_for(kern, kBlock, tiles * kBlock, v.blocks_per_sm, kOrdStageBytes), kBlock, kOrdStageBytes, s>>>(
-          v, round);
+  if constexpr (kOrdOk) {
+    if (ord) {
+      const int n = ordered_round_impl<KW, HB>(v, round, s, &pv);
+      if (n < 0) return -1;
+      launched += n;
     }
-    {
-      Timed t("ord_or", s);
-      auto kern = fused ? ord_or_kernel<HBO, true> : ord_or_kernel<HBO, false>;
-      kern<<<grid_for(kern, kBlock, ~0ull >> 1), kBlock, 0, s>>>(v);
-    }
-    launched += 6;
   }
-  {
+  if (!ord) {
     for (const auto& r : rs) {
       const uint64_t step = bkt ? v.bucket_chunk : r.second - r.first;
       for (uint64_t c0 = r.first; c0 < r.second; c0 += step) {
@@ -3500,8 +3557,8 @@ static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges*
       }
     }
   }
-  RunView pv = v;
   for (const auto& r : rs) {
+    if (ord) break;  // its segments are laid out
     pv = part(r);
     const uint64_t threads = (r.second - r.first + kProbeR - 1) / kProbeR;
     // one candidate-list segment per probe warp
@@ -3513,25 +3570,6 @@ static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges*
     // the list region holds cand_cap 8-byte records, or twice as many 32-bit
     // ones; launched per string there is no list (pass 2 walks C_temp)
     pv.seg_cap = ranges ? 0 : (v.narrow ? 2 * v.cand_cap : v.cand_cap) / pv.n_segments;
-    if (ord) {  // the gather's warps own the list segments, as the probe's would
-      if (fused && cudaMemsetAsync(v.table, 0xFF, (uint64_t)v.o_tcap * v.o_regions * 8, s) != cudaSuccess)
-        return -1;  // every fused table slot empty (all ones)
-      {
-        Timed t("ord_probe", s);
-        auto kern = fused ? ord_probe_kernel<HBO, true> : ord_probe_kernel<HBO, false>;
-        kern<<<grid_for(kern, kBlock, ~0ull >> 1), kBlock, 0, s>>>(v);
-      }
-      if (fused) {
-        Timed t("ord_classify", s);
-        ord_classify_kernel<<<grid_for(ord_classify_kernel, kBlock, ~0ull >> 1), kBlock, 0, s>>>(v);
-        ++launched;
-      }
-      {
-        Timed t("ord_gather", s);
-        ord_gather_kernel<<<grid, kBlock, 0, s>>>(pv, round);
-      }
-      launched += 2;
-    }
     Timed t("pass1_probe", s);
     if (cm) pass1_probe_cm_kernel<KW, HB><<<grid, kBlock, 0, s>>>(pv, round);
     else if (desc) pass1_probe_desc_kernel<kDescOk ? HB : 1><<<grid, kBlock, 0, s>>>(pv, round);
@@ -3616,14 +3654,12 @@ int TWOPACO_PART_NAME(launch_count_, TWOPACO_PART)(const RunView& v, cudaStream_
 int TWOPACO_PART_NAME(launch_map_, TWOPACO_PART)(const RunView& v, cudaStream_t s) {
   Timed t("class_map", s);
   if constexpr (kPartKw < 4) {
-    if (v.o_regions) {
-      auto kern = class_map_ord_kernel<kPartKw>;
-      kern<<<grid_for(kern, kBlock, v.o_tiles * kBlock), kBlock, 0, s>>>(v);
-      // every tile's first member number, per round
-      const uint64_t chunks = (v.o_tiles + kOrdScanTiles - 1) / kOrdScanTiles;
-      ord_tile_sum_kernel<<<(unsigned)(chunks * v.rounds), kBlock, 0, s>>>(v, chunks);
-      ord_tile_scan_kernel<<<(unsigned)(chunks * v.rounds), kBlock, 0, s>>>(v, chunks);
-      return done(3);
+    if (v.o_regions) {  // the sorted tiles instead
+      auto kern = class_sort_kernel<kPartKw>;
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSortBytes) != cudaSuccess)
+        return -1;
+      kern<<<grid_for(kern, kSortBlock, v.o_tiles * kSortBlock, 0, kSortBytes), kSortBlock, kSortBytes, s>>>(v);
+      return done(1);
     }
   }
   auto kern = class_map_kernel<kPartKw>;
@@ -3675,7 +3711,7 @@ int launch_partition(const RunView& v, int rounds, cudaStream_t s) {
 }
 
 int launch_class_map(const RunView& v, cudaStream_t s) {
-  if (!v.cmap || v.m == 0) return 0;
+  if ((!v.cmap && !v.o_regions) || v.m == 0) return 0;
   return v.k <= 31 ? launch_map_1(v, s) : (v.k <= 63 ? launch_map_3(v, s) : launch_map_5(v, s));
 }
 
