@@ -81,7 +81,7 @@ struct Layout {
   uint32_t o_tcap;     // fused: table slots per region
   int o_lg_region_words;
   uint64_t o_rec_cap, o_tiles;
-  uint64_t olist, ofirst, othist, ocsum, ocpre, obtot, ostart, ofill, orecs, odec, ometa;
+  uint64_t olist, otoff, ocsum, ocpre, obtot, ostart, ofill, orecs, odec, ometa;
   uint64_t bucket_cap, bucket_chunk;
   uint64_t n_chunks, run_cap;
   uint64_t total;
@@ -241,16 +241,14 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
   if (L.n_regions) at += align_up(((uint64_t)L.n_regions * L.n_sub + 1) * 128);
   L.brecs = at;
   if (L.n_regions) at += align_up(L.bucket_cap * L.n_regions * L.n_sub * 8);
-  L.olist = L.ofirst = L.othist = L.ocsum = L.ocpre = L.obtot = L.ostart = L.ofill = L.orecs = L.odec = L.ometa = at;
+  L.olist = L.otoff = L.ocsum = L.ocpre = L.obtot = L.ostart = L.ofill = L.orecs = L.odec = L.ometa = at;
   if (L.o_regions) {
     const uint64_t R = L.o_regions;
     L.olist = at;
     at += align_up(L.o_tiles * kOrdTile * 2);
-    L.ofirst = at;
-    at += align_up(L.o_tiles * ((uint64_t)rounds + 1) * 2);
+    L.otoff = at;
+    at += align_up(L.o_tiles * (rounds * R + 1) * 2);
     const uint64_t chunks = (L.o_tiles + kOrdScanTiles - 1) / kOrdScanTiles;
-    L.othist = at;
-    at += align_up(L.o_tiles * rounds * R * 2);
     L.ocsum = at;
     at += align_up(chunks * R * 4);
     L.ocpre = at;
@@ -372,8 +370,7 @@ RunView make_view(const uint8_t* d_bases, const uint64_t* d_offsets, uint64_t n_
   if (L.o_regions) {
     v.o_lg_region_words = L.o_lg_region_words;
     v.o_list = reinterpret_cast<uint16_t*>(base + L.olist);
-    v.o_first = reinterpret_cast<uint16_t*>(base + L.ofirst);
-    v.o_thist = reinterpret_cast<uint16_t*>(base + L.othist);
+    v.o_toff = reinterpret_cast<uint16_t*>(base + L.otoff);
     v.o_csum = reinterpret_cast<uint32_t*>(base + L.ocsum);
     v.o_cpre = reinterpret_cast<unsigned long long*>(base + L.ocpre);
     v.o_btot = reinterpret_cast<unsigned long long*>(base + L.obtot);

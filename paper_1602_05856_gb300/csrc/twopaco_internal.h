@@ -123,8 +123,7 @@ struct RunView {
   uint32_t o_regions;       // filter regions (buckets), at most kOrdMaxRegions
   int o_lg_region_words;    // log2 of the 64-bit words per region (at most 22)
   uint16_t* o_list;         // every tile's positions sorted by class and region (kOrdTile per tile)
-  uint16_t* o_first;        // per tile: the first list entry of every class, then the end (rounds + 1)
-  uint16_t* o_thist;        // per tile, class and region: its positions (tile-major)
+  uint16_t* o_toff;         // per tile: the first list entry of every (class, region), then the end
   uint32_t* o_csum;         // per chunk of kOrdScanTiles tiles and bucket: the round's members
   unsigned long long* o_cpre;  // per chunk and bucket: the round's members in the chunks before
   unsigned long long* o_btot;  // per bucket: the round's members

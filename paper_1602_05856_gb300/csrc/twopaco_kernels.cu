@@ -429,13 +429,56 @@ __device__ __forceinline__ int32_t rel(uint64_t x, uint64_t p0) {
 
 // The occurrence of a listed candidate: its string bounds are not needed,
 // because the list marks candidates at a string end (sentinel positions)
-// and every other candidate has a predecessor and a successor.
+// and every other candidate has a predecessor and a successor. Those are read
+// from one window with the k-mer, which starts at the predecessor: 2 KW + 1
+// aligned words hold any 16 (2 KW) + 1 bases (k = 63 and four-word k-mers read
+// their successor apart).
 template <int KW>
 __device__ __forceinline__ void read_listed(const RunView& v, uint64_t g, bool sentinel, OccT<KW>* oc) {
-  const KeyT<KW> f = load_kmer<KW>(v.packed, g, v.k);
-  const KeyT<KW> r = v.both ? revcomp<KW>(f, v.k) : f;
-  const uint32_t pred = sentinel ? 0u : base_at(v.packed, g - 1);
-  const uint32_t succ = sentinel ? 0u : base_at(v.packed, g + v.k);
+  const int k = v.k;
+  KeyT<KW> f;
+  uint32_t pred = 0, succ = 0;
+  if (sentinel || KW == 4) {
+    f = load_kmer<KW>(v.packed, g, k);
+    if (!sentinel) {
+      pred = base_at(v.packed, g - 1);
+      succ = base_at(v.packed, g + k);
+    }
+  } else {
+    constexpr int W = 2 * KW;
+    const uint32_t* p = v.packed + ((g - 1) >> 4);
+    const uint32_t o2 = 2u * (uint32_t)((g - 1) & 15);
+    uint32_t w[W + 1], x[W + 1];
+#pragma unroll
+    for (int j = 0; j <= W; ++j) w[j] = __ldg(p + j);
+#pragma unroll
+    for (int j = 0; j <= W; ++j) x[j] = __funnelshift_l(j < W ? w[j + 1] : 0u, w[j], o2);  // from g - 1 on
+    pred = x[0] >> 30;
+    // base k + 1 of the window
+    const int sw = (k + 1) >> 4, ss = 30 - 2 * ((k + 1) & 15);
+    if (KW == 2 && k == 63) {
+      succ = base_at(v.packed, g + k);
+    } else {
+      uint32_t y = x[W];
+#pragma unroll
+      for (int j = 0; j < W; ++j)
+        if (j == sw) y = x[j];
+      succ = (y >> ss) & 3u;
+    }
+    uint64_t top[KW];  // the 32 KW bases from g on
+#pragma unroll
+    for (int j = 0; j < KW; ++j)
+      top[j] = ((uint64_t)__funnelshift_l(x[2 * j + 1], x[2 * j], 2) << 32) | __funnelshift_l(x[2 * j + 2], x[2 * j + 1], 2);
+    if constexpr (KW == 1) {
+      f.hi = 0;
+      f.lo = top[0] >> (64 - 2 * k);
+    } else if constexpr (KW == 2) {
+      const int sh = 128 - 2 * k;  // 2 .. 64
+      f.hi = sh == 64 ? 0ull : top[0] >> sh;
+      f.lo = sh == 64 ? top[0] : (top[1] >> sh) | (top[0] << (64 - sh));
+    }
+  }
+  const KeyT<KW> r = v.both ? revcomp<KW>(f, k) : f;
   make_occ<KW>(v, f, r, pred, succ, sentinel, oc);
 }
 
@@ -1715,8 +1758,8 @@ __global__ void __launch_bounds__(kBlock) class_map_kernel(RunView v) {
 // class map: every tile of kOrdTile positions lists the positions that have a
 // k-mer, sorted by (class, filter region) -- 16 bits each, bits 0-13 the
 // position within the tile, kOrdEntrySentinel for the first or last k-mer of a
-// string -- with the count of every (class, region) pair (o_thist) and the first
-// entry of every class (o_first). A round then reads exactly its members, in
+// string -- with the first entry of every (class, region) pair and the end
+// (o_toff). A round then reads exactly its members, in
 // the order of the buckets their records go to: the scatter needs no
 // compaction, no rank per member and no staging to write whole runs, and the
 // gather reads the decisions of a run as consecutive bits. (With a class byte
@@ -1771,18 +1814,13 @@ __global__ void __launch_bounds__(kSortBlock, 2) class_sort_kernel(RunView v) {
       });
     }
     __syncthreads();
-    // exclusive scan of the counts (nh <= 4096: at most 8 per thread), which go out first
+    // exclusive scan of the counts (nh <= 4096: at most 8 per thread)
     uint32_t total;
     {
       const uint32_t per = (nh + kSortBlock - 1) / kSortBlock;
       const uint32_t i0 = min(nh, threadIdx.x * per), i1 = min(nh, i0 + per);
-      uint16_t* th = v.o_thist + t * nh;
       uint32_t sum = 0;
-      for (uint32_t i = i0; i < i1; ++i) {
-        const uint32_t c = hist[i];
-        th[i] = (uint16_t)c;  // at most kOrdTile = 16384
-        sum += c;
-      }
+      for (uint32_t i = i0; i < i1; ++i) sum += hist[i];
       uint32_t inc = sum;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -1799,14 +1837,14 @@ __global__ void __launch_bounds__(kSortBlock, 2) class_sort_kernel(RunView v) {
         total += warp_s[w];
       }
       uint32_t at = before + inc - sum;
-      uint16_t* first = v.o_first + t * (L + 1);
+      uint16_t* toff = v.o_toff + t * (nh + 1);
       for (uint32_t i = i0; i < i1; ++i) {
         const uint32_t c = hist[i];
         hist[i] = at;
-        if (i % R == 0) first[i / R] = (uint16_t)at;
+        toff[i] = (uint16_t)at;  // at most kOrdTile = 16384
         at += c;
       }
-      if (threadIdx.x == 0) first[L] = (uint16_t)total;
+      if (threadIdx.x == 0) toff[nh] = (uint16_t)total;
     }
     __syncthreads();
     for (int e0 = threadIdx.x; e0 < (int)kOrdTile; e0 += kSortBlock) {
@@ -2115,11 +2153,14 @@ template <typename F>
 __device__ __forceinline__ void for_tile_counts(const RunView& v, int round, F&& fn) {
   const uint32_t R = v.o_regions, nh = (uint32_t)v.rounds * R;
   const uint64_t t0 = (uint64_t)blockIdx.x * kOrdScanTiles, t1 = min(t0 + kOrdScanTiles, v.o_tiles);
-  const uint16_t* th = v.o_thist + (uint64_t)round * R + threadIdx.x;
+  const uint16_t* at = v.o_toff + (uint64_t)round * R + threadIdx.x;
   for (uint64_t t = t0; t < t1; t += kRoomAhead) {
     uint32_t c[kRoomAhead];
 #pragma unroll
-    for (int u = 0; u < kRoomAhead; ++u) c[u] = t + u < t1 ? __ldg(th + (t + u) * nh) : 0u;
+    for (int u = 0; u < kRoomAhead; ++u) {
+      const uint16_t* q = at + (t + u) * (nh + 1);
+      c[u] = t + u < t1 ? (uint32_t)__ldg(q + 1) - __ldg(q) : 0u;
+    }
 #pragma unroll
     for (int u = 0; u < kRoomAhead; ++u)
       if (t + u < t1) fn(t + u, c[u]);
@@ -2197,15 +2238,15 @@ struct TileMembers {
 // members' buckets are filled in by R / kBlock-th of the threads each, run by run.
 __device__ __forceinline__ TileMembers ord_tile(const RunView& v, uint64_t t, int round, const uint64_t* start_s,
                                                 unsigned long long* delta_s, uint32_t* run_s, uint8_t* bucket_s) {
-  const uint32_t R = v.o_regions, L = (uint32_t)v.rounds, b = threadIdx.x;
-  const uint32_t count = b < R ? v.o_thist[(t * L + round) * R + b] : 0u;
-  const uint32_t room = b < R ? __ldg(v.o_meta + t * R + b) : 0u;
+  const uint32_t R = v.o_regions, b = threadIdx.x;
+  const uint16_t* toff = v.o_toff + t * ((uint64_t)v.rounds * R + 1) + (uint64_t)round * R;
+  const uint32_t first = toff[0];
   TileMembers tm;
-  const uint16_t* first = v.o_first + t * (L + 1);
-  tm.list = v.o_list + t * kOrdTile + first[round];
-  const uint32_t off = block_exclusive_scan(count, &tm.n);
+  tm.list = v.o_list + t * kOrdTile + first;
+  tm.n = toff[R] - first;
   if (b < R) {
-    delta_s[b] = start_s[b] + room - off;
+    const uint32_t off = toff[b] - first, count = toff[b + 1] - toff[b];
+    delta_s[b] = start_s[b] + __ldg(v.o_meta + t * R + b) - off;
     run_s[b] = off | (count << 16);  // both at most kOrdTile = 2^14
   }
   __syncthreads();
@@ -2541,9 +2582,10 @@ __device__ __forceinline__ void ord_counts_out(const RunView& v, bool fused, con
   if (fused) block_add(o.junctions, &v.hdr->pass2_kept);
 }
 
-// k-mer positions of a tile: the end of its last class.
+// k-mer positions of a tile: the end of its list.
 __device__ __forceinline__ uint32_t ord_tile_positions(const RunView& v, uint64_t t) {
-  return v.o_first[t * ((uint32_t)v.rounds + 1u) + (uint32_t)v.rounds];
+  const uint64_t nh = (uint64_t)v.rounds * v.o_regions;
+  return v.o_toff[t * (nh + 1) + nh];
 }
 
 // The probe loop's outputs in position order: every member of the round's
@@ -2603,8 +2645,8 @@ template <int KW, int HB>
 __global__ void __launch_bounds__(kBlock) list_insert_kernel(RunView v, int round) {
   if (ordered_round(v)) return;  // the region-ordered kernels took this round
   for (uint64_t t = blockIdx.x; t < v.o_tiles; t += gridDim.x) {
-    const uint16_t* first = v.o_first + t * ((uint32_t)v.rounds + 1u);
-    const uint32_t a = first[round], b = first[round + 1];
+    const uint16_t* toff = v.o_toff + t * ((uint64_t)v.rounds * v.o_regions + 1) + (uint64_t)round * v.o_regions;
+    const uint32_t a = toff[0], b = toff[v.o_regions];
     for (uint32_t i = a + threadIdx.x; i < b; i += kBlock) {
       const uint32_t e = v.o_list[t * kOrdTile + i];
       OccT<KW> oc;
@@ -2627,8 +2669,8 @@ __global__ void __launch_bounds__(kBlock) list_probe_kernel(RunView v, int round
   TileOut o{0, 0, 0};
   unsigned long long valid_n = 0;
   for (uint64_t t = blockIdx.x; t < v.o_tiles; t += gridDim.x) {
-    const uint16_t* first = v.o_first + t * ((uint32_t)v.rounds + 1u);
-    const uint32_t a = first[round], b = first[round + 1];
+    const uint16_t* toff = v.o_toff + t * ((uint64_t)v.rounds * v.o_regions + 1) + (uint64_t)round * v.o_regions;
+    const uint32_t a = toff[0], b = toff[v.o_regions];
     if (threadIdx.x == 0) valid_n += ord_tile_positions(v, t);
     for (uint32_t i = a + threadIdx.x; i < b; i += kBlock) {
       const uint32_t e = v.o_list[t * kOrdTile + i], pos = e & kOrdEntryPos;
