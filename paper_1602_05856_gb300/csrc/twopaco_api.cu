@@ -147,10 +147,14 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
   const uint64_t per_chunk = std::min<uint64_t>(per_round, 1ull << 31) * 4 / 5;
   const bool want_bkt =
       o.bucket_inserts == 1 || (o.bucket_inserts == 0 && beyond_l2 && per_chunk >= 16 * (filter_bits / 256));
+  // the ordered passes from 4 ORs per sector on: they read every region once and
+  // write it back, however few records it takes
+  const bool dense = beyond_l2 && per_round >= 4 * (filter_bits / 256);
   // region-ordered first pass: k <= 63, h <= 6, one launch per loop, at most
   // kOrdMaxRegions regions of at most 2^22 words and at most kOrdMaxHist
-  // (round, region) counters; rounds automatically for filters of 1 GiB and more,
-  // and in one round wherever bucketed inserts are wanted
+  // (round, region) counters; automatically for filters beyond L2 that a round
+  // fills densely, and in several rounds for filters of 1 GiB and more; in one
+  // round instead of bucketed inserts
   L.o_regions = 0;
   {
     const uint64_t fwords = filter_bits / 64;
@@ -163,9 +167,10 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
     while (R > r_min && R * (uint64_t)rounds > kOrdMaxHist) R /= 2;
     while (R > r_min && k <= 27 && !o.partial && L.table_slots / R < 1024) R /= 2;
     const uint64_t rw = fwords / R;
-    const bool auto_rounds = filter_bits / 8 >= (1ull << 30);
+    const bool auto_rounds = filter_bits / 8 >= (1ull << 30) || dense;
     const bool want = rounds > 1 ? o.ordered_first_pass == 1 || (o.ordered_first_pass == 0 && auto_rounds)
-                                 : want_bkt && o.ordered_first_pass != 2;
+                                 : o.ordered_first_pass != 2 &&
+                                       (o.bucket_inserts == 1 || (o.bucket_inserts == 0 && dense));
     if (want && rounds <= kMaxMapRounds && k <= 63 && o.hashes <= 6 && !o.per_string_launches &&
         m > 0 && R <= kOrdMaxRegions && R * (uint64_t)rounds <= kOrdMaxHist) {
       L.o_regions = (uint32_t)R;
@@ -263,7 +268,7 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
     L.cands = at;
     at += align_up(std::max<uint64_t>(L.o_rec_cap * 8, L.cand_cap * cand_record_bytes(k)));
     L.odec = at;
-    at += align_up((L.o_rec_cap + 31) / 32 * 4 * (L.o_fused ? 2 : 1));
+    at += align_up((L.o_rec_cap + 31) / 32 * 4 * (o.partial ? 1 : 2));
     L.ometa = at;
     at += align_up(L.o_tiles * R * 4);
   }
@@ -382,6 +387,9 @@ RunView make_view(const uint8_t* d_bases, const uint64_t* d_offsets, uint64_t n_
     v.o_meta = reinterpret_cast<uint32_t*>(base + L.ometa);
     v.o_tiles = L.o_tiles;
     v.o_fused = L.o_fused;
+    v.o_bucketed = k >= 28 && !o.partial;
+    // about 4096 members per work item
+    v.o_item_tiles = (uint32_t)std::max<uint64_t>(8, (uint64_t)L.o_regions * rounds / (kOrdTile / 4096));
     v.o_tcap = L.o_tcap;
   }
   v.tile_count = reinterpret_cast<uint32_t*>(base + L.tile_count);

@@ -19,7 +19,7 @@ struct DevHeader {
   unsigned long long round_kept;   // candidates after pass 1, current round
   unsigned long long table_slots;  // pass-2 table capacity of the current round
   unsigned long long table_max;    // largest capacity used by any round
-  unsigned long long reserved2;
+  unsigned long long part_slots;   // region-ordered pass 2 by buckets: table slots per region (0: not this round)
   unsigned int cand_overflow;      // a warp's list segment ran out of room this round
   unsigned int round_listed;       // pass 2 of this round reads the list (else C_temp)
   unsigned int reserved;
@@ -57,7 +57,7 @@ struct DevHeader {
   unsigned long long input_digest;  // written by launch_digest
   unsigned int out_overflow;        // the output positions did not fit (the offsets are exact)
   unsigned int ord_ok;              // region-ordered first pass: this round's records fit
-  unsigned int ord_ticket[3];       // region-ordered first pass: apply, probe and classify work items
+  unsigned int ord_ticket[4];       // region-ordered passes: apply, probe, classify and insert work items
   unsigned int ord_rounds;          // rounds the region-ordered kernels took
 };
 
@@ -131,10 +131,12 @@ struct RunView {
   uint32_t* o_fill;         // records claimed per bucket, one counter per 128 bytes
   uint64_t* o_recs;         // o_rec_cap records
   uint64_t o_rec_cap;
-  uint32_t* o_dec;          // one decision bit per record slot; fused: word pairs (candidates,
-                            // junctions) per 32 slots
+  uint32_t* o_dec;          // decision bits per 32 record slots: word pairs (candidates, junctions),
+                            // partial: one word
   uint32_t* o_meta;         // per tile and bucket: where the tile's records start in the bucket
   uint64_t o_tiles;         // tiles of kOrdTile positions: ceil(m / kOrdTile)
+  int o_bucketed;           // 28 <= k <= 63, not partial: pass 2 bucket by bucket, through the lists
+  uint32_t o_item_tiles;    // tiles per work item of its insert loop
   int o_fused;              // k <= 27, not partial: pass 2 runs on the records (fused records)
   uint32_t o_tcap;          // fused: table slots per bucket (region), the table is o_regions x o_tcap slots
   int use_desc;             // the insert leaves descriptors and the probe reads them

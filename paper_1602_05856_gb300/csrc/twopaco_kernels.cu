@@ -2149,29 +2149,32 @@ __device__ __forceinline__ unsigned long long block_exclusive_scan64(unsigned lo
 constexpr int kRoomAhead = 8;
 static_assert(kOrdScanTiles % kRoomAhead == 0, "whole groups of tiles");
 
+// (Called by the whole block; fn runs for the threads of a bucket, b < R.)
 template <typename F>
 __device__ __forceinline__ void for_tile_counts(const RunView& v, int round, F&& fn) {
-  const uint32_t R = v.o_regions, nh = (uint32_t)v.rounds * R;
+  const uint32_t R = v.o_regions, nh = (uint32_t)v.rounds * R, b = threadIdx.x;
   const uint64_t t0 = (uint64_t)blockIdx.x * kOrdScanTiles, t1 = min(t0 + kOrdScanTiles, v.o_tiles);
-  const uint16_t* at = v.o_toff + (uint64_t)round * R + threadIdx.x;
+  const uint16_t* at = v.o_toff + (uint64_t)round * R + b;
   for (uint64_t t = t0; t < t1; t += kRoomAhead) {
     uint32_t c[kRoomAhead];
 #pragma unroll
     for (int u = 0; u < kRoomAhead; ++u) {
       const uint16_t* q = at + (t + u) * (nh + 1);
-      c[u] = t + u < t1 ? (uint32_t)__ldg(q + 1) - __ldg(q) : 0u;
+      c[u] = (t + u < t1 && b <= R) ? __ldg(q) : 0u;
     }
 #pragma unroll
-    for (int u = 0; u < kRoomAhead; ++u)
-      if (t + u < t1) fn(t + u, c[u]);
+    for (int u = 0; u < kRoomAhead; ++u) {  // a run ends where the next lane's starts
+      uint32_t end = __shfl_down_sync(0xffffffffu, c[u], 1);
+      if ((b & 31) == 31 && t + u < t1 && b < R) end = __ldg(at + (t + u) * (nh + 1) + 1);
+      if (t + u < t1 && b < R) fn(t + u, end - c[u]);
+    }
   }
 }
 
 __global__ void __launch_bounds__(kBlock) ord_room_sum_kernel(RunView v, int round) {
-  if (threadIdx.x >= v.o_regions) return;
   uint32_t s = 0;
   for_tile_counts(v, round, [&](uint64_t, uint32_t c) { s += c; });
-  v.o_csum[(uint64_t)blockIdx.x * v.o_regions + threadIdx.x] = s;
+  if (threadIdx.x < v.o_regions) v.o_csum[(uint64_t)blockIdx.x * v.o_regions + threadIdx.x] = s;
 }
 
 __global__ void __launch_bounds__(kBlock) ord_room_prefix_kernel(RunView v, uint64_t chunks) {
@@ -2194,8 +2197,7 @@ __global__ void __launch_bounds__(kBlock) ord_room_prefix_kernel(RunView v, uint
 
 __global__ void __launch_bounds__(kBlock) ord_room_scan_kernel(RunView v, int round) {
   const uint32_t R = v.o_regions;
-  if (threadIdx.x >= R) return;
-  unsigned long long run = v.o_cpre[(uint64_t)blockIdx.x * R + threadIdx.x];
+  unsigned long long run = threadIdx.x < R ? v.o_cpre[(uint64_t)blockIdx.x * R + threadIdx.x] : 0ull;
   for_tile_counts(v, round, [&](uint64_t t, uint32_t c) {
     v.o_meta[t * R + threadIdx.x] = (uint32_t)run;  // within a bucket below 2^32 (the setup checks)
     run += c;
@@ -2223,6 +2225,9 @@ __global__ void __launch_bounds__(kBlock) ord_setup_kernel(RunView v, int round)
     v.hdr->ord_ticket[0] = 0;
     v.hdr->ord_ticket[1] = 0;
     v.hdr->ord_ticket[2] = 0;
+    v.hdr->ord_ticket[3] = 0;
+    v.hdr->part_slots = 0;
+    v.hdr->cand_overflow = 0;  // the gather of the round before may have set it after its table_setup
   }
 }
 
@@ -2399,6 +2404,7 @@ __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
   ord_items(v, first_s);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint32_t R = v.o_regions, total = first_s[R];
+  uint32_t kept = 0;
   for (;;) {
     if (threadIdx.x == 0) item_s = atomicAdd(&v.hdr->ord_ticket[1], 1u);
     __syncthreads();
@@ -2455,11 +2461,15 @@ __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
           }
         }
         const uint32_t row = __ballot_sync(0xffffffffu, keep);
-        // fused: word pairs, the candidates' bits then the junctions' (ord_classify)
-        if (lane == 0) v.o_dec[((start + c) >> 5) << (FUSED ? 1 : 0)] = row;
+        // word pairs, the candidates' bits then the junctions' (partial: no junctions)
+        if (lane == 0) {
+          v.o_dec[((start + c) >> 5) << (v.partial ? 0 : 1)] = row;
+          kept += __popc(row);
+        }
       }
     }
   }
+  if (!FUSED && !v.partial) block_add((unsigned long long)kept, &v.hdr->round_kept);  // sizes the table
 }
 
 // Algorithm 1, probe loop, second pass, on fused records, bucket by bucket:
@@ -2517,9 +2527,145 @@ __global__ void __launch_bounds__(kBlock) ord_classify_kernel(RunView v) {
   }
 }
 
+// Pass 2 bucket by bucket for k-mers that no record holds (28 <= k <= 63): the
+// table has one part per filter region (table_setup), and the candidates of a
+// bucket -- found by its records' decision bits, and their positions by the
+// tiles' lists -- are inserted part by part, so that the table's random accesses
+// hit L2. In position order, over a 6 GB table, they ran at DRAM's
+// random-access rate: 15.0 + 5.3 of 31.7 ms for 62 genomes at k = 63.
+// A work item is o_item_tiles tiles of one bucket, taken in bucket order from a
+// ticket; a warp collects the candidates of its tiles' runs and inserts them 32
+// at a time. The slot goes where the candidate's record was (the probe read it
+// last), for the probe loop.
+template <int KW, int TS>
+__global__ void __launch_bounds__(kBlock) ord_insert2_kernel(RunView v, int round) {
+  __shared__ uint32_t item_s;
+  __shared__ uint32_t slot_s[kBlock / 32][64], ent_s[kBlock / 32][64];  // the warp's candidates: record, list entry
+  const uint64_t part = __ldcg(&v.hdr->part_slots);
+  if (!ordered_round(v) || !part) return;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint32_t* slot_q = slot_s[wid];
+  uint32_t* ent_q = ent_s[wid];
+  const uint32_t below = (1u << lane) - 1u;
+  const uint32_t R = v.o_regions, per = v.o_item_tiles;
+  const uint32_t chunks = (uint32_t)((v.o_tiles + per - 1) / per), total = R * chunks;
+  const uint64_t nh = (uint64_t)v.rounds * R;
+  for (;;) {
+    if (threadIdx.x == 0) item_s = atomicAdd(&v.hdr->ord_ticket[3], 1u);
+    __syncthreads();
+    const uint32_t item = item_s;
+    __syncthreads();
+    if (item >= total) break;
+    const uint32_t b = item / chunks;
+    const uint64_t t0 = (uint64_t)(item - b * chunks) * per, t1 = min(t0 + per, v.o_tiles);
+    const uint64_t start = __ldg(v.o_start + b);
+    RunView x = v;
+    x.table = static_cast<char*>(v.table) + (uint64_t)b * part * (32 / SectorOf<TS>::kSlots);
+    auto insert = [&](uint32_t n) {  // the first n candidates of the queue
+      __syncwarp();
+      if ((uint32_t)lane < n) {
+        const uint32_t e = ent_q[lane];
+        const uint64_t g = (t0 + (e >> 16)) * kOrdTile + (e & kOrdEntryPos);
+        OccT<KW> oc;
+        read_listed<KW>(v, g, e & kOrdEntrySentinel, &oc);
+        const uint64_t at = insert_occurrence<KW, TS>(x, part, oc, g);
+        if (at == kNoSlot) v.hdr->overflow = 1;
+        v.o_recs[start + slot_q[lane]] = at;
+      }
+      __syncwarp();
+    };
+    uint32_t n = 0;
+    // the runs of kGroup tiles at a time, one per lane
+    constexpr int kGroup = 8;
+    for (uint64_t tb = t0 + (uint64_t)kGroup * wid; tb < t1; tb += kGroup * (kBlock / 32)) {
+      uint32_t off = 0, cnt = 0, room = 0;
+      if (lane < kGroup && tb + lane < t1) {
+        const uint16_t* q = v.o_toff + (tb + lane) * (nh + 1) + (uint64_t)round * R + b;
+        off = q[0];
+        cnt = q[1] - off;
+        room = __ldg(v.o_meta + (tb + lane) * R + b);
+      }
+      const int tiles = (int)min((uint64_t)kGroup, t1 - tb);
+      for (int i = 0; i < tiles; ++i) {
+        const uint32_t c = __shfl_sync(0xffffffffu, cnt, i), r0 = __shfl_sync(0xffffffffu, room, i);
+        const uint16_t* list = v.o_list + (tb + i) * kOrdTile + __shfl_sync(0xffffffffu, off, i);
+        for (uint32_t j0 = 0; j0 < c; j0 += 32) {
+          const uint32_t j = j0 + lane;
+          const uint64_t s = start + r0 + j;
+          const bool cand = j < c && ((__ldg(v.o_dec + ((s >> 5) << 1)) >> (s & 31)) & 1u);
+          const uint32_t m = __ballot_sync(0xffffffffu, cand);
+          if (cand) {
+            const uint32_t at = n + __popc(m & below);
+            slot_q[at] = r0 + j;
+            ent_q[at] = (uint32_t)(tb + i - t0) << 16 | __ldcs(list + j);
+          }
+          n += __popc(m);
+          if (n >= 32) {
+            insert(32);
+            n -= 32;
+            if ((uint32_t)lane < n) {
+              slot_q[lane] = slot_q[lane + 32];
+              ent_q[lane] = ent_q[lane + 32];
+            }
+            __syncwarp();
+          }
+        }
+      }
+    }
+    insert(n);
+  }
+}
+
+// Its probe loop: a candidate's junction bit from the mask in the slot kept in
+// place of its record (as ord_classify_kernel writes it).
+template <int TS>
+__global__ void __launch_bounds__(kBlock) ord_classify2_kernel(RunView v) {
+  __shared__ uint32_t first_s[kOrdMaxRegions + 1];
+  __shared__ uint32_t item_s;
+  const uint64_t part = __ldcg(&v.hdr->part_slots);
+  if (!ordered_round(v) || !part) return;
+  ord_items(v, first_s);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t R = v.o_regions, total = first_s[R];
+  for (;;) {
+    if (threadIdx.x == 0) item_s = atomicAdd(&v.hdr->ord_ticket[2], 1u);
+    __syncthreads();
+    const uint32_t item = item_s;
+    __syncthreads();
+    if (item >= total) break;
+    const uint32_t b = ord_item_bucket(first_s, R, item);
+    const uint64_t n = __ldcg(v.o_fill + (uint64_t)b * kOrdFillStride);
+    const uint64_t i0 = (uint64_t)(item - first_s[b]) * kOrdPiece, i1 = min(i0 + kOrdPiece, n);
+    const uint64_t start = __ldg(v.o_start + b);  // a multiple of 32, as is i0
+    RunView x = v;
+    x.table = static_cast<char*>(v.table) + (uint64_t)b * part * (32 / SectorOf<TS>::kSlots);
+    constexpr int U = 4;
+    for (uint64_t w0 = i0 + 32 * wid; w0 < i1; w0 += U * kBlock) {
+      uint64_t slot[U];
+      bool cand[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint64_t c = w0 + (uint64_t)u * kBlock;
+        const uint32_t row = c < i1 ? __ldcg(v.o_dec + (((start + c) >> 5) << 1)) : 0u;
+        cand[u] = (row >> lane) & 1u;
+        slot[u] = cand[u] ? __ldcs(v.o_recs + start + c + lane) : kNoSlot;
+      }
+      int mk[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) mk[u] = slot[u] != kNoSlot ? table_mask<TS>(x, slot[u]) : -1;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint64_t c = w0 + (uint64_t)u * kBlock;
+        const uint32_t row = __ballot_sync(0xffffffffu, cand[u] && (mk[u] < 0 || is_junction_mask(mk[u])));
+        if (lane == 0 && c < i1) v.o_dec[(((start + c) >> 5) << 1) + 1] = row;
+      }
+    }
+  }
+}
+
 // What a tile's decisions leave behind, called by the whole block with the
-// tile's candidate, junction (fused) and sentinel bits in shared memory: the
-// tile's words of C_temp, its junctions (fused) or, partial, its candidates in
+// tile's candidate, junction and sentinel bits in shared memory: the tile's
+// words of C_temp, its junctions (decided) or, partial, its candidates in
 // C_final -- a tile has one block and rounds own disjoint positions, so no
 // atomic -- or its candidates in the warp's segment of the pass-2 list, in
 // position order. Clears the bits for the next tile.
@@ -2530,7 +2676,7 @@ struct TileOut {
   uint64_t seg_used;
 };
 
-__device__ __forceinline__ void ord_tile_out(const RunView& v, uint64_t t, bool fused, uint32_t* keep_s, uint32_t* jun_s,
+__device__ __forceinline__ void ord_tile_out(const RunView& v, uint64_t t, bool decided, uint32_t* keep_s, uint32_t* jun_s,
                                              uint32_t* sent_s, TileOut* o) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint32_t warp_id = (blockIdx.x * kBlock + threadIdx.x) >> 5;
@@ -2549,7 +2695,7 @@ __device__ __forceinline__ void ord_tile_out(const RunView& v, uint64_t t, bool 
     const uint32_t n = __popc(keep);
     o->kept += n;
     o->junctions += __popc(jun);
-    if (v.partial || fused) continue;
+    if (v.partial || decided) continue;
     uint32_t inc = n;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -2571,15 +2717,15 @@ __device__ __forceinline__ void ord_tile_out(const RunView& v, uint64_t t, bool 
 }
 
 // The counts and the list segment's length after a block's last tile.
-__device__ __forceinline__ void ord_counts_out(const RunView& v, bool fused, const TileOut& o) {
+__device__ __forceinline__ void ord_counts_out(const RunView& v, bool decided, const TileOut& o) {
   const uint32_t warp_id = (blockIdx.x * kBlock + threadIdx.x) >> 5;
   if ((threadIdx.x & 31) == 0) {
     v.seg_count[warp_id] = (uint32_t)(o.seg_used < v.seg_cap ? o.seg_used : v.seg_cap);
     if (o.seg_used > v.seg_cap) v.hdr->cand_overflow = 1;
   }
   block_add(o.kept, &v.hdr->pass1_kept);
-  block_add(o.kept, v.partial ? &v.hdr->pass2_kept : &v.hdr->round_kept);
-  if (fused) block_add(o.junctions, &v.hdr->pass2_kept);
+  if (v.partial) block_add(o.kept, &v.hdr->pass2_kept);
+  if (decided) block_add(o.junctions, &v.hdr->pass2_kept);
 }
 
 // k-mer positions of a tile: the end of its list.
@@ -2601,7 +2747,9 @@ __global__ void __launch_bounds__(kBlock) ord_gather_kernel(RunView v, int round
   if (!ordered_round(v)) return;
   for (uint32_t b = threadIdx.x; b < v.o_regions; b += kBlock) start_s[b] = v.o_start[b];
   for (uint32_t i = threadIdx.x; i < kOrdTileWords; i += kBlock) keep_s[i] = jun_s[i] = sent_s[i] = 0;
-  const bool fused = v.o_fused, listed = !fused && !v.partial;
+  // the junctions are known: pass 2 ran on the records or bucket by bucket
+  const bool decided = v.o_fused || __ldcg(&v.hdr->part_slots) != 0;
+  const bool listed = !decided && !v.partial;
   TileOut o{0, 0, 0};
   unsigned long long valid_n = 0;
   for (uint64_t t = blockIdx.x; t < v.o_tiles; t += gridDim.x) {
@@ -2619,23 +2767,23 @@ __global__ void __launch_bounds__(kBlock) ord_gather_kernel(RunView v, int round
         e[u] = __ldcs(tm.list + i);
         const uint64_t s = delta_s[bucket_s[i]] + i;
         bit[u] = (uint32_t)s & 31u;
-        if (fused) d[u] = __ldg(reinterpret_cast<const uint2*>(v.o_dec) + (s >> 5));  // candidates, junctions
-        else d[u].x = __ldg(v.o_dec + (s >> 5));
+        if (v.partial) d[u].x = __ldg(v.o_dec + (s >> 5));
+        else d[u] = __ldg(reinterpret_cast<const uint2*>(v.o_dec) + (s >> 5));  // candidates, junctions
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (i0 + u * kBlock >= tm.n || !((d[u].x >> bit[u]) & 1u)) continue;  // a junction is a candidate
         const uint32_t pos = e[u] & kOrdEntryPos, m = 1u << (pos & 31u);
         atomicOr(keep_s + (pos >> 5), m);
-        if ((d[u].y >> bit[u]) & 1u) atomicOr(jun_s + (pos >> 5), m);
+        if (decided && ((d[u].y >> bit[u]) & 1u)) atomicOr(jun_s + (pos >> 5), m);
         if (listed && (e[u] & kOrdEntrySentinel)) atomicOr(sent_s + (pos >> 5), m);
       }
     }
     __syncthreads();
-    ord_tile_out(v, t, fused, keep_s, jun_s, sent_s, &o);
+    ord_tile_out(v, t, decided, keep_s, jun_s, sent_s, &o);
     __syncthreads();  // the shared arrays serve the next tile
   }
-  ord_counts_out(v, fused, o);
+  ord_counts_out(v, decided, o);
   if (round == v.count_round) block_add((unsigned long long)valid_n, &v.hdr->positions);
 }
 
@@ -2693,6 +2841,7 @@ __global__ void __launch_bounds__(kBlock) list_probe_kernel(RunView v, int round
     __syncthreads();
   }
   ord_counts_out(v, false, o);
+  if (!v.partial) block_add(o.kept, &v.hdr->round_kept);
   if (round == v.count_round) block_add((unsigned long long)valid_n, &v.hdr->positions);
 }
 
@@ -2702,6 +2851,8 @@ __global__ void __launch_bounds__(kBlock) list_probe_kernel(RunView v, int round
 constexpr double kTableLoadWord = 2.5, kTableLoad = 2.0;
 // pass-2 list work: parts of about this many records, at most kMaxParts per segment
 constexpr unsigned long long kPartRecords = 128, kMaxParts = 4096;
+// pass 2 bucket by bucket: tables of more than this (several times L2)
+constexpr unsigned long long kPartTableBytes = 512ull << 20;
 
 // Size the pass-2 table of this round: 2.5 or 2 times the number of distinct
 // candidate k-mers, as the probe's linear counting estimates it (at least 1024
@@ -2711,6 +2862,7 @@ constexpr unsigned long long kPartRecords = 128, kMaxParts = 4096;
 // detected and reported, never silently wrong. One block: the sampled bitmap is
 // at most 1 MiB, and a grid that counts it and hands the sum to its last block
 // took 10-13 us of every round.
+template <int TS>
 __global__ void __launch_bounds__(1024) table_setup_kernel(RunView v) {
   __shared__ unsigned int part[32];
   DevHeader* h = v.hdr;
@@ -2756,6 +2908,22 @@ __global__ void __launch_bounds__(1024) table_setup_kernel(RunView v) {
       (unsigned long long)((v.k <= 27 ? kTableLoadWord : kTableLoad) * (double)distinct);
   if (cap < 1024ull) cap = 1024ull;
   cap = (cap + 31) / 32 * 32;  // any capacity works (slot_start); whole 32-slot groups
+  if (v.o_bucketed && ordered_round(v)) {
+    // one part per region, of whole sectors: twice the region's share of the
+    // estimate and 64 slots, which is more than eight standard deviations of the
+    // share on top of it; a reserve without room for that keeps one table (and the
+    // candidate list)
+    const unsigned long long part = (cap / v.o_regions + 64 + 3) / 4 * 4;
+    // worth it where the table is far beyond L2 and the candidates are not a small
+    // share of the members, which all have to be looked at: 62 genomes at k = 63 (65%
+    // of 312 M, 6 GB) 21.2 -> 11.5 ms with the gather, but 800 Mbp at k = 31 (12%, 141
+    // MB) 6.3 -> 12.3 ms
+    const bool pays = part * v.o_regions * (32 / SectorOf<TS>::kSlots) > kPartTableBytes && 4 * kept >= v.o_start[v.o_regions];
+    if (pays && part * v.o_regions <= v.table_max_slots) {
+      h->part_slots = part;
+      cap = part * v.o_regions;
+    }
+  }
   if (cap > v.table_max_slots) cap = v.table_max_slots;
   h->table_slots = cap;
   if (cap > h->table_max) h->table_max = cap;
@@ -2824,15 +2992,26 @@ __device__ __forceinline__ void for_rows(const RunView& v, F&& fn) {
 
 constexpr int kClassifyAhead = 2;  // rows of the list in flight per warp
 
+// Pass 2 of this round ran with the region-ordered kernels.
+__device__ __forceinline__ bool pass2_done(const RunView& v) {
+  return ordered_round(v) && (v.o_fused || __ldcg(&v.hdr->part_slots) != 0);
+}
+
+// Pass 2 reads the list: every candidate of the round is in it (a region-ordered
+// round writes its list after table_setup).
+__device__ __forceinline__ bool list_complete(const RunView& v) {
+  return *(volatile unsigned int*)&v.hdr->round_listed && !*(volatile unsigned int*)&v.hdr->cand_overflow;
+}
+
 // Algorithm 1, insert loop, second pass: every candidate ORs its in/out bases
 // (or the sentinel bit) into the exact table entry of its k-mer. Reads the
 // candidate list and keeps the slot of each listed candidate for the probe
 // loop; if the list overflowed, walks C_temp instead.
 template <int KW, int TS>
 __global__ void __launch_bounds__(kBlock) pass2_insert_kernel(RunView v) {
-  if (v.o_fused && ordered_round(v)) return;  // the fused records took this round's pass 2
+  if (pass2_done(v)) return;
   const uint64_t cap = *(volatile unsigned long long*)&v.hdr->table_slots;
-  if (*(volatile unsigned int*)&v.hdr->round_listed) {
+  if (list_complete(v)) {
     const uint32_t lane = threadIdx.x & 31;
     for_rows<1>(v, [&](uint64_t i0, uint32_t, uint32_t left) {
       if (lane >= left) return;
@@ -2862,10 +3041,10 @@ __global__ void __launch_bounds__(kBlock) pass2_insert_kernel(RunView v) {
 // slot the insert loop kept (or looks its k-mer up when no slots were kept).
 template <int KW, int TS>
 __global__ void __launch_bounds__(kBlock) pass2_classify_kernel(RunView v) {
-  if (v.o_fused && ordered_round(v)) return;  // the fused records took this round's pass 2
+  if (pass2_done(v)) return;
   const uint64_t cap = *(volatile unsigned long long*)&v.hdr->table_slots;
   unsigned long long found = 0;
-  if (*(volatile unsigned int*)&v.hdr->round_listed) {
+  if (list_complete(v)) {
     constexpr int U = kClassifyAhead;
     const uint32_t lane = threadIdx.x & 31;
     for_rows<U>(v, [&](uint64_t i0, uint32_t row, uint32_t left) {
@@ -3467,9 +3646,24 @@ static void with_hashes(int h, F&& f) {
   }
 }
 
-// A round's first pass in filter-region order (and, fused, its second pass):
-// launches every kernel of it; *pv gets the list segments. Kernels launched, or -1.
-template <int KW, int HB>
+// The pass-2 table of a round, sized and cleared.
+template <int TS>
+static void launch_table(const RunView& v, cudaStream_t s) {
+  {
+    Timed t("table_setup", s);
+    table_setup_kernel<TS><<<1, 1024, 0, s>>>(v);
+  }
+  {
+    Timed t("table_clear", s);
+    table_clear_kernel<TS><<<grid_for(table_clear_kernel<TS>, kBlock, v.table_max_slots), kBlock, 0, s>>>(v);
+  }
+}
+
+// A round's first pass in filter-region order, and its second on the records or
+// bucket by bucket:
+// launches every kernel of it up to the candidate list's pass 2; *pv gets the
+// list segments. Kernels launched, or -1.
+template <int KW, int HB, int TS>
 static int ordered_round_impl(const RunView& v, int round, cudaStream_t s, RunView* pv) {
   const bool fused = KW == 1 && v.o_fused;
   {
@@ -3515,14 +3709,32 @@ static int ordered_round_impl(const RunView& v, int round, cudaStream_t s, RunVi
     ord_classify_kernel<<<grid_for(ord_classify_kernel, kBlock, ~0ull >> 1), kBlock, 0, s>>>(v);
   }
   {
-    Timed t("ord_gather", s);
-    ord_gather_kernel<<<grid, kBlock, 0, s>>>(*pv, round);
-  }
-  {
     Timed t("list_probe", s);
     list_probe_kernel<KW, HB><<<grid, kBlock, 0, s>>>(*pv, round);
   }
-  return fused ? 11 : 10;
+  int launched = fused ? 10 : 9;
+  if (!v.partial) {
+    launch_table<TS>(*pv, s);
+    launched += 2;
+    if (!fused) {
+      {
+        Timed t("ord_insert2", s);
+        auto kern = ord_insert2_kernel<KW, TS>;
+        kern<<<grid_for(kern, kBlock, ~0ull >> 1), kBlock, 0, s>>>(*pv, round);
+      }
+      {
+        Timed t("ord_classify2", s);
+        auto kern = ord_classify2_kernel<TS>;
+        kern<<<grid_for(kern, kBlock, ~0ull >> 1), kBlock, 0, s>>>(*pv);
+      }
+      launched += 2;
+    }
+  }
+  {
+    Timed t("ord_gather", s);
+    ord_gather_kernel<<<grid, kBlock, 0, s>>>(*pv, round);
+  }
+  return launched + 1;
 }
 
 template <int KW, bool RD, int HB, int TS>
@@ -3553,7 +3765,7 @@ static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges*
   const bool bkt = kBktOk && v.n_regions > 0;
   if constexpr (kOrdOk) {
     if (ord) {
-      const int n = ordered_round_impl<KW, HB>(v, round, s, &pv);
+      const int n = ordered_round_impl<KW, HB, TS>(v, round, s, &pv);
       if (n < 0) return -1;
       launched += n;
     }
@@ -3619,15 +3831,10 @@ static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges*
     ++launched;
   }
   if (v.partial) return done(launched);  // the partially compacted graph: no second pass
-  {
-    Timed t("table_setup", s);
-    table_setup_kernel<<<1, 1024, 0, s>>>(pv);
+  if (!ord) {
+    launch_table<TS>(pv, s);
+    launched += 2;
   }
-  {
-    Timed t("table_clear", s);
-    table_clear_kernel<TS><<<grid_for(table_clear_kernel<TS>, kBlock, v.table_max_slots), kBlock, 0, s>>>(pv);
-  }
-  launched += 2;
   // pass 2: one resident wave; the warps share out the list's segment parts
   const unsigned g2 = grid_for(pass2_insert_kernel<KW, TS>, kBlock, ~0ull >> 1, v.blocks_per_sm);
   const unsigned g3 = grid_for(pass2_classify_kernel<KW, TS>, kBlock, ~0ull >> 1, v.blocks_per_sm);
