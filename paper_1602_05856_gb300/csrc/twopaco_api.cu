@@ -161,11 +161,13 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
     // as many regions as a byte can number, so that a region, the next one (read
     // ahead) and a part of the table are well inside L2, of at most 2^22 words (32
     // MiB) each; fewer where the counters of many rounds, or table parts of at least
-    // 1024 slots (k <= 27), want it
+    // 256 slots (k <= 31), want it
     const uint64_t r_min = std::max<uint64_t>(1, fwords >> kRegionWordsLog2);
     uint64_t R = std::max<uint64_t>(r_min, std::min<uint64_t>(kOrdMaxRegions, fwords));
+    // (k <= 31: regions of whole blocks of four words, so that they are the top bits of H)
+    if (k <= 31 && !o.partial && fwords / 4 >= 64) R = std::min(R, fwords / 4);
     while (R > r_min && R * (uint64_t)rounds > kOrdMaxHist) R /= 2;
-    while (R > r_min && k <= 27 && !o.partial && L.table_slots / R < 1024) R /= 2;
+    while (R > r_min && k <= 31 && !o.partial && L.table_slots / R < 256) R /= 2;
     const uint64_t rw = fwords / R;
     const bool auto_rounds = filter_bits / 8 >= (1ull << 30) || dense;
     const bool want = rounds > 1 ? o.ordered_first_pass == 1 || (o.ordered_first_pass == 0 && auto_rounds)
@@ -181,10 +183,12 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
       // records do not fit takes the direct kernels
       L.o_rec_cap = per_round + per_round / 4 + 32ull * R + 4096;
       L.o_tiles = (m + kOrdTile - 1) / kOrdTile;
-      // pass 2 on the records too (one-word table slots, k <= 27): the table
-      // reserve split into one part per region, at least 1024 slots each
+      // pass 2 on the records too (one-word k-mers, k <= 31, whose hash the bucket and
+      // 58 bits give back): the table reserve split into one part of one-word slots
+      // per region, at least 256 each (half full, more than eight standard deviations
+      // of a part's k-mers fit)
       const uint64_t tcap = L.table_slots / R;
-      if (k <= 27 && !o.partial && tcap >= 1024 && tcap < (1ull << 32)) {
+      if (k <= 31 && !o.partial && R >= 64 && tcap >= 256 && tcap < (1ull << 32)) {
         L.o_fused = 1;
         L.o_tcap = (uint32_t)tcap;
       }
@@ -312,17 +316,17 @@ RunView make_view(const uint8_t* d_bases, const uint64_t* d_offsets, uint64_t n_
   v.lg_blocks = log2_exact(filter_bits / 256);
   v.qmask = o.partition_bins - 1u;
   // The pre-pass needs the proportions of the bins, not their counts: the classes
-  // are runs of bins of a hash, so a sample balances them as well. From 2^27 bases
-  // it walks a 2^-c share of the chunks of 65536 positions (at least 2^26
+  // are runs of bins of a hash, so a sample balances them as well. From 2^25 bases
+  // it walks a 2^-c share of the chunks of 65536 positions (at least 2^24
   // positions, c <= 16), and of what it walks it counts a hash-chosen 2^-s of the
-  // k-mers once that is 2^24 positions and more (at least 2^22 sampled positions,
-  // s <= 8: 64 per bin of the default 65536, a class of ell = 4 to about 0.1%).
+  // k-mers once that is 2^23 positions and more (at least 2^21 sampled positions,
+  // s <= 8: 32 per bin of the default 65536, a class of ell = 4 to about 0.15%).
   // Every counted k-mer is a random atomic in a filter beyond L2: on 200 M bases
   // counting all of them took 4.2 ms of a 13.6 ms build.
   int chunk_log2 = 0, sample_log2 = 0;
-  while (chunk_log2 < 16 && (m >> (chunk_log2 + 1)) >= (1ull << 26)) ++chunk_log2;
-  while (sample_log2 < 8 && ((m >> chunk_log2) >> (sample_log2 + 1)) >= (1ull << 22)) ++sample_log2;
-  if ((m >> chunk_log2) < (1ull << 24)) sample_log2 = 0;
+  while (chunk_log2 < 16 && (m >> (chunk_log2 + 1)) >= (1ull << 24)) ++chunk_log2;
+  while (sample_log2 < 8 && ((m >> chunk_log2) >> (sample_log2 + 1)) >= (1ull << 21)) ++sample_log2;
+  if ((m >> chunk_log2) < (1ull << 23)) sample_log2 = 0;
   v.part_chunks = (1u << chunk_log2) - 1u;
   v.part_sample = ((1ull << sample_log2) - 1ull) << std::max(16, log2_exact(o.partition_bins));
   v.hdr = reinterpret_cast<DevHeader*>(base + L.header);
@@ -387,7 +391,7 @@ RunView make_view(const uint8_t* d_bases, const uint64_t* d_offsets, uint64_t n_
     v.o_meta = reinterpret_cast<uint32_t*>(base + L.ometa);
     v.o_tiles = L.o_tiles;
     v.o_fused = L.o_fused;
-    v.o_bucketed = k >= 28 && !o.partial;
+    v.o_bucketed = k >= 32 && !o.partial;
     // about 4096 members per work item
     v.o_item_tiles = (uint32_t)std::max<uint64_t>(8, (uint64_t)L.o_regions * rounds / (kOrdTile / 4096));
     v.o_tcap = L.o_tcap;

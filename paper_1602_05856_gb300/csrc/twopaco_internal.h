@@ -135,9 +135,9 @@ struct RunView {
                             // partial: one word
   uint32_t* o_meta;         // per tile and bucket: where the tile's records start in the bucket
   uint64_t o_tiles;         // tiles of kOrdTile positions: ceil(m / kOrdTile)
-  int o_bucketed;           // 28 <= k <= 63, not partial: pass 2 bucket by bucket, through the lists
+  int o_bucketed;           // 32 <= k <= 63, not partial: pass 2 bucket by bucket, through the lists
   uint32_t o_item_tiles;    // tiles per work item of its insert loop
-  int o_fused;              // k <= 27, not partial: pass 2 runs on the records (fused records)
+  int o_fused;              // k <= 31, not partial: pass 2 runs on the records (fused records)
   uint32_t o_tcap;          // fused: table slots per bucket (region), the table is o_regions x o_tcap slots
   int use_desc;             // the insert leaves descriptors and the probe reads them
   uint64_t cand_cap;        // records the list can hold
@@ -175,7 +175,7 @@ constexpr uint64_t kOrdTile = 16384;       // region-ordered first pass: positio
 constexpr uint32_t kOrdMaxRegions = 256;   // buckets (filter regions), at most
 constexpr uint32_t kOrdMaxHist = 4096;     // rounds x regions, at most
 constexpr uint32_t kOrdFillStride = 32;    // bucket fill counters 128 bytes apart
-constexpr uint32_t kOrdScanTiles = 128;    // tiles per block of the scans over tiles
+constexpr uint32_t kOrdScanTiles = 64;     // tiles per block of the scans over tiles
 
 // Kernel launch helpers (twopaco_kernels.cu). Each returns the number of
 // kernels it launched, or -1 after a launch error.

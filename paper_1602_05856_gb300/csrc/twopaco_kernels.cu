@@ -431,55 +431,64 @@ __device__ __forceinline__ int32_t rel(uint64_t x, uint64_t p0) {
 // because the list marks candidates at a string end (sentinel positions)
 // and every other candidate has a predecessor and a successor. Those are read
 // from one window with the k-mer, which starts at the predecessor: 2 KW + 1
-// aligned words hold any 16 (2 KW) + 1 bases (k = 63 and four-word k-mers read
-// their successor apart).
+// aligned words hold any 32 KW + 1 bases.
+//
+// word(i) gives word i of the window's packed words: the window starts at the
+// base p (2 bits) of word 0 (the predecessor, or a sentinel's first base).
+template <int KW, typename F>
+__device__ __forceinline__ void read_window(const RunView& v, uint32_t p, bool sentinel, F&& word, OccT<KW>* oc) {
+  static_assert(KW <= 2, "four-word k-mers are read apart");
+  constexpr int W = 2 * KW;
+  const int k = v.k;
+  uint32_t w[W + 1], x[W + 1];
+#pragma unroll
+  for (int j = 0; j <= W; ++j) w[j] = word(j);
+#pragma unroll
+  for (int j = 0; j <= W; ++j) x[j] = __funnelshift_l(j < W ? w[j + 1] : 0u, w[j], 2u * p);
+  uint32_t pred = 0, succ = 0;
+  if (sentinel) {  // the window starts at the k-mer: move it to where the others have it
+#pragma unroll
+    for (int j = W; j >= 0; --j) x[j] = __funnelshift_r(x[j], j ? x[j - 1] : 0u, 2);
+  } else {
+    pred = x[0] >> 30;
+    const int sw = (k + 1) >> 4;  // base k + 1 of the window
+    uint32_t y = x[W];
+#pragma unroll
+    for (int j = 0; j < W; ++j)
+      if (j == sw) y = x[j];
+    succ = (y >> (30 - 2 * ((k + 1) & 15))) & 3u;
+  }
+  uint64_t top[KW];  // the 32 KW bases after the window's first
+#pragma unroll
+  for (int j = 0; j < KW; ++j)
+    top[j] = ((uint64_t)__funnelshift_l(x[2 * j + 1], x[2 * j], 2) << 32) | __funnelshift_l(x[2 * j + 2], x[2 * j + 1], 2);
+  Key f;
+  if constexpr (KW == 1) {
+    f.hi = 0;
+    f.lo = top[0] >> (64 - 2 * k);
+  } else {
+    const int sh = 128 - 2 * k;  // 2 .. 64
+    f.hi = sh == 64 ? 0ull : top[0] >> sh;
+    f.lo = sh == 64 ? top[0] : (top[1] >> sh) | (top[0] << (64 - sh));
+  }
+  const Key r = v.both ? revcomp<KW>(f, k) : f;
+  make_occ<KW>(v, f, r, pred, succ, sentinel, oc);
+}
+
 template <int KW>
 __device__ __forceinline__ void read_listed(const RunView& v, uint64_t g, bool sentinel, OccT<KW>* oc) {
-  const int k = v.k;
-  KeyT<KW> f;
-  uint32_t pred = 0, succ = 0;
-  if (sentinel || KW == 4) {
-    f = load_kmer<KW>(v.packed, g, k);
-    if (!sentinel) {
-      pred = base_at(v.packed, g - 1);
-      succ = base_at(v.packed, g + k);
-    }
+  if constexpr (KW == 4) {
+    const int k = v.k;
+    const Key4 f = load_kmer<4>(v.packed, g, k);
+    const Key4 r = v.both ? revcomp<4>(f, k) : f;
+    const uint32_t pred = sentinel ? 0u : base_at(v.packed, g - 1);
+    const uint32_t succ = sentinel ? 0u : base_at(v.packed, g + k);
+    make_occ<4>(v, f, r, pred, succ, sentinel, oc);
   } else {
-    constexpr int W = 2 * KW;
-    const uint32_t* p = v.packed + ((g - 1) >> 4);
-    const uint32_t o2 = 2u * (uint32_t)((g - 1) & 15);
-    uint32_t w[W + 1], x[W + 1];
-#pragma unroll
-    for (int j = 0; j <= W; ++j) w[j] = __ldg(p + j);
-#pragma unroll
-    for (int j = 0; j <= W; ++j) x[j] = __funnelshift_l(j < W ? w[j + 1] : 0u, w[j], o2);  // from g - 1 on
-    pred = x[0] >> 30;
-    // base k + 1 of the window
-    const int sw = (k + 1) >> 4, ss = 30 - 2 * ((k + 1) & 15);
-    if (KW == 2 && k == 63) {
-      succ = base_at(v.packed, g + k);
-    } else {
-      uint32_t y = x[W];
-#pragma unroll
-      for (int j = 0; j < W; ++j)
-        if (j == sw) y = x[j];
-      succ = (y >> ss) & 3u;
-    }
-    uint64_t top[KW];  // the 32 KW bases from g on
-#pragma unroll
-    for (int j = 0; j < KW; ++j)
-      top[j] = ((uint64_t)__funnelshift_l(x[2 * j + 1], x[2 * j], 2) << 32) | __funnelshift_l(x[2 * j + 2], x[2 * j + 1], 2);
-    if constexpr (KW == 1) {
-      f.hi = 0;
-      f.lo = top[0] >> (64 - 2 * k);
-    } else if constexpr (KW == 2) {
-      const int sh = 128 - 2 * k;  // 2 .. 64
-      f.hi = sh == 64 ? 0ull : top[0] >> sh;
-      f.lo = sh == 64 ? top[0] : (top[1] >> sh) | (top[0] << (64 - sh));
-    }
+    const uint64_t a = sentinel ? g : g - 1;
+    const uint32_t* p = v.packed + (a >> 4);
+    read_window<KW>(v, (uint32_t)a & 15u, sentinel, [&](int j) { return __ldg(p + j); }, oc);
   }
-  const KeyT<KW> r = v.both ? revcomp<KW>(f, k) : f;
-  make_occ<KW>(v, f, r, pred, succ, sentinel, oc);
 }
 
 // A k-mer as 2 KW 32-bit words, w[0] the most significant.
@@ -2033,85 +2042,89 @@ __global__ void __launch_bounds__(kBlock) pass1_probe_cm_kernel(RunView v, int r
 // A record: bits 0-21 the word within its region, 22-51 the bits 32-61 of G
 // (the bit bases of up to 6 bits per item), 52-56 and 57-61 the items (two
 // for a palindrome's orientations), bit 62 the sentinel flag. With pass 2 on
-// the records (k <= 27) a record holds the occurrence instead (fused_record).
+// the records (k <= 31) a record holds the occurrence instead (fused_record).
 // ---------------------------------------------------------------------------
 
 constexpr uint32_t kOrdPiece = 4096;  // records per apply or probe work item (a multiple of 32)
 constexpr unsigned long long kOrdSentinel = 1ull << 62;
 
-// Fused records (k <= 27, o_fused): the round's pass 2 runs on the same
-// records. A record then holds the occurrence itself -- bits 7-60 the
-// normalized k-mer, 6 the sentinel flag, 5 and 4 whether the string reads the
-// k-mer's reverse complement and the k-mer itself there (both for a
-// palindrome), 2-3 and 0-1 the predecessor and successor bases -- and the
-// kernels that apply it recompute H, G, the filter word and the items.
-__device__ __forceinline__ unsigned long long fused_record(const RunView& v, uint64_t g, bool sentinel) {
-  // one window of 32 bases from the predecessor on holds it all (k + 2 <= 29)
-  const uint64_t x = sentinel ? bases32(v.packed, g) >> 2 : bases32(v.packed, g - 1);
-  Key f;
-  f.hi = 0;
-  f.lo = (x << 2) >> (64 - 2 * v.k);
-  const Key r = v.both ? revcomp<1>(f, v.k) : f;
-  const uint32_t pred = sentinel ? 0u : (uint32_t)(x >> 62);
-  const uint32_t succ = sentinel ? 0u : (uint32_t)(x >> (60 - 2 * v.k)) & 3u;
-  const bool use_f = !v.both || !key_less(r, f);
-  const bool use_r = v.both && !key_less(f, r);
-  const uint64_t key = use_f ? f.lo : r.lo;
-  return (key << 7) | ((uint64_t)sentinel << 6) | ((uint64_t)use_r << 5) | ((uint64_t)use_f << 4) |
-         ((uint64_t)pred << 2) | succ;
+// Fused records (k <= 31, o_fused): the round's pass 2 runs on the same
+// records. The hash of a one-word k-mer is a bijection, and the bucket gives
+// its top bits, so a record holds the k-mer as the low 64 - log2(R) bits of H
+// (bits 6 up), with the item its occurrence inserts (bits 0-3), whether the
+// k-mer is a palindrome (4: the other strand's item too) and whether it is a
+// sentinel (5). The kernels that apply it hash nothing but G: with the k-mer
+// and its bases in the record, each of them mixed it again, and the probe and
+// the classify were bound by their integer instructions (73% issue).
+constexpr uint32_t kFusedPalindrome = 16u, kFusedSentinel = 32u;
+constexpr int kFusedBits = 6;
+
+template <int KW>
+__device__ __forceinline__ unsigned long long fused_record(const OccT<KW>& oc) {
+  return (oc.H << kFusedBits) | (oc.sentinel ? kFusedSentinel : (oc.j1 | (oc.j2 != oc.j1 ? kFusedPalindrome : 0u)));
 }
 
 struct FusedOcc {
-  uint64_t key, H, G;
-  uint32_t j1, j2, tbits;
+  uint64_t H, G;
+  uint32_t j1, j2;
   bool sentinel;
 };
 
-__device__ __forceinline__ FusedOcc fused_occ(unsigned long long rec) {
+// top: the bucket's bits of H, in place (fused_top).
+__device__ __forceinline__ FusedOcc fused_occ(unsigned long long rec, uint64_t top, uint64_t low_mask) {
   FusedOcc o;
-  o.key = rec >> 7;
-  o.sentinel = (rec >> 6) & 1u;
-  occ_bits((uint32_t)(rec >> 2) & 3u, (uint32_t)rec & 3u, (rec >> 4) & 1u, (rec >> 5) & 1u, o.sentinel, &o.j1, &o.j2,
-           &o.tbits);
-  o.H = mix64(o.key);  // key_hash of a one-word k-mer
+  o.H = top | ((rec >> kFusedBits) & low_mask);
   o.G = second_hash(o.H);
+  const uint32_t f = (uint32_t)rec, j = f & 15u;
+  o.sentinel = f & kFusedSentinel;
+  o.j1 = o.sentinel ? 16u : j;
+  o.j2 = (f & kFusedPalindrome) ? item_reverse(j >> 2, j & 3u) : o.j1;
   return o;
 }
 
-// The fused pass-2 table: bucket b owns the o_tcap one-word slots (key << 9 |
-// mask) from b * o_tcap, so that its inserts and lookups stay in L2 beside
-// the filter region; a k-mer starts at bits 16-47 of H scaled to o_tcap
-// (Lemire's multiply-high) and probes linearly within the part. Slot by slot,
+// Buckets are the top bits of H: R regions, a power of two of at least 64.
+__device__ __forceinline__ int fused_low_bits(const RunView& v) { return 64 - (31 - __clz(v.o_regions)); }
+
+// The fused pass-2 table: bucket b owns the o_tcap one-word slots from b *
+// o_tcap, so that its inserts and lookups stay in L2 beside the filter region.
+// A slot: the k-mer as the low bits of H (bits 5 up), the item of its first
+// occurrence (1-4), and whether it is a junction (0) -- a sentinel, or seen with
+// two items, which differ in the in- or the out-base. Empty: all ones, which no
+// slot is (58 bits of H at most). A k-mer starts at bits 16-47 of H scaled to
+// o_tcap (Lemire's multiply-high) and probes linearly within the part. Slot by slot,
 // unlike the direct table: the whole reserve is the table, at a load of a few
 // percent, so that the first slot mostly decides (a sector at a time took the
 // probe of 6 Gbp from 7.6 to 11.4 ps per position).
-__device__ __forceinline__ bool fused_table_insert(const RunView& v, uint32_t b, uint64_t key, uint64_t H,
-                                                   uint32_t tbits) {
+__device__ __forceinline__ bool fused_table_insert(const RunView& v, uint32_t b, const FusedOcc& o,
+                                                   uint64_t low_mask) {
   const uint32_t cap = v.o_tcap;
   unsigned long long* T = static_cast<unsigned long long*>(v.table) + (uint64_t)b * cap;
-  uint32_t i = __umulhi((uint32_t)(H >> 16), cap);
+  const bool junction = o.sentinel || o.j1 != o.j2;
+  const unsigned long long mine = ((o.H & low_mask) << 5) | ((o.j1 & 15u) << 1) | (junction ? 1u : 0u);
+  uint32_t i = __umulhi((uint32_t)(o.H >> 16), cap);
   for (uint32_t probe = 0; probe < cap; ++probe, i = i + 1 == cap ? 0u : i + 1) {
     unsigned long long cur = __ldcg(T + i);
     if (cur == kEmpty) {
-      cur = atomicCAS(T + i, kEmpty, (key << kMaskBits) | tbits);
+      cur = atomicCAS(T + i, kEmpty, mine);
       if (cur == kEmpty) return true;
     }
-    if ((cur >> kMaskBits) != key) continue;
-    if ((cur & tbits) != tbits) atomicOr(T + i, (unsigned long long)tbits);
+    if ((cur ^ mine) >> 5) continue;
+    if (!(cur & 1u) && cur != mine) atomicOr(T + i, 1ull);
     return true;
   }
   return false;
 }
 
-// Mask of key in the fused table, or -1 if absent.
-__device__ __forceinline__ int fused_table_find(const RunView& v, uint32_t b, uint64_t key, uint64_t H) {
+// 1 or 0: the k-mer of H is a junction or not; -1: absent.
+__device__ __forceinline__ int fused_table_find(const RunView& v, uint32_t b, uint64_t H, uint64_t low_mask) {
   const uint32_t cap = v.o_tcap;
   const unsigned long long* T = static_cast<const unsigned long long*>(v.table) + (uint64_t)b * cap;
+  const uint64_t key = H & low_mask;
   uint32_t i = __umulhi((uint32_t)(H >> 16), cap);
   for (uint32_t probe = 0; probe < cap; ++probe, i = i + 1 == cap ? 0u : i + 1) {
     const unsigned long long cur = __ldcg(T + i);
     if (cur == kEmpty) return -1;
-    if ((cur >> kMaskBits) == key) return (int)(cur & ((1u << kMaskBits) - 1u));
+    if ((cur >> 5) == key) return (int)(cur & 1u);
   }
   return -1;
 }
@@ -2272,10 +2285,20 @@ __global__ void __launch_bounds__(kBlock) ord_scatter_kernel(RunView v, int roun
   __shared__ unsigned long long delta_s[kOrdMaxRegions];
   __shared__ uint64_t start_s[kOrdMaxRegions];
   __shared__ uint32_t run_s[kOrdMaxRegions];
+  // the tile's packed words, from the one before on: the members come in bucket
+  // order, so a warp's windows lie all over the tile, and as many lines of L1 as
+  // lanes (L1 at 71% bounded the kernel)
+  constexpr int kWords = (int)(kOrdTile / 16), kStaged = 1 + kWords + 2 * KW + 1;
+  __shared__ uint32_t words_s[kStaged];
   if (!ordered_round(v)) return;
   for (uint32_t b = threadIdx.x; b < v.o_regions; b += kBlock) start_s[b] = v.o_start[b];
   const uint64_t local_mask = (1ull << v.o_lg_region_words) - 1ull;
   for (uint64_t t = blockIdx.x; t < v.o_tiles; t += gridDim.x) {
+    const uint64_t w0 = t * kWords;  // words_s[i] = packed word w0 + i - 1
+    for (int i = threadIdx.x; i < kStaged; i += kBlock) {
+      const uint64_t w = w0 + i;
+      words_s[i] = w && w <= v.packed_words ? __ldg(v.packed + w - 1) : 0u;
+    }
     const TileMembers tm = ord_tile(v, t, round, start_s, delta_s, run_s, bucket_s);
     constexpr int U = KW == 1 ? 4 : 2;
     for (uint32_t i0 = threadIdx.x; i0 < tm.n; i0 += U * kBlock) {
@@ -2287,13 +2310,13 @@ __global__ void __launch_bounds__(kBlock) ord_scatter_kernel(RunView v, int roun
         const uint32_t i = i0 + u * kBlock;
         if (i >= tm.n) break;
         const bool sentinel = e[u] & kOrdEntrySentinel;
-        const uint64_t g = t * kOrdTile + (e[u] & kOrdEntryPos);
+        const uint32_t a = 16u + (e[u] & kOrdEntryPos) - (sentinel ? 0u : 1u);  // base of words_s
+        OccT<KW> oc;
+        read_window<KW>(v, a & 15u, sentinel, [&](int j) { return words_s[(a >> 4) + j]; }, &oc);
         unsigned long long rec;
         if constexpr (FUSED) {
-          rec = fused_record(v, g, sentinel);
+          rec = fused_record(oc);
         } else {
-          OccT<KW> oc;
-          read_listed<KW>(v, g, sentinel, &oc);
           const uint64_t G = second_hash(oc.H);
           const uint64_t word = filter_index(v, oc.H, G);
           rec = (word & local_mask) | (((G >> 32) & 0x3FFFFFFFull) << 22) | ((uint64_t)oc.j1 << 52) |
@@ -2363,6 +2386,8 @@ __global__ void __launch_bounds__(kBlock) ord_or_kernel(RunView v) {
     const uint64_t i0 = (uint64_t)(item - first_s[b]) * kOrdPiece, i1 = min(i0 + kOrdPiece, n);
     const uint64_t* recs = v.o_recs + __ldg(v.o_start + b);
     unsigned long long* region = v.filter + ((uint64_t)b << v.o_lg_region_words);
+    const uint64_t low_mask = FUSED ? (1ull << fused_low_bits(v)) - 1ull : 0ull;
+    const uint64_t top = FUSED ? (uint64_t)b << fused_low_bits(v) : 0ull;
     for (uint64_t i = i0 + threadIdx.x; i < i1; i += 4 * kBlock) {
       uint64_t r[4];
 #pragma unroll
@@ -2371,7 +2396,7 @@ __global__ void __launch_bounds__(kBlock) ord_or_kernel(RunView v) {
       for (int u = 0; u < 4; ++u) {
         if (r[u] == ~0ull) continue;
         if constexpr (FUSED) {
-          const FusedOcc o = fused_occ(r[u]);
+          const FusedOcc o = fused_occ(r[u], top, low_mask);
           const ItemPattern pat = item_pattern<HB>(o.G, v.hashes);
           uint64_t m = item_bits(pat, o.j1);
           if (o.j2 != o.j1) m |= item_bits(pat, o.j2);
@@ -2421,6 +2446,8 @@ __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
     // U chunks of 32 records per warp and step: their records, then their filter
     // words, all in flight at once
     constexpr int U = FUSED ? 2 : 4;
+    const uint64_t low_mask = FUSED ? (1ull << fused_low_bits(v)) - 1ull : 0ull;
+    const uint64_t top = FUSED ? (uint64_t)b << fused_low_bits(v) : 0ull;
     for (uint64_t w0 = i0 + 32 * wid; w0 < i1; w0 += U * kBlock) {
       unsigned long long rec[U], word[U];
 #pragma unroll
@@ -2433,7 +2460,7 @@ __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
         word[u] = 0;
         if (rec[u] == ~0ull) continue;
         if constexpr (FUSED) {
-          const FusedOcc o = fused_occ(rec[u]);
+          const FusedOcc o = fused_occ(rec[u], top, low_mask);
           if (!o.sentinel) word[u] = __ldcg(v.filter + filter_index(v, o.H, o.G));
         } else {
           if (!(rec[u] & kOrdSentinel)) word[u] = __ldcg(v.filter + (region | (rec[u] & 0x3FFFFFull)));
@@ -2446,10 +2473,10 @@ __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
         bool keep = false;
         if (rec[u] != ~0ull) {
           if constexpr (FUSED) {  // the decision, and the candidate's edges into the region's table
-            const FusedOcc o = fused_occ(rec[u]);
+            const FusedOcc o = fused_occ(rec[u], top, low_mask);
             const uint32_t pres = present_items<HB>(o.G, word[u], v.hashes);
             keep = o.sentinel || (pres >> 16) || __popc(pres & 0xFFFFu) >= 2;
-            if (keep && !fused_table_insert(v, b, o.key, o.H, o.tbits)) v.hdr->overflow = 1;
+            if (keep && !fused_table_insert(v, b, o, low_mask)) v.hdr->overflow = 1;
           } else {
             const uint64_t G = ((rec[u] >> 22) & 0x3FFFFFFFull) << 32;
             const uint32_t pres = present_items<HB>(G, word[u], v.hashes);
@@ -2475,9 +2502,8 @@ __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
 // Algorithm 1, probe loop, second pass, on fused records, bucket by bucket:
 // every candidate record (decision bit set) looks its k-mer up in the
 // region's table; its bit in the junction word of o_dec says whether the
-// k-mer is a junction (the table mask holds the sentinel bit or more than
-// one in- or out-base).
-__global__ void __launch_bounds__(kBlock) ord_classify_kernel(RunView v) {
+// k-mer is a junction.
+__global__ void __launch_bounds__(kBlock, 8) ord_classify_kernel(RunView v) {
   __shared__ uint32_t first_s[kOrdMaxRegions + 1];
   __shared__ uint32_t item_s;
   if (!ordered_round(v)) return;
@@ -2494,6 +2520,7 @@ __global__ void __launch_bounds__(kBlock) ord_classify_kernel(RunView v) {
     const uint64_t n = __ldcg(v.o_fill + (uint64_t)b * kOrdFillStride);
     const uint64_t i0 = (uint64_t)(item - first_s[b]) * kOrdPiece, i1 = min(i0 + kOrdPiece, n);
     const uint64_t start = __ldg(v.o_start + b);  // a multiple of 32, as is i0
+    const uint64_t low_mask = (1ull << fused_low_bits(v)) - 1ull, top = (uint64_t)b << fused_low_bits(v);
     const uint64_t* recs = v.o_recs + start;
     // four chunks of 32 records per warp and step: their loads all in flight at once
     constexpr int U = 4;
@@ -2515,10 +2542,9 @@ __global__ void __launch_bounds__(kBlock) ord_classify_kernel(RunView v) {
         const uint64_t c = w0 + (uint64_t)u * kBlock;
         bool junction = false;
         if (rec[u] != ~0ull) {
-          const FusedOcc o = fused_occ(rec[u]);
-          const int mk = fused_table_find(v, b, o.key, o.H);
-          if (mk < 0) v.hdr->overflow = 1;
-          junction = mk < 0 || is_junction_mask(mk);
+          const int j = fused_table_find(v, b, top | ((rec[u] >> kFusedBits) & low_mask), low_mask);
+          if (j < 0) v.hdr->overflow = 1;
+          junction = j != 0;
         }
         const uint32_t row = __ballot_sync(0xffffffffu, junction);
         if (lane == 0 && c < i1) v.o_dec[(((start + c) >> 5) << 1) + 1] = row;
@@ -2527,7 +2553,7 @@ __global__ void __launch_bounds__(kBlock) ord_classify_kernel(RunView v) {
   }
 }
 
-// Pass 2 bucket by bucket for k-mers that no record holds (28 <= k <= 63): the
+// Pass 2 bucket by bucket for k-mers that no record holds (32 <= k <= 63): the
 // table has one part per filter region (table_setup), and the candidates of a
 // bucket -- found by its records' decision bits, and their positions by the
 // tiles' lists -- are inserted part by part, so that the table's random accesses
@@ -3716,7 +3742,7 @@ static int ordered_round_impl(const RunView& v, int round, cudaStream_t s, RunVi
   if (!v.partial) {
     launch_table<TS>(*pv, s);
     launched += 2;
-    if (!fused) {
+    if constexpr (KW == 2) {
       {
         Timed t("ord_insert2", s);
         auto kern = ord_insert2_kernel<KW, TS>;
