@@ -199,15 +199,13 @@ int launch_edges(const DevHeader* hdr_dev, const uint64_t* d_offsets, uint64_t n
                  const uint64_t* d_out_offsets, const uint64_t* d_out_positions,
                  uint64_t* d_edge_offsets, void* d_edges, uint64_t edge_capacity, cudaStream_t s);
 
-// Pass-2 slot layout for this k: 0 = one 64-bit word (key << 9 | mask, k <= 27),
-// 1 = 16 bytes (k <= 31), 2 = 32 bytes (128-bit key).
 // Pass-2 table slots: 0 = one word (key << 9 | mask, k <= 27); 1 = 16 B key +
-// mask (k <= 31); 2 = 32 B 128-bit key + mask (k <= 63); 3 = 16 B reference
-// to an occurrence + mask (k <= 127).
+// mask (k <= 31); 2 = 32 B 128-bit key + mask (k <= 63); 3 = one word, a
+// reference to an occurrence + mask (k <= 127).
 inline int table_slot_kind(int k) { return k <= 27 ? 0 : (k <= 31 ? 1 : (k <= 63 ? 2 : 3)); }
 inline uint64_t table_slot_bytes(int k) {
   const int t = table_slot_kind(k);
-  return t == 3 ? 16ull : (8ull << t);
+  return t == 3 ? 8ull : (8ull << t);
 }
 
 // Bytes per candidate record (a global position).

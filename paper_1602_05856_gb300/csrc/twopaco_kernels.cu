@@ -19,6 +19,7 @@
 // of a k-mer is min(k-mer, reverse complement)), and complement is 3 - x.
 #include "twopaco_internal.h"
 
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 #include <string>
@@ -95,6 +96,11 @@ struct Timed {
 // Consecutive positions per thread (at most 16: one 32-bit word of successor
 // bases) in the first-pass kernels and the partition pre-pass.
 constexpr int kInsertR = 16;
+// Inputs below kInsertSmall positions take fewer per thread, so that all SMs
+// have warps to spare: 16 per thread left 0.2 M positions on 46 blocks (insert
+// 16 -> 10 us); at 3.8 M positions 16 are the better ones (126 us a build to 129).
+constexpr int kInsertSmallR = 4;
+constexpr uint64_t kInsertSmall = 1ull << 21;
 constexpr int kProbeR = 8;
 constexpr bool kProbePrefetch = true;  // the probe's descriptors loaded one step ahead
 constexpr int kR = 8;  // partition pre-pass
@@ -856,22 +862,22 @@ __device__ __forceinline__ void cas128(unsigned long long* addr, uint64_t cmp_lo
 
 constexpr uint64_t kNoSlot = ~0ull;
 
-// Slots of a 32-byte sector (four one-word slots, two 16-byte ones): a probe
+// Slots of a 32-byte sector (four 8-byte slots, two 16-byte ones): a probe
 // starts at a k-mer's sector and reads a whole sector at a time, so that a
 // k-mer mostly costs one round trip. Slot by slot from any start, the longest
 // of a warp's 32 chains -- six to eight slots at a load of 0.4 -- cost one each,
 // and the rest of the warp its instructions. Tables hold whole sectors.
 template <int TS>
 struct SectorOf {
-  static constexpr int kSlots = TS == 0 ? 4 : (TS == 2 ? 1 : 2);
-  unsigned long long key[kSlots];   // the slot's word (TS 0), key (1), low key word (2) or reference (3)
-  unsigned long long more[kSlots];  // its mask (1, 3) or high key word (2)
+  static constexpr int kSlots = TS == 0 || TS == 3 ? 4 : (TS == 2 ? 1 : 2);
+  unsigned long long key[kSlots];   // the slot's word (TS 0, 3), key (1) or low key word (2)
+  unsigned long long more[kSlots];  // its mask (1) or high key word (2)
   unsigned int mask;                // TS 2: its mask
 
   __device__ __forceinline__ void load(const void* table, uint64_t first) {  // first: a multiple of kSlots
     const ulonglong2* p = reinterpret_cast<const ulonglong2*>(static_cast<const char*>(table) + first * (32 / kSlots));
     const ulonglong2 a = __ldcg(p), b = __ldcg(p + 1);
-    if constexpr (TS == 0) {
+    if constexpr (TS == 0 || TS == 3) {
       key[0] = a.x; key[1] = a.y; key[2] = b.x; key[3] = b.y;
     } else if constexpr (TS == 2) {
       key[0] = a.x; more[0] = a.y;
@@ -1011,17 +1017,15 @@ __device__ __forceinline__ int table_find(const RunView& v, uint64_t cap, const 
 
 // Slots of k-mers of 64 to 127 bases (kind 3): instead of the key, a
 // reference to one occurrence of it -- bits 0-47 its position + 1, bit 48
-// whether the string reads the key's reverse complement there, bits 49-63
-// the top 15 bits of H as a tag. 0 is empty. Keys are compared by reading the
-// referenced occurrence back from the packed input, so one 64-bit CAS claims
-// a slot for a key of any length.
-struct alignas(16) Slot3 {
-  unsigned long long ref;
-  unsigned int mask;
-  unsigned int pad;
-};
-
+// whether the string reads the key's reverse complement there -- with the
+// pass-2 mask (bits 49-57) and the top six bits of H as a tag (58-63). 0 is
+// empty. Keys are compared by reading the referenced occurrence back from the
+// packed input, so one 64-bit CAS claims a slot for a key of any length, its
+// first bits included. (With the mask in a second word beside a 15-bit tag, a
+// new k-mer took a CAS and an OR, and the table twice the memory: 672 us for
+// 11.6 M candidates, 10 M of them new, in a 328 MB table.)
 constexpr uint64_t kRefPos = (1ull << 48) - 1;
+constexpr int kRefMask = 49, kRefTag = 58;
 
 __device__ __forceinline__ bool ref_holds(const RunView& v, uint64_t ref, const Key4& key) {
   Key4 x = load_kmer<4>(v.packed, (ref & kRefPos) - 1, v.k);
@@ -1032,43 +1036,45 @@ __device__ __forceinline__ bool ref_holds(const RunView& v, uint64_t ref, const 
 __device__ __forceinline__ uint64_t table_insert_ref(const RunView& v, uint64_t cap, const Key4& key,
                                                      uint64_t H, uint64_t start, uint32_t bits, uint64_t g,
                                                      bool rc) {
-  const uint64_t tag = H >> 49;
-  const unsigned long long mine = (tag << 49) | ((uint64_t)rc << 48) | (g + 1);
+  const uint64_t tag = H >> kRefTag, add = (uint64_t)bits << kRefMask;
+  const unsigned long long mine = (tag << kRefTag) | add | ((uint64_t)rc << 48) | (g + 1);
   uint64_t base = start;
-  for (uint64_t seen = 0; seen < cap; seen += 2) {
+  for (uint64_t seen = 0; seen < cap; seen += 4) {
     SectorOf<3> q;
     q.load(v.table, base);
 #pragma unroll
-    for (uint64_t k = 0; k < 2; ++k) {
-      Slot3* s = static_cast<Slot3*>(v.table) + base + k;
+    for (uint64_t k = 0; k < 4; ++k) {
+      unsigned long long* s = static_cast<unsigned long long*>(v.table) + base + k;
       unsigned long long cur = q.key[k];
-      uint32_t have = (uint32_t)q.more[k];
       if (cur == 0) {
-        cur = atomicCAS(&s->ref, 0ull, mine);
-        have = 0;
-        if (cur == 0) cur = mine;  // claimed
+        cur = atomicCAS(s, 0ull, mine);
+        if (cur == 0) return base + k;
       }
-      if (cur != mine && ((cur >> 49) != tag || !ref_holds(v, cur, key))) continue;
-      if ((have & bits) != bits) atomicOr(&s->mask, bits);
+      if ((cur >> kRefTag) != tag || !ref_holds(v, cur, key)) continue;
+      if ((cur & add) != add) atomicOr(s, (unsigned long long)add);
       return base + k;
     }
-    base = base + 2 == cap ? 0 : base + 2;
+    base = base + 4 == cap ? 0 : base + 4;
   }
   return kNoSlot;
 }
 
+__device__ __forceinline__ int ref_mask(unsigned long long slot) {
+  return (int)(slot >> kRefMask) & ((1 << kMaskBits) - 1);
+}
+
 __device__ __forceinline__ int table_find_ref(const RunView& v, uint64_t cap, const Key4& key, uint64_t H) {
-  const uint64_t tag = H >> 49;
-  uint64_t base = slot_start<2>(H, cap);
-  for (uint64_t seen = 0; seen < cap; seen += 2) {
+  const uint64_t tag = H >> kRefTag;
+  uint64_t base = slot_start<4>(H, cap);
+  for (uint64_t seen = 0; seen < cap; seen += 4) {
     SectorOf<3> q;
     q.load(v.table, base);
 #pragma unroll
-    for (uint64_t k = 0; k < 2; ++k) {
+    for (uint64_t k = 0; k < 4; ++k) {
       if (q.key[k] == 0) return -1;
-      if ((q.key[k] >> 49) == tag && ref_holds(v, q.key[k], key)) return (int)(uint32_t)q.more[k];
+      if ((q.key[k] >> kRefTag) == tag && ref_holds(v, q.key[k], key)) return ref_mask(q.key[k]);
     }
-    base = base + 2 == cap ? 0 : base + 2;
+    base = base + 4 == cap ? 0 : base + 4;
   }
   return -1;
 }
@@ -1077,7 +1083,7 @@ __device__ __forceinline__ int table_find_ref(const RunView& v, uint64_t cap, co
 template <int KW, int TS>
 __device__ __forceinline__ uint64_t insert_occurrence(const RunView& v, uint64_t cap, const OccT<KW>& oc,
                                                       uint64_t g) {
-  if constexpr (TS == 3) return table_insert_ref(v, cap, oc.key, oc.H, slot_start<2>(oc.H, cap), oc.tbits, g, oc.rc);
+  if constexpr (TS == 3) return table_insert_ref(v, cap, oc.key, oc.H, slot_start<4>(oc.H, cap), oc.tbits, g, oc.rc);
   else return table_insert<TS>(v, cap, oc.key, slot_start<SectorOf<TS>::kSlots>(oc.H, cap), oc.tbits);
 }
 
@@ -1092,7 +1098,7 @@ template <int TS>
 __device__ __forceinline__ int table_mask(const RunView& v, uint64_t i) {
   if (TS == 0) return (int)(__ldcg(static_cast<const unsigned long long*>(v.table) + i) & ((1u << kMaskBits) - 1u));
   if (TS == 1) return (int)__ldcg(&(static_cast<const Slot1*>(v.table) + i)->mask);
-  if (TS == 3) return (int)__ldcg(&(static_cast<const Slot3*>(v.table) + i)->mask);
+  if (TS == 3) return ref_mask(__ldcg(static_cast<const unsigned long long*>(v.table) + i));
   return (int)__ldcg(&(static_cast<const Slot2*>(v.table) + i)->mask);
 }
 
@@ -1474,18 +1480,19 @@ __device__ __forceinline__ uint64_t make_desc(const RunView& v, uint64_t H, uint
 // descriptors are staged in shared memory (16-byte pairs, columns swizzled by
 // the owning thread so that neither side conflicts) and written out in
 // order, whole sectors at a time.
-template <int KW, bool ROUNDS, int HB, bool DESC, bool BKT = false>
+// R consecutive positions per thread: kInsertR, or kInsertSmallR for small inputs.
+template <int KW, bool ROUNDS, int HB, bool DESC, bool BKT = false, int R = kInsertR>
 __global__ void __launch_bounds__(kBlock) pass1_insert_kernel(RunView v, int round) {
-  constexpr int kTile = kBlock * kInsertR;  // positions per block per pass
-  constexpr int kPairs = kInsertR / 2;      // 16-byte descriptor pairs per thread
+  constexpr int kTile = kBlock * R;  // positions per block per pass
+  constexpr int kPairs = R / 2;      // 16-byte descriptor pairs per thread
   __shared__ ulonglong2 stage[DESC ? kTile / 2 : 1];
   const uint64_t stride = (uint64_t)gridDim.x * kTile;
   const int t = threadIdx.x;
   for (uint64_t base = v.p_begin + (uint64_t)blockIdx.x * kTile; base < v.p_end; base += stride) {
-    const uint64_t p0 = base + (uint64_t)t * kInsertR;
+    const uint64_t p0 = base + (uint64_t)t * R;
     if (p0 < v.m) {
       uint64_t prev = 0;
-      walk<KW, kInsertR>(v, p0, [&](int i, uint64_t, bool valid, const auto& oc) {
+      walk<KW, R>(v, p0, [&](int i, uint64_t, bool valid, const auto& oc) {
         uint64_t d = 0;
         if (valid) {
           if (ROUNDS && !in_round(v, oc.H, round)) {
@@ -2876,7 +2883,7 @@ __global__ void __launch_bounds__(kBlock) list_probe_kernel(RunView v, int round
 // where a smaller table stays in L2 (measured at k = 25, 31 and 63).
 constexpr double kTableLoadWord = 2.5, kTableLoad = 2.0;
 // pass-2 list work: parts of about this many records, at most kMaxParts per segment
-constexpr unsigned long long kPartRecords = 128, kMaxParts = 4096;
+constexpr unsigned long long kPartRecords = 128, kMaxParts = 4096, kPartWarps = 8192;
 // pass 2 bucket by bucket: tables of more than this (several times L2)
 constexpr unsigned long long kPartTableBytes = 512ull << 20;
 
@@ -2954,8 +2961,11 @@ __global__ void __launch_bounds__(1024) table_setup_kernel(RunView v) {
   h->table_slots = cap;
   if (cap > h->table_max) h->table_max = cap;
   h->round_listed = overflowed ? 0u : 1u;
-  // pass 2 cuts every list segment into parts of about kPartRecords records
-  const unsigned long long parts = (kept / v.n_segments + kPartRecords) / kPartRecords;
+  // pass 2 cuts every list segment into parts of about kPartRecords records, or
+  // down to one row where there are fewer such parts than warps
+  unsigned long long parts = (kept / v.n_segments + kPartRecords) / kPartRecords;
+  if (parts * v.n_segments < kPartWarps)
+    parts = max(parts, min(kept / v.n_segments / 32 + 1, (unsigned long long)(kPartWarps / v.n_segments)));
   h->list_parts = (unsigned int)(parts < kMaxParts ? parts : kMaxParts);
 }
 
@@ -2970,7 +2980,7 @@ __global__ void __launch_bounds__(kBlock) table_clear_kernel(RunView v) {
       Slot1* s = static_cast<Slot1*>(v.table) + i;
       *reinterpret_cast<ulonglong2*>(s) = make_ulonglong2(kEmpty, 0ull);
     } else if (TS == 3) {
-      reinterpret_cast<ulonglong2*>(v.table)[i] = make_ulonglong2(0ull, 0ull);
+      static_cast<unsigned long long*>(v.table)[i] = 0ull;
     } else {
       Slot2* s = static_cast<Slot2*>(v.table) + i;
       reinterpret_cast<ulonglong2*>(s)[0] = make_ulonglong2(kEmpty, kEmpty);
@@ -3581,21 +3591,59 @@ __global__ void __launch_bounds__(kBlock) edges_kernel(const DevHeader* hdr, con
 // Launch helpers
 // ---------------------------------------------------------------------------
 
-int sm_count() {
-  int dev = 0, n = 0;
-  cudaGetDevice(&dev);
+int sm_count(int dev) {
+  int n = 0;
   cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
   return n > 0 ? n : 1;
 }
 
-// Grid of at most (SMs x resident blocks per SM) blocks for work_items threads.
+// SMs and resident blocks per SM of a kernel: asked for once per kernel and
+// device (three runtime calls before every launch cost more host time than the
+// launch). Packed as SMs << 32 | blocks; devices past the table ask every time.
 template <typename K>
-unsigned grid_for(K kernel, int block, uint64_t work_items, int cap_per_sm = 0, size_t dyn_smem = 0) {
+uint64_t resident_blocks(K kernel, int block, size_t dyn_smem) {
+  struct Known {
+    std::atomic<const void*> kernel{nullptr};
+    std::atomic<uint64_t> value{0};
+  };
+  constexpr int kDevices = 16, kKernels = 64;
+  static Known known[kDevices][kKernels];  // one table per kernel signature
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const void* key = reinterpret_cast<const void*>(kernel);
+  Known* at = nullptr;
+  if (dev >= 0 && dev < kDevices) {
+    for (int i = 0; i < kKernels; ++i) {
+      const void* k = known[dev][i].kernel.load(std::memory_order_acquire);
+      if (k == key) {
+        const uint64_t v = known[dev][i].value.load(std::memory_order_acquire);
+        if (v) return v;
+        at = &known[dev][i];
+        break;
+      }
+      if (!k) {
+        if (known[dev][i].kernel.compare_exchange_strong(k, key) || k == key) {
+          at = &known[dev][i];
+          break;
+        }
+      }
+    }
+  }
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, dyn_smem);
+  const uint64_t v = ((uint64_t)sm_count(dev) << 32) | (uint32_t)std::max(per_sm, 1);
+  if (at) at->value.store(v, std::memory_order_release);  // the same from any thread
+  return v;
+}
+
+// Grid of at most (SMs x resident blocks per SM) blocks for work_items threads.
+// (A kernel is always launched with the same block size and dynamic memory.)
+template <typename K>
+unsigned grid_for(K kernel, int block, uint64_t work_items, int cap_per_sm = 0, size_t dyn_smem = 0) {
+  const uint64_t known = resident_blocks(kernel, block, dyn_smem);
+  int per_sm = (int)(uint32_t)known;
   if (cap_per_sm > 0 && per_sm > cap_per_sm) per_sm = cap_per_sm;  // a chosen launch shape
-  if (per_sm < 1) per_sm = 1;
-  const uint64_t full = (uint64_t)sm_count() * per_sm;
+  const uint64_t full = (known >> 32) * per_sm;
   const uint64_t need = (work_items + block - 1) / block;
   return (unsigned)(need < full ? (need ? need : 1) : full);
 }
@@ -3802,6 +3850,12 @@ static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges*
       for (uint64_t c0 = r.first; c0 < r.second; c0 += step) {
         const RunView x = part({c0, std::min(r.second, c0 + step)});
         const uint64_t threads = (x.p_end - x.p_begin + kInsertR - 1) / kInsertR;
+        constexpr int kSmallR = !RD ? kInsertSmallR : kInsertR;  // one round
+        const bool small = kSmallR < kInsertR && x.p_end - x.p_begin < kInsertSmall;
+        auto launch_insert = [&](auto kern, int r) {
+          const uint64_t n = (x.p_end - x.p_begin + r - 1) / r;
+          kern<<<grid_for(kern, kBlock, n, v.blocks_per_sm), kBlock, 0, s>>>(x, round);
+        };
         {
         Timed t("pass1_insert", s);
         if (bkt && cudaMemsetAsync(v.bucket_fill, 0, ((uint64_t)v.n_regions * v.n_sub + 1) * kFillStride * 4,
@@ -3816,16 +3870,17 @@ static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges*
         else if (desc && bkt)
           pass1_insert_kernel<KW, RD, HB, kDescOk, kBktOk>
               <<<grid_for(pass1_insert_kernel<KW, RD, HB, kDescOk, kBktOk>, kBlock, threads, v.blocks_per_sm), kBlock, 0, s>>>(x, round);
+        else if (desc && small)
+          launch_insert(pass1_insert_kernel<KW, RD, HB, kDescOk, false, kSmallR>, kSmallR);
         else if (desc)
-          pass1_insert_kernel<KW, RD, HB, kDescOk><<<grid_for(pass1_insert_kernel<KW, RD, HB, kDescOk>, kBlock,
-                                                              threads),
-                                                     kBlock, 0, s>>>(x, round);
+          launch_insert(pass1_insert_kernel<KW, RD, HB, kDescOk>, kInsertR);
         else if (bkt)
           pass1_insert_kernel<KW, RD, HB, false, kBktOk>
               <<<grid_for(pass1_insert_kernel<KW, RD, HB, false, kBktOk>, kBlock, threads, v.blocks_per_sm), kBlock, 0, s>>>(x, round);
+        else if (small)
+          launch_insert(pass1_insert_kernel<KW, RD, HB, false, false, kSmallR>, kSmallR);
         else
-          pass1_insert_kernel<KW, RD, HB, false><<<grid_for(pass1_insert_kernel<KW, RD, HB, false>, kBlock, threads, v.blocks_per_sm),
-                                                   kBlock, 0, s>>>(x, round);
+          launch_insert(pass1_insert_kernel<KW, RD, HB, false>, kInsertR);
         }
         ++launched;
         if (bkt) {
