@@ -605,7 +605,7 @@ __device__ __forceinline__ void walk_inside(const RunView& v, uint64_t p0, F&& f
 // piece) boundary or the input's end among them: rolling the k-mer from each
 // position to the next within a string and reading it from scratch after a
 // string boundary. b: the bounds at p0.
-template <int KW, int R, typename F>
+template <int KW, int R, bool ROLLED, typename F>
 __device__ __forceinline__ void walk_edges(const RunView& v, uint64_t p0, Bounds b, F&& fn) {
   static_assert(R >= 1 && R <= 16, "successor bases come from one 32-bit word");
   const int k = v.k;
@@ -616,8 +616,7 @@ __device__ __forceinline__ void walk_edges(const RunView& v, uint64_t p0, Bounds
   const uint32_t next = bases16(v.packed, p0 + (uint64_t)k);
   KeyT<KW> f{}, r{};
   bool fresh = true;
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
+  auto visit = [&](int i) {
     const uint64_t p = p0 + i;
     OccT<KW> oc;
     bool valid = false;
@@ -648,17 +647,27 @@ __device__ __forceinline__ void walk_edges(const RunView& v, uint64_t p0, Bounds
       }
     }
     fn(i, p, valid, oc);
+  };
+  if constexpr (ROLLED) {
+#pragma unroll 1
+    for (int i = 0; i < R; ++i) visit(i);
+  } else {
+#pragma unroll
+    for (int i = 0; i < R; ++i) visit(i);
   }
 }
 
 
 // Visit the R consecutive positions p0 .. p0 + R - 1 (p0 < m): fn(i, p, valid,
 // occ) runs for every i, with i a compile-time constant once unrolled.
-template <int KW, int R, typename F>
+// ROLLED: the rare walks over a boundary stay a loop, with i a run-time value
+// (an fn that does not index registers by it): unrolled beside the other walk
+// they made the inserts of four-word k-mers miss the instruction cache.
+template <int KW, int R, bool ROLLED = false, typename F>
 __device__ __forceinline__ void walk(const RunView& v, uint64_t p0, F&& fn) {
   const Bounds b = kmer_bounds(v, p0);
   if (b.start < p0 && p0 + (uint64_t)(R - 1 + v.k) < b.end) walk_inside<KW, R>(v, p0, fn);
-  else walk_edges<KW, R>(v, p0, b, fn);
+  else walk_edges<KW, R, ROLLED>(v, p0, b, fn);
 }
 
 __device__ __forceinline__ bool in_round(const RunView& v, uint64_t H, int round) {
@@ -1169,25 +1178,6 @@ __device__ __forceinline__ void lc_mark(const RunView& v, uint64_t h) {
 
 constexpr uint64_t kLcMul = 0xff51afd7ed558ccdull;
 
-// OR the bits of a row of positions into a bitmap: lane by lane ascending
-// positions g (lanes without one: g = ~0, set = false), bit g set where `set`.
-// The lanes of one bitmap word are combined into one atomic.
-__device__ __forceinline__ void or_row(uint32_t* bitmap, uint64_t g, bool set) {
-  const int lane = threadIdx.x & 31;
-  const uint64_t w = g >> 5;
-  const uint64_t prev = __shfl_up_sync(0xffffffffu, w, 1);
-  const bool head = lane == 0 || w != prev;
-  const uint32_t later = __ballot_sync(0xffffffffu, head) & (0xFFFFFFFEu << lane);  // heads after this lane
-  const int end = later ? __ffs(later) - 1 : 32;
-  uint32_t bits = set ? 1u << (g & 31) : 0u;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_down_sync(0xffffffffu, bits, o);
-    if (lane + o < end) bits |= y;
-  }
-  if (head && bits) atomicOr(bitmap + w, bits);
-}
-
 // ---------------------------------------------------------------------------
 // Kernels
 // ---------------------------------------------------------------------------
@@ -1492,7 +1482,7 @@ __global__ void __launch_bounds__(kBlock) pass1_insert_kernel(RunView v, int rou
     const uint64_t p0 = base + (uint64_t)t * R;
     if (p0 < v.m) {
       uint64_t prev = 0;
-      walk<KW, R>(v, p0, [&](int i, uint64_t, bool valid, const auto& oc) {
+      walk<KW, R, true>(v, p0, [&](int i, uint64_t, bool valid, const auto& oc) {
         uint64_t d = 0;
         if (valid) {
           if (ROUNDS && !in_round(v, oc.H, round)) {
@@ -1817,7 +1807,7 @@ __global__ void __launch_bounds__(kSortBlock, 2) class_sort_kernel(RunView v) {
         for (int i = 0; i < kInsertR; ++i) ent[i * kUnits + unit] = kSortNone;
         continue;
       }
-      walk<KW, kInsertR>(v, p0, [&](int i, uint64_t, bool valid, const auto& oc) {
+      walk<KW, kInsertR, true>(v, p0, [&](int i, uint64_t, bool valid, const auto& oc) {
         uint32_t e = kSortNone;
         if (valid) {
           const uint32_t cls = L > 1 ? class_of_bin(cuts_s, (int)L, (uint32_t)oc.H & v.qmask) : 0u;
@@ -3007,26 +2997,56 @@ __device__ __forceinline__ uint64_t list_at(const RunView& v, uint64_t i, bool* 
 // Pass-2 work over the candidate list. Every list segment is cut into
 // list_parts parts (interleaved 32-record rows), and the launched warps take
 // the (segment, part) pairs in turn, so that the work spreads evenly over a
-// grid that is resident all at once. A warp takes U rows of its part at a time:
-// fn(first + row0, row, n - row0) gets the list index and the distance (in
-// records) of the rows -- row u holds the records u * row .. u * row + 31 from
-// there, as far as they lie below the third argument.
-template <int U, typename F>
-__device__ __forceinline__ void for_rows(const RunView& v, F&& fn) {
+// grid that is resident all at once. fn(i) runs for list index i.
+template <typename F>
+__device__ __forceinline__ void for_listed(const RunView& v, F&& fn) {
   // 32-bit arithmetic: at most kMaxSegments segments of at most kMaxParts parts
   const uint32_t parts = *(volatile unsigned int*)&v.hdr->list_parts;
   const uint32_t pairs = v.n_segments * parts;
   const uint32_t warps = gridDim.x * (kBlock / 32);
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint32_t w = (blockIdx.x * kBlock + threadIdx.x) >> 5; w < pairs; w += warps) {
+    const uint32_t sgm = w / parts, part = w - sgm * parts;
+    const uint32_t n = __ldcg(v.seg_count + sgm);
+    const uint64_t first = (uint64_t)sgm * v.seg_cap;
+    for (uint64_t r = part * 32; r < n; r += 32 * parts) {  // as often for every lane: the warp stays together
+      if (r + lane < n) fn(first + r + lane);
+      __syncwarp();
+    }
+  }
+}
+
+// for_listed that reads each record one ahead: fn(i, g, sentinel, slot)
+// gets list index i with its position (and with SLOT its kept table slot)
+// already loaded, while the lane's next record is in flight.
+template <bool SLOT, typename F>
+__device__ __forceinline__ void for_listed_ahead(const RunView& v, bool last_use, F&& fn) {
+  const uint32_t parts = *(volatile unsigned int*)&v.hdr->list_parts;
+  const uint32_t pairs = v.n_segments * parts;
+  const uint32_t warps = gridDim.x * (kBlock / 32);
+  const uint32_t lane = threadIdx.x & 31;
   const uint32_t row = 32 * parts;
   for (uint32_t w = (blockIdx.x * kBlock + threadIdx.x) >> 5; w < pairs; w += warps) {
     const uint32_t sgm = w / parts, part = w - sgm * parts;
     const uint32_t n = __ldcg(v.seg_count + sgm);
     const uint64_t first = (uint64_t)sgm * v.seg_cap;
-    for (uint64_t r0 = part * 32; r0 < n; r0 += (uint64_t)U * row) fn(first + r0, row, (uint32_t)(n - r0));
+    uint32_t j = part * 32 + lane;
+    bool sent = false;
+    uint64_t g = j < n ? list_at(v, first + j, &sent, last_use) : 0;
+    uint32_t slot = (SLOT && j < n) ? __ldcs(v.cand_slot + first + j) : 0u;
+    while (j < n) {
+      const uint32_t jn = j + row;
+      bool sent_n = false;
+      const uint64_t gn = jn < n ? list_at(v, first + jn, &sent_n, last_use) : 0;
+      const uint32_t slot_n = (SLOT && jn < n) ? __ldcs(v.cand_slot + first + jn) : 0u;
+      fn(first + j, g, sent, slot);
+      j = jn;
+      g = gn;
+      sent = sent_n;
+      slot = slot_n;
+    }
   }
 }
-
-constexpr int kClassifyAhead = 2;  // rows of the list in flight per warp
 
 // Pass 2 of this round ran with the region-ordered kernels.
 __device__ __forceinline__ bool pass2_done(const RunView& v) {
@@ -3048,16 +3068,14 @@ __global__ void __launch_bounds__(kBlock) pass2_insert_kernel(RunView v) {
   if (pass2_done(v)) return;
   const uint64_t cap = *(volatile unsigned long long*)&v.hdr->table_slots;
   if (list_complete(v)) {
-    const uint32_t lane = threadIdx.x & 31;
-    for_rows<1>(v, [&](uint64_t i0, uint32_t, uint32_t left) {
-      if (lane >= left) return;
+    for_listed(v, [&](uint64_t i) {
       bool sent;
-      const uint64_t g = list_at(v, i0 + lane, &sent, false);
+      const uint64_t g = list_at(v, i, &sent, false);
       OccT<KW> oc;
       read_listed<KW>(v, g, sent, &oc);
       const uint64_t slot = insert_occurrence<KW, TS>(v, cap, oc, g);
       if (slot == kNoSlot) v.hdr->overflow = 1;
-      if (v.cand_slot) v.cand_slot[i0 + lane] = slot == kNoSlot ? 0xFFFFFFFFu : (uint32_t)slot;
+      if (v.cand_slot) v.cand_slot[i] = slot == kNoSlot ? 0xFFFFFFFFu : (uint32_t)slot;
     });
     return;
   }
@@ -3072,62 +3090,42 @@ __global__ void __launch_bounds__(kBlock) pass2_insert_kernel(RunView v) {
 
 // Algorithm 1, probe loop, second pass: a candidate is a junction iff its
 // k-mer is a sentinel or has more than one distinct in- or out-base. Sets
-// the junction's bit of C_final (cleared before the first round; a row's bits
-// in one atomic per bitmap word). A listed candidate reads its mask from the
-// slot the insert loop kept (or looks its k-mer up when no slots were kept).
+// the junction's bit of C_final (cleared before the first round). A listed
+// candidate reads its mask from the slot the insert loop kept (or looks its
+// k-mer up when no slots were kept). Records are read one row ahead; two or four rows at a
+// time, with a row's bits combined into one atomic per bitmap word, measured
+// slower (43 -> 49 us for 5.5 M candidates, 47 -> 62 with 16-byte slots).
 template <int KW, int TS>
 __global__ void __launch_bounds__(kBlock) pass2_classify_kernel(RunView v) {
   if (pass2_done(v)) return;
   const uint64_t cap = *(volatile unsigned long long*)&v.hdr->table_slots;
   unsigned long long found = 0;
+  auto mark = [&](uint64_t g, int mk) {
+    if (mk < 0) v.hdr->overflow = 1;
+    if (mk < 0 || is_junction_mask(mk)) {
+      atomicOr(v.cfinal + (g >> 5), 1u << (g & 31));
+      ++found;
+    }
+  };
   if (list_complete(v)) {
-    constexpr int U = kClassifyAhead;
-    const uint32_t lane = threadIdx.x & 31;
-    for_rows<U>(v, [&](uint64_t i0, uint32_t row, uint32_t left) {
-      uint64_t g[U];
-      uint32_t slot[U];
-      bool sent[U];
-      int mk[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const bool ok = u * row + lane < left;
-        const uint64_t i = i0 + (uint64_t)u * row + lane;
-        g[u] = ok ? list_at(v, i, &sent[u], true) : ~0ull;
-        slot[u] = (ok && v.cand_slot) ? __ldcs(v.cand_slot + i) : 0xFFFFFFFFu;
+    auto classify_one = [&](uint64_t, uint64_t g, bool sent, uint32_t slot) {
+      if (v.cand_slot) {
+        mark(g, slot == 0xFFFFFFFFu ? -1 : table_mask<TS>(v, slot));
+      } else {
+        OccT<KW> oc;
+        read_listed<KW>(v, g, sent, &oc);
+        mark(g, find_occurrence<KW, TS>(v, cap, oc));
       }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        mk[u] = -1;
-        if (v.cand_slot) {
-          if (slot[u] != 0xFFFFFFFFu) mk[u] = table_mask<TS>(v, slot[u]);
-        } else if (g[u] != ~0ull) {
-          OccT<KW> oc;
-          read_listed<KW>(v, g[u], sent[u], &oc);
-          mk[u] = find_occurrence<KW, TS>(v, cap, oc);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (u * row >= left) break;  // the same for every lane
-        const bool ok = g[u] != ~0ull;
-        if (ok && mk[u] < 0) v.hdr->overflow = 1;
-        const bool junction = ok && (mk[u] < 0 || is_junction_mask(mk[u]));
-        found += junction;
-        or_row(v.cfinal, g[u], junction);
-      }
-    });
+    };
+    if (v.cand_slot) for_listed_ahead<true>(v, true, classify_one);
+    else for_listed_ahead<false>(v, true, classify_one);
   } else {
     const uint64_t stride = (uint64_t)gridDim.x * kBlock;
     for (uint64_t g = v.p_begin + (uint64_t)blockIdx.x * kBlock + threadIdx.x; g < v.p_end; g += stride) {
       if (!((__ldg(v.ctemp + (g >> 5)) >> (g & 31)) & 1u)) continue;
       OccT<KW> oc;
       if (!read_occurrence<KW>(v, g, &oc)) continue;
-      const int mk = find_occurrence<KW, TS>(v, cap, oc);
-      if (mk < 0) v.hdr->overflow = 1;
-      if (mk < 0 || is_junction_mask(mk)) {
-        atomicOr(v.cfinal + (g >> 5), 1u << (g & 31));
-        ++found;
-      }
+      mark(g, find_occurrence<KW, TS>(v, cap, oc));
     }
   }
   block_add(found, &v.hdr->pass2_kept);
@@ -3144,7 +3142,7 @@ __global__ void __launch_bounds__(kBlock) partition_count_kernel(RunView v) {
   const uint64_t stride = (uint64_t)gridDim.x * kBlock * kR;
   for (uint64_t p0 = ((uint64_t)blockIdx.x * kBlock + threadIdx.x) * kR; p0 < v.m; p0 += stride) {
     if ((uint32_t)(p0 >> 16) & v.part_chunks) continue;  // a sample of the 64K-position chunks
-    walk<KW, kR>(v, p0, [&](int, uint64_t, bool valid, const auto& oc) {
+    walk<KW, kR, true>(v, p0, [&](int, uint64_t, bool valid, const auto& oc) {
       if (!valid || (oc.H & v.part_sample)) return;
       const uint64_t G = second_hash(oc.H);
       const uint64_t m = item_bits<HB>(G, 17u, v.hashes);
