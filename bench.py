@@ -220,9 +220,20 @@ def kernel_work(name, st, m, n_seqs, table_bytes, rounds=1):
     pos = st["positions"]
     cand = st["pass1_marks"]
     junc = st["pass2_marks"]
-    # the region-ordered first pass: every round reads the class and region planes
+    # the region-ordered passes (class_sort, tile_*, ord_*); ord_scatter and ord_gather model
+    # profiles of the passes over class and region planes, which no kernel reads any more
     if name == "ord_scatter":  # planes + the members' k-mers; an 8 B record and a 2 B rank per member
         return rounds * (2 * m + m / 4) + 10 * pos, "hbm"
+    if name == "class_sort":    # packed read + two bytes of sorted list per position
+        return m / 4 + 2 * m, "hbm"
+    if name == "tile_scatter":  # list entry, packed input, an 8 B record per member
+        return rounds * m / 4 + 10 * pos, "hbm"
+    if name == "tile_gather":   # list entries + decision word pairs; C_temp and C_final words
+        return 2 * pos + pos / 4 + rounds * m / 4, "hbm"
+    if name == "ord_insert2":
+        return cand, "l2_or"        # one table slot per candidate, its region's part in L2
+    if name == "ord_classify2":
+        return cand, "l2_read"
     if name == "ord_or":
         return pos, "l2_or"         # one OR per record into an L2-resident filter region
     if name == "ord_probe":

@@ -70,7 +70,7 @@ typedef struct twopaco_options {
                               0 = automatic. A round sizes its table from an estimate of its
                               distinct candidates, within the reserve; pass 2 on ordered
                               records (ordered_first_pass) uses the whole reserve, one part
-                              per filter region */
+                              per filter region. At least 4 */
   uint64_t candidate_records; /* pass-2 candidate list size in 8-byte units; 0 =
                                  automatic (half a round's positions). It
                                  holds twice as many candidates when the input has
@@ -111,20 +111,22 @@ typedef struct twopaco_options {
                               the batched launch). The call reads the string offsets
                               back and synchronises the stream; twopaco_plan_create
                               refuses it. 0 (default): one launch per loop. */
-  int bucket_inserts;      /* first-pass inserts through region buckets: each OR into the
-                              filter becomes an 8-byte record in the bucket of its filter
-                              region (32 MiB, or a quarter of a smaller filter), and the
-                              records are then applied region by region while each region
-                              sits in L2 -- a filter beyond L2 otherwise takes its random
-                              ORs at DRAM's random-access rate. The workspace holds the
-                              buckets (records for a round's positions and a quarter more,
-                              at most 2^31); the positions go through in chunks that fill
-                              them to about 80%, and a full bucket takes the OR directly.
-                              Same results. 0 (default): for filters of more than 64 MiB
-                              whose chunks put at least 16 ORs on every 32-byte filter
-                              sector on average (sparser, the regions' cold misses cost
-                              more than direct ORs); 1: for any filter; 2: never. Needs
-                              hashes <= 6 and a filter of at most 2^38 bits (else the ORs
+  int bucket_inserts;      /* one-round runs with a filter beyond L2, which takes random ORs
+                              and probes at DRAM's random-access rate. 0 (default): such a run
+                              (k <= 63, hashes <= 6) takes the passes in filter-region order
+                              that ordered_first_pass describes, in its one round, for filters
+                              of more than 64 MiB with at least 4 positions per 32-byte filter
+                              sector; 1: for any filter; 2: never. Where those passes do not go
+                              (k > 63, per_string_launches, ordered_first_pass = 2) the ORs
+                              alone go through region buckets: each becomes an 8-byte record
+                              in the bucket of its filter region (32 MiB, or a quarter of a
+                              smaller filter), and the records are applied region by region
+                              while each region sits in L2; the positions go through in chunks
+                              that fill the buckets (records for a round's positions and a
+                              quarter more, at most 2^31) to about 80%, and a full bucket
+                              takes the OR directly -- 0: from 16 ORs of a chunk per filter
+                              sector on; 1: for any filter; 2: never. Same results. Buckets
+                              need hashes <= 6 and a filter of at most 2^38 bits (else the ORs
                               are direct). */
   int launch_blocks_per_sm; /* launch shape of the pass kernels (insert, probe, pass-2
                               insert and classify): at most this many resident blocks of
@@ -132,26 +134,32 @@ typedef struct twopaco_options {
                               many as fit. Same results (every loop strides over its
                               work); a latency-bound kernel can gain from fewer blocks
                               contending for L2. */
-  int ordered_first_pass;  /* the first pass of a class-map run (rounds 2..64, k <= 63,
-                              hashes <= 6) in filter-region order: every position of a
-                              round's class becomes an 8-byte record in the bucket of its
-                              k-mer's filter region (at most 32 MiB, which L2 holds); the
-                              ORs and then the probes are applied bucket by bucket, and the
-                              decisions are gathered back in position order. A filter
-                              beyond L2 otherwise takes every OR and probe at DRAM's
-                              random-access rate. For k <= 27 (and partial 0) pass 2 runs
-                              on the same records: the table reserve (table_slots) is split
-                              into one part per filter region, each candidate's edges are
-                              inserted while its region is in L2, and a lookup per
-                              candidate record decides the junctions -- no candidate list
-                              and no table sizing per round; a part that fills up reports
-                              TWOPACO_EOVERFLOW (twopaco_build and twopaco_build_ctx grow
-                              the reserve and run again). The workspace holds a region byte
-                              per position and records for a round's positions and a
-                              quarter more (the candidate list shares their room); a round
-                              with more positions takes the direct kernels. Same results.
-                              0 (default): for filters of 1 GiB (2^33 bits) and more; 1:
-                              for any filter; 2: never. Not with per_string_launches. */
+  int ordered_first_pass;  /* the passes of a run of 2..64 rounds (k <= 63, hashes <= 6) in
+                              filter-region order: the positions of every 16384-position tile
+                              are sorted once by class and filter region (up to 256 regions
+                              of at most 32 MiB, which L2 holds); every position of a round's
+                              class then becomes an 8-byte record in the bucket of its
+                              k-mer's region, the ORs and then the probes are applied bucket
+                              by bucket, and the decisions are gathered back in position
+                              order. A filter beyond L2 otherwise takes every OR and probe at
+                              DRAM's random-access rate. For k <= 31 (and partial 0) pass 2
+                              runs on the same records: the table reserve (table_slots) is
+                              split into one part per filter region, each candidate is
+                              inserted while its region is in L2, and a lookup per candidate
+                              record decides the junctions -- no candidate list and no table
+                              sizing per round; a part that fills up reports
+                              TWOPACO_EOVERFLOW (twopaco_build and twopaco_build_ctx grow the
+                              reserve and run again). For longer k-mers a round whose table
+                              is far beyond L2 also splits it by region, where the reserve has
+                              room for the split. The workspace holds two bytes per position
+                              and records for a round's positions and a quarter more (the
+                              candidate list shares their room); a round with more positions
+                              takes the direct kernels. Same results. 0 (default): for
+                              filters of 1 GiB (2^33 bits) and more, and for filters of more
+                              than 64 MiB with at least 4 of a round's positions per 32-byte
+                              filter sector; 1: for any filter; 2: never (a one-round run
+                              then keeps to bucket_inserts' buckets). Not with
+                              per_string_launches. */
 } twopaco_options;
 
 /* Counters of one run, in the spirit of Table 4 (marks after each pass). */
@@ -168,7 +176,7 @@ typedef struct twopaco_stats {
                               output again into a larger buffer */
   uint32_t timeout;        /* nonzero: a bounded device wait gave up */
   uint32_t ordered_rounds; /* rounds whose first pass ran in filter-region order
-                              (options->ordered_first_pass) */
+                              (options->ordered_first_pass, bucket_inserts) */
   uint32_t pad;
 } twopaco_stats;
 

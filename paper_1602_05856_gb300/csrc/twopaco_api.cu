@@ -161,13 +161,13 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
     // as many regions as a byte can number, so that a region, the next one (read
     // ahead) and a part of the table are well inside L2, of at most 2^22 words (32
     // MiB) each; fewer where the counters of many rounds, or table parts of at least
-    // 256 slots (k <= 31), want it
+    // 1024 slots (k <= 31), want it
     const uint64_t r_min = std::max<uint64_t>(1, fwords >> kRegionWordsLog2);
     uint64_t R = std::max<uint64_t>(r_min, std::min<uint64_t>(kOrdMaxRegions, fwords));
     // (k <= 31: regions of whole blocks of four words, so that they are the top bits of H)
     if (k <= 31 && !o.partial && fwords / 4 >= 64) R = std::min(R, fwords / 4);
     while (R > r_min && R * (uint64_t)rounds > kOrdMaxHist) R /= 2;
-    while (R > r_min && k <= 31 && !o.partial && L.table_slots / R < 256) R /= 2;
+    while (R > r_min && k <= 31 && !o.partial && L.table_slots / R < 1024) R /= 2;
     const uint64_t rw = fwords / R;
     const bool auto_rounds = filter_bits / 8 >= (1ull << 30) || dense;
     const bool want = rounds > 1 ? o.ordered_first_pass == 1 || (o.ordered_first_pass == 0 && auto_rounds)
@@ -185,10 +185,10 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
       L.o_tiles = (m + kOrdTile - 1) / kOrdTile;
       // pass 2 on the records too (one-word k-mers, k <= 31, whose hash the bucket and
       // 58 bits give back): the table reserve split into one part of one-word slots
-      // per region, at least 256 each (half full, more than eight standard deviations
-      // of a part's k-mers fit)
+      // per region, at least 1024 each (a part's share of the k-mers varies by its
+      // square root)
       const uint64_t tcap = L.table_slots / R;
-      if (k <= 31 && !o.partial && R >= 64 && tcap >= 256 && tcap < (1ull << 32)) {
+      if (k <= 31 && !o.partial && R >= 64 && tcap >= 1024 && tcap < (1ull << 32)) {
         L.o_fused = 1;
         L.o_tcap = (uint32_t)tcap;
       }

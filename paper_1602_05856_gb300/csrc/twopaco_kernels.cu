@@ -3804,7 +3804,7 @@ static int ordered_round_impl(const RunView& v, int round, cudaStream_t s, RunVi
     ord_setup_kernel<<<1, kBlock, 0, s>>>(v, round);
   }
   {
-    Timed t("ord_scatter", s);
+    Timed t("tile_scatter", s);
     auto kern = ord_scatter_kernel<KW, HB, false>;
     if constexpr (KW == 1)
       if (fused) kern = ord_scatter_kernel<KW, HB, true>;
@@ -3860,7 +3860,7 @@ static int ordered_round_impl(const RunView& v, int round, cudaStream_t s, RunVi
     }
   }
   {
-    Timed t("ord_gather", s);
+    Timed t("tile_gather", s);
     ord_gather_kernel<<<grid, kBlock, 0, s>>>(*pv, round);
   }
   return launched + 1;
@@ -4037,7 +4037,7 @@ int TWOPACO_PART_NAME(launch_count_, TWOPACO_PART)(const RunView& v, cudaStream_
 #if TWOPACO_PART == 1 || TWOPACO_PART == 3 || TWOPACO_PART == 5
 // The class map of this k-mer width.
 int TWOPACO_PART_NAME(launch_map_, TWOPACO_PART)(const RunView& v, cudaStream_t s) {
-  Timed t("class_map", s);
+  Timed t(v.o_regions ? "class_sort" : "class_map", s);
   if constexpr (kPartKw < 4) {
     if (v.o_regions) {  // the sorted tiles instead
       auto kern = class_sort_kernel<kPartKw>;
