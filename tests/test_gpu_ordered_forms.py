@@ -57,7 +57,8 @@ FORMS = [  # k, filter bits, hashes, rounds, options: widths of k-mer words and 
     (31, 1 << 18, 4, 1, {"split_at_n": True}), (32, 1 << 20, 4, 1, {}), (33, 1 << 18, 5, 2, {"split_at_n": True}),
     (62, 1 << 20, 1, 1, {}), (63, 1 << 18, 4, 1, {"partial": True}), (25, 1 << 20, 4, 64, {}),
     (24, 1 << 18, 4, 16, {"split_at_n": True}), (31, 1 << 20, 4, 1, {"partial": True}),
-    (25, 1 << 20, 4, 1, {"table_slots": 1 << 12, "candidate_records": 600}),  # pass 2 over C_temp
+    # a table with room for fewer than 64 parts: the candidate list, which overflows: pass 2 over C_temp
+    (25, 1 << 21, 4, 1, {"table_slots": 1 << 15, "candidate_records": 600}),
 ]
 
 
