@@ -3640,12 +3640,6 @@ __global__ void __launch_bounds__(kBlock) edges_kernel(const DevHeader* hdr, con
 // Launch helpers
 // ---------------------------------------------------------------------------
 
-int sm_count(int dev) {
-  int n = 0;
-  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-  return n > 0 ? n : 1;
-}
-
 // SMs and resident blocks per SM of a kernel: asked for once per kernel and
 // device (three runtime calls before every launch cost more host time than the
 // launch). Packed as SMs << 32 | blocks; devices past the table ask every time.
@@ -3678,10 +3672,12 @@ uint64_t resident_blocks(K kernel, int block, size_t dyn_smem) {
       }
     }
   }
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, dyn_smem);
-  const uint64_t v = ((uint64_t)sm_count(dev) << 32) | (uint32_t)std::max(per_sm, 1);
-  if (at) at->value.store(v, std::memory_order_release);  // the same from any thread
+  int per_sm = 0, sms = 0;
+  const bool known_now =
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, dyn_smem) == cudaSuccess &&
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && per_sm > 0 && sms > 0;
+  const uint64_t v = ((uint64_t)std::max(sms, 1) << 32) | (uint32_t)std::max(per_sm, 1);
+  if (at && known_now) at->value.store(v, std::memory_order_release);  // the same from any thread
   return v;
 }
 
