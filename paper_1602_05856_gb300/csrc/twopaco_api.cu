@@ -186,9 +186,11 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
       // pass 2 on the records too (one-word k-mers, k <= 31, whose hash the bucket and
       // 58 bits give back): the table reserve split into one part of one-word slots
       // per region, at least 1024 each (a part's share of the k-mers varies by its
-      // square root)
+      // square root). Regions of whole blocks only: a smaller one is named by bits of
+      // the second hash too, and two bits of H would be neither in the record nor in
+      // its bucket (filters of 2^12 and 2^13 bits)
       const uint64_t tcap = L.table_slots / R;
-      if (k <= 31 && !o.partial && R >= 64 && tcap >= 1024 && tcap < (1ull << 32)) {
+      if (k <= 31 && !o.partial && R >= 64 && rw >= 4 && tcap >= 1024 && tcap < (1ull << 32)) {
         L.o_fused = 1;
         L.o_tcap = (uint32_t)tcap;
       }

@@ -2082,7 +2082,8 @@ __device__ __forceinline__ FusedOcc fused_occ(unsigned long long rec, uint64_t t
   return o;
 }
 
-// Buckets are the top bits of H: R regions, a power of two of at least 64.
+// Buckets are the top bits of H: R regions, a power of two of at least 64, each of
+// whole filter blocks (four words or more).
 __device__ __forceinline__ int fused_low_bits(const RunView& v) { return 64 - (31 - __clz(v.o_regions)); }
 
 // The fused pass-2 table: bucket b owns the o_tcap one-word slots from b *
