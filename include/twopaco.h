@@ -116,8 +116,10 @@ typedef struct twopaco_options {
                               (k <= 63, hashes <= 6) takes the passes in filter-region order
                               that ordered_first_pass describes, in its one round, for filters
                               of more than 64 MiB with at least 4 positions per 32-byte filter
-                              sector; 1: for any filter; 2: never. Where those passes do not go
-                              (k > 63, per_string_launches, ordered_first_pass = 2) the ORs
+                              sector; 1: for any filter; 2: never; in either case only where
+                              the workspace is at most 8 GiB larger for it. Where those passes
+                              do not go (k > 63, per_string_launches, ordered_first_pass = 2,
+                              the workspace) the ORs
                               alone go through region buckets: each becomes an 8-byte record
                               in the bucket of its filter region (32 MiB, or a quarter of a
                               smaller filter), and the records are applied region by region
@@ -157,9 +159,9 @@ typedef struct twopaco_options {
                               takes the direct kernels. Same results. 0 (default): for
                               filters of 1 GiB (2^33 bits) and more, and for filters of more
                               than 64 MiB with at least 4 of a round's positions per 32-byte
-                              filter sector; 1: for any filter; 2: never (a one-round run
-                              then keeps to bucket_inserts' buckets). Not with
-                              per_string_launches. */
+                              filter sector if the workspace is at most 8 GiB larger for it;
+                              1: for any filter; 2: never (a one-round run then keeps to
+                              bucket_inserts' buckets). Not with per_string_launches. */
 } twopaco_options;
 
 /* Counters of one run, in the spirit of Table 4 (marks after each pass). */

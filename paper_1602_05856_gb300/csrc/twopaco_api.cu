@@ -16,6 +16,7 @@ namespace {
 
 constexpr uint64_t kAlign = 256;
 constexpr uint64_t kStreamChunkMin = 64 << 10;  // bytes per staging half, at least
+constexpr uint64_t kOrdExtraBytes = 8ull << 30;  // automatic ordered passes: workspace over the direct passes', at most
 
 uint64_t align_up(uint64_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
@@ -297,6 +298,19 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
     at += align_up((L.run_cap + 1) * 4);
   }
   L.total = at;
+  // The ordered passes hold 10 bytes of records per position of a round and 2 of lists
+  // per position; the passes they stand in for hold at most 2^31 records, and at 2^31
+  // bases and more no descriptors. So where they are not asked for by name (and not the
+  // rule of filters of 1 GiB and more in several rounds) they may cost kOrdExtraBytes
+  // over the direct passes and no more: one round of 24 G bases with a 2^36-bit filter
+  // takes 89 GB direct and would take 387, more than the GPU has.
+  const bool bounded = rounds == 1 || (o.ordered_first_pass == 0 && filter_bits / 8 < (1ull << 30));
+  if (L.o_regions && bounded) {
+    twopaco_options direct = o;
+    direct.ordered_first_pass = 2;
+    const Layout D = layout(m, n_seqs, k, filter_bits, rounds, direct);
+    if (L.total > D.total + kOrdExtraBytes) return D;
+  }
   return L;
 }
 
