@@ -168,6 +168,10 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
     // (k <= 31: regions of whole blocks of four words, so that they are the top bits of H)
     if (k <= 31 && !o.partial && fwords / 4 >= 64) R = std::min(R, fwords / 4);
     while (R > r_min && R * (uint64_t)rounds > kOrdMaxHist) R /= 2;
+    // (a filter inside L2 gains nothing from more than 64 of them, and their offsets and
+    // rooms, 2 rounds + 4 bytes per region and tile, are workspace: asked for there by
+    // name, in many rounds, they took what fits the allocation-free run's 32 MiB out of it)
+    while (!beyond_l2 && R > std::max<uint64_t>(r_min, 64) && R * (uint64_t)rounds > 1024) R /= 2;
     while (R > r_min && k <= 31 && !o.partial && L.table_slots / R < 1024) R /= 2;
     const uint64_t rw = fwords / R;
     const bool auto_rounds = filter_bits / 8 >= (1ull << 30) || dense;

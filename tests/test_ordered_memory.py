@@ -52,3 +52,13 @@ def test_sizes_within_the_bound_stay_ordered():
         assert _ws(m, 1 << lg, rounds, k=k) != _ws(m, 1 << lg, rounds, k=k, ordered_first_pass=2)
     # several rounds with a filter of 1 GiB and more: the rule there was, whatever it asks for
     assert _ws(24_000_000_000, 1 << 36, 4) == _ws(24_000_000_000, 1 << 36, 4, ordered_first_pass=1)
+
+
+@pytest.mark.parametrize("m,k,lg,rounds,kw", [
+    (6_450_000, 15, 17, 16, {}), (8_780_000, 63, 18, 12, dict(partial=True)),
+    (6_060_000, 31, 22, 24, dict(split_at_n=True)), (8_940_000, 25, 16, 64, dict(table_slots=1 << 18)),
+    (5_880_000, 45, 23, 7, dict(table_slots=1 << 16)),
+])
+def test_asked_for_by_name_the_small_runs_fit_the_allocation_free_scratch(m, k, lg, rounds, kw):
+    """Runs just within the 32 MiB with 64 regions, a class byte and a region byte per position."""
+    assert _ws(m, 1 << lg, rounds, k=k, ordered_first_pass=1, **kw) <= 32 << 20
