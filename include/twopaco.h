@@ -149,11 +149,13 @@ typedef struct twopaco_options {
                               split into one part per filter region, each candidate is
                               inserted while its region is in L2, and a lookup per candidate
                               record decides the junctions -- no candidate list and no table
-                              sizing per round; a part that fills up reports
-                              TWOPACO_EOVERFLOW (twopaco_build and twopaco_build_ctx grow the
-                              reserve and run again). For longer k-mers a round whose table
-                              is far beyond L2 also splits it by region, where the reserve has
-                              room for the split. The workspace holds two bytes per position
+                              sizing per round; a round with a part that fills up takes the
+                              list and one table of the whole reserve instead, which reports
+                              TWOPACO_EOVERFLOW if it fills up too (twopaco_build and
+                              twopaco_build_ctx then grow the reserve and run again). For
+                              longer k-mers a round whose table is far beyond L2 also splits
+                              it by region, where the reserve has room for the split. The
+                              workspace holds two bytes per position
                               and records for a round's positions and a quarter more (the
                               candidate list shares their room); a round with more positions
                               takes the direct kernels. Same results. 0 (default): for

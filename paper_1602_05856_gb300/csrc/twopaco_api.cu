@@ -415,6 +415,7 @@ RunView make_view(const uint8_t* d_bases, const uint64_t* d_offsets, uint64_t n_
     // about 4096 members per work item
     v.o_item_tiles = (uint32_t)std::max<uint64_t>(8, (uint64_t)L.o_regions * rounds / (kOrdTile / 4096));
     v.o_tcap = L.o_tcap;
+    v.o_chain = std::min(L.o_tcap, kFusedChain);
   }
   v.tile_count = reinterpret_cast<uint32_t*>(base + L.tile_count);
   v.tile_prefix = reinterpret_cast<uint64_t*>(base + L.tile_prefix);

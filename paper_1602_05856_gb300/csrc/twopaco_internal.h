@@ -22,7 +22,7 @@ struct DevHeader {
   unsigned long long part_slots;   // region-ordered pass 2 by buckets: table slots per region (0: not this round)
   unsigned int cand_overflow;      // a warp's list segment ran out of room this round
   unsigned int round_listed;       // pass 2 of this round reads the list (else C_temp)
-  unsigned int reserved;
+  unsigned int part_full;          // pass 2 on the records: a part of this round's table filled up
   unsigned int list_parts;         // pass-2 parts per list segment this round
   unsigned long long emit_ticket;  // next emit tile to claim
   unsigned int overflow;           // the pass-2 table or a boundary list out of room
@@ -138,6 +138,7 @@ struct RunView {
   int o_bucketed;           // 32 <= k <= 63, not partial: pass 2 bucket by bucket, through the lists
   uint32_t o_item_tiles;    // tiles per work item of its insert loop
   int o_fused;              // k <= 31, not partial: pass 2 runs on the records (fused records)
+  uint32_t o_chain;         // fused: slots an insert tries before its part counts as full
   uint32_t o_tcap;          // fused: table slots per bucket (region), the table is o_regions x o_tcap slots
   int use_desc;             // the insert leaves descriptors and the probe reads them
   uint64_t cand_cap;        // records the list can hold
@@ -175,6 +176,7 @@ constexpr uint64_t kOrdTile = 16384;       // region-ordered first pass: positio
 constexpr uint32_t kOrdMaxRegions = 256;   // buckets (filter regions), at most
 constexpr uint32_t kOrdMaxHist = 4096;     // rounds x regions, at most
 constexpr uint32_t kOrdFillStride = 32;    // bucket fill counters 128 bytes apart
+constexpr uint32_t kFusedChain = 4096;     // pass 2 on the records: slots an insert tries, at most
 constexpr uint32_t kOrdScanTiles = 64;     // tiles per block of the scans over tiles
 
 // Kernel launch helpers (twopaco_kernels.cu). Each returns the number of

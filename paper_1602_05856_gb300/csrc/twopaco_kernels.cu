@@ -1911,6 +1911,11 @@ __device__ __forceinline__ bool ordered_round(const RunView& v) {
   return v.o_regions && *reinterpret_cast<volatile const unsigned int*>(&v.hdr->ord_ok);
 }
 
+// Pass 2 of this (ordered) round runs on its records: no part of the table filled up.
+__device__ __forceinline__ bool fused_pass2(const RunView& v) {
+  return v.o_fused && !*reinterpret_cast<volatile const unsigned int*>(&v.hdr->part_full);
+}
+
 // Algorithm 1, insert loop, first pass, over this round's class only.
 template <int KW, int HB, bool BKT = false>
 __global__ void __launch_bounds__(kBlock) pass1_insert_cm_kernel(RunView v, int round) {
@@ -2095,7 +2100,11 @@ __device__ __forceinline__ int fused_low_bits(const RunView& v) { return 64 - (3
 // o_tcap (Lemire's multiply-high) and probes linearly within the part. Slot by slot,
 // unlike the direct table: the whole reserve is the table, at a load of a few
 // percent, so that the first slot mostly decides (a sector at a time took the
-// probe of 6 Gbp from 7.6 to 11.4 ps per position).
+// probe of 6 Gbp from 7.6 to 11.4 ps per position). A part counts as full when a
+// k-mer finds no slot in kFusedChain steps (o_chain: in the whole of a smaller part): at
+// a load of 0.9 the longest run of taken slots in a million is about 2600. A full part
+// (its share of the k-mers varies, and a tight reserve has no room for that) is no error:
+// the round's pass 2 then goes over the candidate list and one table of the whole reserve.
 __device__ __forceinline__ bool fused_table_insert(const RunView& v, uint32_t b, const FusedOcc& o,
                                                    uint64_t low_mask) {
   const uint32_t cap = v.o_tcap;
@@ -2103,7 +2112,7 @@ __device__ __forceinline__ bool fused_table_insert(const RunView& v, uint32_t b,
   const bool junction = o.sentinel || o.j1 != o.j2;
   const unsigned long long mine = ((o.H & low_mask) << 5) | ((o.j1 & 15u) << 1) | (junction ? 1u : 0u);
   uint32_t i = __umulhi((uint32_t)(o.H >> 16), cap);
-  for (uint32_t probe = 0; probe < cap; ++probe, i = i + 1 == cap ? 0u : i + 1) {
+  for (uint32_t probe = 0; probe < v.o_chain; ++probe, i = i + 1 == cap ? 0u : i + 1) {
     unsigned long long cur = __ldcg(T + i);
     if (cur == kEmpty) {
       cur = atomicCAS(T + i, kEmpty, mine);
@@ -2122,7 +2131,7 @@ __device__ __forceinline__ int fused_table_find(const RunView& v, uint32_t b, ui
   const unsigned long long* T = static_cast<const unsigned long long*>(v.table) + (uint64_t)b * cap;
   const uint64_t key = H & low_mask;
   uint32_t i = __umulhi((uint32_t)(H >> 16), cap);
-  for (uint32_t probe = 0; probe < cap; ++probe, i = i + 1 == cap ? 0u : i + 1) {
+  for (uint32_t probe = 0; probe < kFusedChain; ++probe, i = i + 1 == cap ? 0u : i + 1) {
     const unsigned long long cur = __ldcg(T + i);
     if (cur == kEmpty) return -1;
     if ((cur >> 5) == key) return (int)(cur & 1u);
@@ -2241,6 +2250,7 @@ __global__ void __launch_bounds__(kBlock) ord_setup_kernel(RunView v, int round)
     v.hdr->ord_ticket[2] = 0;
     v.hdr->ord_ticket[3] = 0;
     v.hdr->part_slots = 0;
+    v.hdr->part_full = 0;
     v.hdr->cand_overflow = 0;  // the gather of the round before may have set it after its table_setup
   }
 }
@@ -2412,11 +2422,12 @@ __global__ void __launch_bounds__(kBlock) ord_or_kernel(RunView v) {
 // bit; the linear-counting bit of every candidate is set from the k-mer's
 // filter word index and bit bases. FUSED: instead, every candidate inserts
 // its in/out bases into its region's part of the pass-2 table (Algorithm 1's
-// insert loop, second pass) while the region is in L2.
+// insert loop, second pass) while the region is in L2, until a part fills up.
 template <int HB, bool FUSED>
 __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
   __shared__ uint32_t first_s[kOrdMaxRegions + 1];
   __shared__ uint32_t item_s;
+  __shared__ bool insert_s;
   if (!ordered_round(v)) return;
   ord_items(v, first_s);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -2424,8 +2435,10 @@ __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
   uint32_t kept = 0;
   for (;;) {
     if (threadIdx.x == 0) item_s = atomicAdd(&v.hdr->ord_ticket[1], 1u);
+    if (FUSED && threadIdx.x == 32) insert_s = fused_pass2(v);  // beside the ticket's round trip
     __syncthreads();
     const uint32_t item = item_s;
+    const bool insert = FUSED && insert_s;
     __syncthreads();
     if (item >= total) break;
     const uint32_t b = ord_item_bucket(first_s, R, item);
@@ -2468,7 +2481,7 @@ __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
             const FusedOcc o = fused_occ(rec[u], top, low_mask);
             const uint32_t pres = present_items<HB>(o.G, word[u], v.hashes);
             keep = o.sentinel || (pres >> 16) || __popc(pres & 0xFFFFu) >= 2;
-            if (keep && !fused_table_insert(v, b, o, low_mask)) v.hdr->overflow = 1;
+            if (keep && insert && !fused_table_insert(v, b, o, low_mask)) v.hdr->part_full = 1;
           } else {
             const uint64_t G = ((rec[u] >> 22) & 0x3FFFFFFFull) << 32;
             const uint32_t pres = present_items<HB>(G, word[u], v.hashes);
@@ -2488,7 +2501,7 @@ __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
       }
     }
   }
-  if (!FUSED && !v.partial) block_add((unsigned long long)kept, &v.hdr->round_kept);  // sizes the table
+  if (!v.partial) block_add((unsigned long long)kept, &v.hdr->round_kept);  // sizes the table and its work
 }
 
 // Algorithm 1, probe loop, second pass, on fused records, bucket by bucket:
@@ -2498,7 +2511,7 @@ __global__ void __launch_bounds__(kBlock) ord_probe_kernel(RunView v) {
 __global__ void __launch_bounds__(kBlock, 8) ord_classify_kernel(RunView v) {
   __shared__ uint32_t first_s[kOrdMaxRegions + 1];
   __shared__ uint32_t item_s;
-  if (!ordered_round(v)) return;
+  if (!ordered_round(v) || !fused_pass2(v)) return;
   ord_items(v, first_s);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint32_t R = v.o_regions, total = first_s[R];
@@ -2766,7 +2779,7 @@ __global__ void __launch_bounds__(kBlock) ord_gather_kernel(RunView v, int round
   for (uint32_t b = threadIdx.x; b < v.o_regions; b += kBlock) start_s[b] = v.o_start[b];
   for (uint32_t i = threadIdx.x; i < kOrdTileWords; i += kBlock) keep_s[i] = jun_s[i] = sent_s[i] = 0;
   // the junctions are known: pass 2 ran on the records or bucket by bucket
-  const bool decided = v.o_fused || __ldcg(&v.hdr->part_slots) != 0;
+  const bool decided = fused_pass2(v) || __ldcg(&v.hdr->part_slots) != 0;
   const bool listed = !decided && !v.partial;
   TileOut o{0, 0, 0};
   unsigned long long valid_n = 0;
@@ -2884,7 +2897,8 @@ template <int TS>
 __global__ void __launch_bounds__(1024) table_setup_kernel(RunView v) {
   __shared__ unsigned int part[32];
   DevHeader* h = v.hdr;
-  if (v.o_fused && ordered_round(v)) {  // the round's table was the fused one: nothing to size or clear
+  const bool parted = v.o_fused && ordered_round(v);  // the probe inserted into the table's parts
+  if (parted && fused_pass2(v)) {  // that was the round's table: nothing to size or clear
     if (threadIdx.x == 0) {
       const unsigned long long used = (unsigned long long)v.o_tcap * v.o_regions;
       h->cand_overflow = 0;
@@ -2942,7 +2956,8 @@ __global__ void __launch_bounds__(1024) table_setup_kernel(RunView v) {
       cap = part * v.o_regions;
     }
   }
-  if (cap > v.table_max_slots) cap = v.table_max_slots;
+  // (no estimate in a round whose probe inserted; a part that filled up asks for all there is)
+  if (parted || cap > v.table_max_slots) cap = v.table_max_slots;
   h->table_slots = cap;
   if (cap > h->table_max) h->table_max = cap;
   h->round_listed = overflowed ? 0u : 1u;
@@ -3045,7 +3060,7 @@ __device__ __forceinline__ void for_listed_ahead(const RunView& v, bool last_use
 
 // Pass 2 of this round ran with the region-ordered kernels.
 __device__ __forceinline__ bool pass2_done(const RunView& v) {
-  return ordered_round(v) && (v.o_fused || __ldcg(&v.hdr->part_slots) != 0);
+  return ordered_round(v) && (fused_pass2(v) || __ldcg(&v.hdr->part_slots) != 0);
 }
 
 // Pass 2 reads the list: every candidate of the round is in it (a region-ordered

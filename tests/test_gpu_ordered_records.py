@@ -66,3 +66,48 @@ def test_filters_smaller_than_64_blocks(lg_bits, rounds, strings):
         words = b.state(T().STATE_CANDIDATES, (m + 31) // 32)
         assert np.array_equal(np.unpackbits(words.view(np.uint8), bitorder="little")[:m], marks)
         assert sb["pass1_marks"] == kept
+
+
+def _full_parts(k, rounds, seed=5):
+    """Distinct k-mers, all of them candidates of a saturated filter: 250 to 260 thousand a
+    round, which 2^18 slots hold but 256 parts of 1024 do not (a part's share of them has a
+    standard deviation of 31)."""
+    n = 259_000 if rounds == 1 else 500_000
+    return G.concat(G.random_strings(seed, 1, n, n) + [np.frombuffer(b"ACGT" * 40, np.uint8)])
+
+
+@pytest.mark.parametrize("k,rounds,extra", [
+    (25, 1, {}), (31, 1, {}), (25, 2, {}), (30, 2, {}), (27, 1, {"wide_layout": 1}),
+    (31, 1, {"wide_layout": 2}), (24, 1, {"candidate_records": 5000}), (25, 1, {"both_strands": False}),
+])
+def test_a_full_part_of_the_table_takes_one_table(k, rounds, extra):
+    bases, off = _full_parts(k, rounds)
+    base = dict(hashes=4, partition_bins=256, table_slots=1 << 18, **extra)
+    run = T().DeviceBuild(bases, off, k, 1 << 16, rounds,
+                          T().Options(bucket_inserts=1, ordered_first_pass=int(rounds > 1), **base))
+    want = O.junctions((bases, off), k, both_strands=extra.get("both_strands", True))
+    for again in range(3):  # launched twice, then replayed
+        if again == 2:
+            run.capture()
+        run.run()
+        st = run.stats()
+        assert st["ordered_rounds"] == rounds and st["table_slots"] == 1 << 18
+        assert st["positions"] == st["pass1_marks"]  # saturated: the parts are as full as they get
+        assert st["pass2_marks"] == sum(len(w) for w in want)
+        _eq(run.result(), want)
+    run.release_plan()
+
+
+def test_a_full_reserve_is_reported_and_recovered():
+    """Half the slots: the parts fill up and the one table too. The run says so, and the host
+    build grows the reserve and runs again, on the records."""
+    bases, off = _full_parts(25, 1)
+    opts = T().Options(hashes=4, bucket_inserts=1, table_slots=1 << 17)
+    run = T().DeviceBuild(bases, off, 25, 1 << 16, 1, opts)
+    run.run()
+    st = run.stats(check=False)
+    assert st["rc"] == T().EOVERFLOW and st["overflow"] and st["ordered_rounds"] == 1
+    seqs = [bases[int(off[t]):int(off[t + 1])] for t in range(len(off) - 1)]
+    got, st = T().twopaco_build_ex(seqs, 25, 1 << 16, 1, opts)
+    _eq(got, O.junctions((bases, off), 25))
+    assert st["table_slots"] == 1 << 19 and st["ordered_rounds"] == 1
