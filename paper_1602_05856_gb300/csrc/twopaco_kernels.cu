@@ -902,12 +902,12 @@ struct SectorOf {
 };
 
 // Insert into the one-word slots T[0 .. cap), probing from the sector at i (a
-// multiple of 4 below cap): the key's slot, or kNoSlot if every slot was tried
-// (the table is full). Bits already present are not written again. A word is
-// key << 9 | mask bits; never all ones for a key < 2^54.
+// multiple of 4 below cap): the key's slot, or kNoSlot if `tries` slots were tried
+// (all of them: the table is full). Bits already present are not written again. A
+// word is key << 9 | mask bits; never all ones for a key < 2^54.
 __device__ __forceinline__ uint64_t word_insert(unsigned long long* T, uint64_t cap, uint64_t i, uint64_t key,
-                                                uint32_t bits) {
-  for (uint64_t seen = 0; seen < cap; seen += 4) {
+                                                uint32_t bits, uint64_t tries) {
+  for (uint64_t seen = 0; seen < tries; seen += 4) {
     SectorOf<0> q;
     q.load(T, i);
     for (;;) {  // again only after another k-mer took the empty slot
@@ -959,17 +959,17 @@ __device__ __forceinline__ int word_find(const unsigned long long* T, uint64_t c
 
 // Insert (key, bits) into a table of cap TS-kind slots (table_slot_kind),
 // probing from the sector at start (below cap); the key's slot, or kNoSlot if
-// every slot was tried (the table is full). Bits already present are not
-// written again.
+// `tries` slots were tried (all of them: the table is full). Bits already present
+// are not written again.
 template <int TS>
 __device__ __forceinline__ uint64_t table_insert(const RunView& v, uint64_t cap, const Key& key,
-                                             uint64_t start, uint32_t bits) {
+                                             uint64_t start, uint32_t bits, uint64_t tries) {
   if constexpr (TS == 0) {
-    return word_insert(static_cast<unsigned long long*>(v.table), cap, start, key.lo, bits);
+    return word_insert(static_cast<unsigned long long*>(v.table), cap, start, key.lo, bits, tries);
   } else {
     constexpr uint64_t N = SectorOf<TS>::kSlots;
     uint64_t base = start;
-    for (uint64_t seen = 0; seen < cap; seen += N) {
+    for (uint64_t seen = 0; seen < tries; seen += N) {
       SectorOf<TS> q;
       if constexpr (TS == 1) q.load(v.table, base);  // TS 2: the CAS itself is the first look
 #pragma unroll
@@ -1091,12 +1091,19 @@ __device__ __forceinline__ int table_find_ref(const RunView& v, uint64_t cap, co
   return -1;
 }
 
-// The table slot of an occurrence at g (inserted), or its mask (found).
+// The table slot of an occurrence at g (inserted; after at most `tries` slots), or its
+// mask (found).
+template <int KW, int TS>
+__device__ __forceinline__ uint64_t insert_occurrence(const RunView& v, uint64_t cap, const OccT<KW>& oc,
+                                                      uint64_t g, uint64_t tries) {
+  if constexpr (TS == 3) return table_insert_ref(v, cap, oc.key, oc.H, slot_start<4>(oc.H, cap), oc.tbits, g, oc.rc);
+  else return table_insert<TS>(v, cap, oc.key, slot_start<SectorOf<TS>::kSlots>(oc.H, cap), oc.tbits, tries);
+}
+
 template <int KW, int TS>
 __device__ __forceinline__ uint64_t insert_occurrence(const RunView& v, uint64_t cap, const OccT<KW>& oc,
                                                       uint64_t g) {
-  if constexpr (TS == 3) return table_insert_ref(v, cap, oc.key, oc.H, slot_start<4>(oc.H, cap), oc.tbits, g, oc.rc);
-  else return table_insert<TS>(v, cap, oc.key, slot_start<SectorOf<TS>::kSlots>(oc.H, cap), oc.tbits);
+  return insert_occurrence<KW, TS>(v, cap, oc, g, cap);
 }
 
 template <int KW, int TS>
@@ -3069,21 +3076,36 @@ __device__ __forceinline__ bool list_complete(const RunView& v) {
   return *(volatile unsigned int*)&v.hdr->round_listed && !*(volatile unsigned int*)&v.hdr->cand_overflow;
 }
 
+// Slots tried by an insert into the one table that stands in for full parts: a
+// cluster of 2^20 taken slots is to be expected from a load of 0.993 on. A reserve
+// too small for the round reports so after this, not after a walk of the whole table
+// for every k-mer that finds no room.
+constexpr uint64_t kWholeTries = 1ull << 20;
+
+__device__ __forceinline__ bool overflowed(const RunView& v) {
+  return *reinterpret_cast<volatile const unsigned int*>(&v.hdr->overflow);
+}
+
 // Algorithm 1, insert loop, second pass: every candidate ORs its in/out bases
 // (or the sentinel bit) into the exact table entry of its k-mer. Reads the
 // candidate list and keeps the slot of each listed candidate for the probe
-// loop; if the list overflowed, walks C_temp instead.
-template <int KW, int TS>
+// loop; if the list overflowed, walks C_temp instead. AFTER_PARTS: of a run whose
+// pass 2 goes on the records; this kernel then has the rounds that did not fit and
+// those with a full part.
+template <int KW, int TS, bool AFTER_PARTS = false>
 __global__ void __launch_bounds__(kBlock) pass2_insert_kernel(RunView v) {
   if (pass2_done(v)) return;
   const uint64_t cap = *(volatile unsigned long long*)&v.hdr->table_slots;
+  uint64_t tries = cap;
+  if (AFTER_PARTS && ordered_round(v)) tries = min(cap, kWholeTries);
   if (list_complete(v)) {
     for_listed(v, [&](uint64_t i) {
       bool sent;
       const uint64_t g = list_at(v, i, &sent, false);
       OccT<KW> oc;
       read_listed<KW>(v, g, sent, &oc);
-      const uint64_t slot = insert_occurrence<KW, TS>(v, cap, oc, g);
+      uint64_t slot = kNoSlot;
+      if (!AFTER_PARTS || !overflowed(v)) slot = insert_occurrence<KW, TS>(v, cap, oc, g, tries);
       if (slot == kNoSlot) v.hdr->overflow = 1;
       if (v.cand_slot) v.cand_slot[i] = slot == kNoSlot ? 0xFFFFFFFFu : (uint32_t)slot;
     });
@@ -3092,9 +3114,10 @@ __global__ void __launch_bounds__(kBlock) pass2_insert_kernel(RunView v) {
   const uint64_t stride = (uint64_t)gridDim.x * kBlock;
   for (uint64_t g = v.p_begin + (uint64_t)blockIdx.x * kBlock + threadIdx.x; g < v.p_end; g += stride) {
     if (!((__ldg(v.ctemp + (g >> 5)) >> (g & 31)) & 1u)) continue;
+    if (AFTER_PARTS && overflowed(v)) return;
     OccT<KW> oc;
     if (!read_occurrence<KW>(v, g, &oc)) continue;
-    if (insert_occurrence<KW, TS>(v, cap, oc, g) == kNoSlot) v.hdr->overflow = 1;
+    if (insert_occurrence<KW, TS>(v, cap, oc, g, tries) == kNoSlot) v.hdr->overflow = 1;
   }
 }
 
@@ -3108,6 +3131,7 @@ __global__ void __launch_bounds__(kBlock) pass2_insert_kernel(RunView v) {
 template <int KW, int TS>
 __global__ void __launch_bounds__(kBlock) pass2_classify_kernel(RunView v) {
   if (pass2_done(v)) return;
+  if (v.o_fused && __syncthreads_or(overflowed(v))) return;  // no table to go by
   const uint64_t cap = *(volatile unsigned long long*)&v.hdr->table_slots;
   unsigned long long found = 0;
   auto mark = [&](uint64_t g, int mk) {
@@ -3978,7 +4002,10 @@ static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges*
     launched += 2;
   }
   // pass 2: one resident wave; the warps share out the list's segment parts
-  const unsigned g2 = grid_for(pass2_insert_kernel<KW, TS>, kBlock, ~0ull >> 1, v.blocks_per_sm);
+  auto insert = pass2_insert_kernel<KW, TS>;
+  if constexpr (KW == 1 && kOrdOk)
+    if (v.o_fused) insert = pass2_insert_kernel<KW, TS, true>;
+  const unsigned g2 = grid_for(insert, kBlock, ~0ull >> 1, v.blocks_per_sm);
   const unsigned g3 = grid_for(pass2_classify_kernel<KW, TS>, kBlock, ~0ull >> 1, v.blocks_per_sm);
   {
     Timed t("pass2_insert", s);
@@ -3986,7 +4013,7 @@ static int round_impl(const RunView& v, int round, cudaStream_t s, const Ranges*
       RunView x = part(r);
       x.n_segments = pv.n_segments;
       x.seg_cap = pv.seg_cap;
-      pass2_insert_kernel<KW, TS><<<g2, kBlock, 0, s>>>(x);
+      insert<<<g2, kBlock, 0, s>>>(x);
       ++launched;
     }
   }

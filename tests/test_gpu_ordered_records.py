@@ -98,11 +98,12 @@ def test_a_full_part_of_the_table_takes_one_table(k, rounds, extra):
     run.release_plan()
 
 
-def test_a_full_reserve_is_reported_and_recovered():
-    """Half the slots: the parts fill up and the one table too. The run says so, and the host
-    build grows the reserve and runs again, on the records."""
-    bases, off = _full_parts(25, 1)
-    opts = T().Options(hashes=4, bucket_inserts=1, table_slots=1 << 17)
+@pytest.mark.parametrize("n,slots", [(259_000, 1 << 17), (3_000_000, 1 << 21), (3_000_000, 1 << 20)])
+def test_a_full_reserve_is_reported_and_recovered(n, slots):
+    """Fewer slots than k-mers: the parts fill up and the one table too. The run says so, and
+    the host build grows the reserve and runs again, on the records."""
+    bases, off = G.concat(G.random_strings(5, 1, n, n) + [np.frombuffer(b"ACGT" * 40, np.uint8)])
+    opts = T().Options(hashes=4, bucket_inserts=1, table_slots=slots)
     run = T().DeviceBuild(bases, off, 25, 1 << 16, 1, opts)
     run.run()
     st = run.stats(check=False)
@@ -110,4 +111,4 @@ def test_a_full_reserve_is_reported_and_recovered():
     seqs = [bases[int(off[t]):int(off[t + 1])] for t in range(len(off) - 1)]
     got, st = T().twopaco_build_ex(seqs, 25, 1 << 16, 1, opts)
     _eq(got, O.junctions((bases, off), 25))
-    assert st["table_slots"] == 1 << 19 and st["ordered_rounds"] == 1
+    assert st["table_slots"] == 4 * slots and st["ordered_rounds"] == 1
