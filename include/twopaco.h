@@ -537,7 +537,10 @@ int twopaco_edges_ctx(twopaco_context* ctx, twopaco_edge_list* out);
 /* Which internal state twopaco_read_state copies out. */
 #define TWOPACO_STATE_CANDIDATES 0 /* C_temp of the last round: ceil(total_bases/32) uint32 words */
 #define TWOPACO_STATE_JUNCTIONS 1  /* C_final: ceil(total_bases/32) uint32 words */
-#define TWOPACO_STATE_BINS 2       /* partition counters e_i (rounds > 1): q uint32 */
+#define TWOPACO_STATE_BINS 2       /* partition counters e_i (rounds > 1): q uint32. From 2^23
+                                      bases on they count a sample of the k-mers: of some
+                                      chunks of 65536 positions, the k-mers with some hash
+                                      bits zero */
 #define TWOPACO_STATE_CUTS 3       /* class boundaries: rounds + 1 uint32 */
 
 /*

@@ -349,6 +349,14 @@ RunView make_view(const uint8_t* d_bases, const uint64_t* d_offsets, uint64_t n_
   if ((m >> chunk_log2) < (1ull << 23)) sample_log2 = 0;
   v.part_chunks = (1u << chunk_log2) - 1u;
   v.part_sample = ((1ull << sample_log2) - 1ull) << std::max(16, log2_exact(o.partition_bins));
+  // A sample with too few k-mers (chunks of N or of strings shorter than k, long repeats)
+  // would cut classes of any size: the pre-pass then goes on over every k-mer up to 2^29
+  // bases, and over a 2^-floor(log2(m / 2^28)) of them, of every fourth chunk from 2^33
+  // bases, above.
+  int all_log2 = 0;
+  while (all_log2 < 8 && (m >> (28 + all_log2 + 1)) > 0) ++all_log2;
+  v.part_chunks_all = m >= (1ull << 33) ? 3u : 0u;
+  v.part_sample_all = ((1ull << all_log2) - 1ull) << std::max(16, log2_exact(o.partition_bins));
   v.hdr = reinterpret_cast<DevHeader*>(base + L.header);
   v.packed = reinterpret_cast<uint32_t*>(base + L.packed);
   v.packed_words = L.packed_words;

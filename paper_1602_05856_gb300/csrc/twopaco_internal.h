@@ -59,6 +59,7 @@ struct DevHeader {
   unsigned int ord_ok;              // region-ordered first pass: this round's records fit
   unsigned int ord_ticket[4];       // region-ordered passes: apply, probe, classify and insert work items
   unsigned int ord_rounds;          // rounds the region-ordered kernels took
+  unsigned long long part_counted;  // k-mers the partition pre-pass counted in its sample
 };
 
 // Device view of one run: every buffer lives inside the workspace except the
@@ -83,6 +84,8 @@ struct RunView {
                             // (next to the bin's, from bit 16 up) all zero (0: every k-mer)
   uint32_t part_chunks;     // ... and walks the chunks of 65536 positions whose index has these
                             // bits zero (0: every chunk)
+  uint64_t part_sample_all; // the same two where that sample came short of kPartMin k-mers
+  uint32_t part_chunks_all;
   DevHeader* hdr;
   uint32_t* packed;         // 2-bit packed input, ceil(m/16) + pad words
   uint64_t packed_words;    // words written by the pack kernel (incl. pad)
@@ -172,6 +175,7 @@ constexpr uint32_t kMinBuckets = 256;      // buckets of bucketed inserts, at le
 constexpr uint32_t kMaxBuckets = 1024;
 constexpr int kRegionWordsLog2 = 22;       // 32 MiB regions (words of 8 bytes)
 constexpr uint32_t kCmWindowPositions = 512;  // positions per class-map window (one warp's)
+constexpr unsigned long long kPartMin = 1ull << 17;  // k-mers the partition pre-pass wants to have counted
 constexpr uint64_t kOrdTile = 16384;       // region-ordered first pass: positions per tile
 constexpr uint32_t kOrdMaxRegions = 256;   // buckets (filter regions), at most
 constexpr uint32_t kOrdMaxHist = 4096;     // rounds x regions, at most
@@ -221,6 +225,7 @@ int launch_round_2(const RunView& v, int round, int rounds, cudaStream_t s, cons
 int launch_round_3(const RunView& v, int round, int rounds, cudaStream_t s, const PartRanges* ranges);
 int launch_round_4(const RunView& v, int round, int rounds, cudaStream_t s, const PartRanges* ranges);
 int launch_round_5(const RunView& v, int round, int rounds, cudaStream_t s, const PartRanges* ranges);
+// (the counts: kernels launched, or -1)
 int launch_count_1(const RunView& v, cudaStream_t s);
 int launch_count_2(const RunView& v, cudaStream_t s);
 int launch_count_3(const RunView& v, cudaStream_t s);

@@ -3167,25 +3167,36 @@ __global__ void __launch_bounds__(kBlock) pass2_classify_kernel(RunView v) {
 
 // Partition counters (section "Multiple Rounds"): a Bloom pre-pass over all
 // k-mers; counter f(k-mer) grows when the k-mer was not yet in the filter. On
-// large inputs only a hash-chosen sample of the k-mers is counted (bits of H
-// that neither the bin nor the filter block uses): every bin's count then
-// shrinks by the same factor in expectation, which keeps the cut's balance
-// while the random filter accesses drop by that factor.
+// large inputs only a hash-chosen sample of the k-mers of some of the chunks is
+// counted (bits of H that neither the bin nor the filter block uses): every bin's
+// count then shrinks by the same factor in expectation, which keeps the cut's balance
+// while the random filter accesses drop by that factor. What balances the cut is
+// the number of k-mers counted, and what a chunk holds is the input's choice: the
+// second launch (all) counts the rest where the sample came short of kPartMin
+// (2^17 k-mers: a class of 4 to 0.5%, of 64 to 2.2%), and returns at once otherwise.
 template <int KW, int HB>
-__global__ void __launch_bounds__(kBlock) partition_count_kernel(RunView v) {
+__global__ void __launch_bounds__(kBlock) partition_count_kernel(RunView v, int all) {
+  if (all && __ldcg(&v.hdr->part_counted) >= kPartMin) return;
+  const uint32_t chunks = all ? v.part_chunks_all : v.part_chunks;
+  const uint64_t sample = all ? v.part_sample_all : v.part_sample;
   const uint64_t stride = (uint64_t)gridDim.x * kBlock * kR;
+  uint32_t counted = 0;
   for (uint64_t p0 = ((uint64_t)blockIdx.x * kBlock + threadIdx.x) * kR; p0 < v.m; p0 += stride) {
-    if ((uint32_t)(p0 >> 16) & v.part_chunks) continue;  // a sample of the 64K-position chunks
+    if ((uint32_t)(p0 >> 16) & chunks) continue;  // a sample of the 64K-position chunks
     walk<KW, kR, true>(v, p0, [&](int, uint64_t, bool valid, const auto& oc) {
-      if (!valid || (oc.H & v.part_sample)) return;
+      if (!valid || (oc.H & sample)) return;
       const uint64_t G = second_hash(oc.H);
       const uint64_t m = item_bits<HB>(G, 17u, v.hashes);
       unsigned long long* w = filter_word(v, oc.H, G);
       if ((__ldcg(w) & m) == m) return;
       const unsigned long long old = atomicOr(w, (unsigned long long)m);
-      if ((old & m) != m) atomicAdd(v.bins + ((uint32_t)oc.H & v.qmask), 1u);
+      if ((old & m) != m) {
+        atomicAdd(v.bins + ((uint32_t)oc.H & v.qmask), 1u);
+        ++counted;
+      }
     });
   }
+  if (!all) block_add((unsigned long long)counted, &v.hdr->part_counted);
 }
 
 // Greedy class cut over the q counters: class r takes a maximal run of bins
@@ -4051,11 +4062,14 @@ static int part_round(const RunView& v, int round, int rounds, cudaStream_t s, c
 
 static int part_count(const RunView& v, cudaStream_t s) {
   const uint64_t threads = (v.m + kR - 1) / kR;
+  const bool sampled = v.part_chunks || v.part_sample;
   with_hashes(v.hashes, [&](auto hb) {
     auto kern = partition_count_kernel<kPartKw, decltype(hb)::value>;
-    kern<<<grid_for(kern, kBlock, threads), kBlock, 0, s>>>(v);
+    const unsigned grid = grid_for(kern, kBlock, threads);
+    kern<<<grid, kBlock, 0, s>>>(v, 0);
+    if (sampled) kern<<<grid, kBlock, 0, s>>>(v, 1);
   });
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
+  return cudaPeekAtLastError() == cudaSuccess ? (sampled ? 2 : 1) : -1;
 }
 
 // The parts' entry points, one set per translation unit.
@@ -4110,22 +4124,23 @@ int launch_partition(const RunView& v, int rounds, cudaStream_t s) {
   if (v.m == 0) return 0;
   // the filter is clear (pack kernel); the pre-pass uses it, round 0 clears it again
   if (cudaMemsetAsync(v.bins, 0, (uint64_t)(v.qmask + 1u) * 4, s) != cudaSuccess) return -1;
+  int counts;
   {
     Timed t("partition_count", s);
     const int part = part_of(v);
-    const int rc = part == 1   ? launch_count_1(v, s)
-                   : part == 2 ? launch_count_2(v, s)
-                   : part == 3 ? launch_count_3(v, s)
-                   : part == 4 ? launch_count_4(v, s)
-                               : launch_count_5(v, s);
-    if (rc < 0) return -1;
+    counts = part == 1   ? launch_count_1(v, s)
+             : part == 2 ? launch_count_2(v, s)
+             : part == 3 ? launch_count_3(v, s)
+             : part == 4 ? launch_count_4(v, s)
+                         : launch_count_5(v, s);
+    if (counts < 0) return -1;
   }
   uint64_t* prefix = reinterpret_cast<uint64_t*>(v.bins + (v.qmask + 1u));
   {
     Timed t("partition_cut", s);
     partition_cut_kernel<<<1, 1024, 0, s>>>(v, rounds, prefix);
   }
-  return done(2);
+  return done(counts + 1);
 }
 
 int launch_class_map(const RunView& v, cudaStream_t s) {
