@@ -116,8 +116,9 @@ typedef struct twopaco_options {
                               (k <= 63, hashes <= 6) takes the passes in filter-region order
                               that ordered_first_pass describes, in its one round, for filters
                               of more than 64 MiB with at least 4 positions per 32-byte filter
-                              sector; 1: for any filter; 2: never; in either case only where
-                              the workspace is at most 8 GiB larger for it. Where those passes
+                              sector (128 MiB: 9, with partial 6, for k >= 32 16); 1: for any
+                              filter; 2: never; in either case only where the workspace is at
+                              most 8 GiB larger for it. Where those passes
                               do not go (k > 63, per_string_launches, ordered_first_pass = 2,
                               the workspace) the ORs
                               alone go through region buckets: each becomes an 8-byte record

@@ -149,8 +149,15 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
   const bool want_bkt =
       o.bucket_inserts == 1 || (o.bucket_inserts == 0 && beyond_l2 && per_chunk >= 16 * (filter_bits / 256));
   // the ordered passes from 4 ORs per sector on: they read every region once and
-  // write it back, however few records it takes
-  const bool dense = beyond_l2 && per_round >= 4 * (filter_bits / 256);
+  // write it back, however few records it takes. In one round a filter of 128 MiB,
+  // which L2 nearly holds, takes the direct passes well, and the ordered ones pay only
+  // from 9 ORs per sector on (6 without pass 2, 16 with two-word k-mers): k = 25, 8 per
+  // sector (34 M positions) 1.08 ms direct and 1.25 ordered, 10 (42 M) 1.38 and 1.45,
+  // 16 (67 M) 2.13 and 2.08; k = 63, 15 (64 M) 2.10 and 2.19, 16 (67 M) 2.31 and 2.29;
+  // partial, k = 25, 6 (25 M) 0.72 and 0.71; but 256 MiB and 4 (35 M) 1.83 and 1.34
+  uint64_t per_sector = 4;
+  if (rounds == 1 && filter_bits / 8 == (128ull << 20)) per_sector = k > 31 ? 16 : (o.partial ? 6 : 9);
+  const bool dense = beyond_l2 && per_round >= per_sector * (filter_bits / 256);
   // region-ordered first pass: k <= 63, h <= 6, one launch per loop, at most
   // kOrdMaxRegions regions of at most 2^22 words and at most kOrdMaxHist
   // (round, region) counters; automatically for filters beyond L2 that a round

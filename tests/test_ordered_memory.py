@@ -1,5 +1,5 @@
-"""The workspace that the region-ordered passes may ask for without being asked by name
-(host only)."""
+"""Where the region-ordered passes go without being asked for by name: the workspace that
+they may take, and the filters about as large as L2 (host only)."""
 import random
 
 import pytest
@@ -62,3 +62,19 @@ def test_sizes_within_the_bound_stay_ordered():
 def test_asked_for_by_name_the_small_runs_fit_the_allocation_free_scratch(m, k, lg, rounds, kw):
     """Runs just within the 32 MiB with 64 regions, a class byte and a region byte per position."""
     assert _ws(m, 1 << lg, rounds, k=k, ordered_first_pass=1, **kw) <= 32 << 20
+
+
+@pytest.mark.parametrize("k,partial,least", [(25, False, 9), (31, False, 9), (25, True, 6), (32, False, 16), (63, True, 16)])
+def test_one_round_with_a_filter_about_as_large_as_l2(k, partial, least):
+    """A 128 MiB filter, nearly in L2: one-round runs below so many positions per 32-byte sector
+    are faster direct (17 M positions, k = 25: 0.60 ms direct, 0.75 ordered)."""
+    def ordered(m, lg, rounds=1):
+        kw = dict(k=k, partial=partial)
+        return _ws(m, 1 << lg, rounds, **kw) != _ws(m, 1 << lg, rounds, ordered_first_pass=2, **kw)
+
+    sectors = 1 << 22
+    assert not ordered(4 * sectors, 30) and not ordered(least * sectors - 1, 30)
+    assert ordered(least * sectors, 30) and ordered(338_000_000, 30)
+    # larger filters, and several rounds: from 4 on
+    assert ordered(8 * sectors, 31) and not ordered(8 * sectors - 1, 31)
+    assert ordered(8 * sectors, 30, 2)
