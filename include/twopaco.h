@@ -69,8 +69,10 @@ typedef struct twopaco_options {
   uint64_t table_slots;    /* pass-2 table reserve in slots (rounded up to a power of two);
                               0 = automatic. A round sizes its table from an estimate of its
                               distinct candidates, within the reserve; pass 2 on ordered
-                              records (ordered_first_pass) uses the whole reserve, one part
-                              per filter region. At least 4 */
+                              records (ordered_first_pass) splits the reserve, one part per
+                              filter region: all of it, or with fewer than 16 of a round's
+                              positions per 32-byte filter sector at most 1.25 slots per
+                              position. At least 4 */
   uint64_t candidate_records; /* pass-2 candidate list size in 8-byte units; 0 =
                                  automatic (half a round's positions). It
                                  holds twice as many candidates when the input has

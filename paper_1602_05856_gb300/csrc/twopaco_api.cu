@@ -152,8 +152,8 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
   // write it back, however few records it takes. In one round a filter of 128 MiB,
   // which L2 nearly holds, takes the direct passes well, and the ordered ones pay only
   // from 9 ORs per sector on (6 without pass 2, 16 with two-word k-mers): k = 25, 8 per
-  // sector (34 M positions) 1.08 ms direct and 1.25 ordered, 10 (42 M) 1.38 and 1.45,
-  // 16 (67 M) 2.13 and 2.08; k = 63, 15 (64 M) 2.10 and 2.19, 16 (67 M) 2.31 and 2.29;
+  // sector (34 M positions) 1.08 ms direct and 1.25 ordered, 10 (42 M) 1.38 and 1.37,
+  // 15 (64 M) 2.04 and 1.95; k = 63, 15 (64 M) 2.10 and 2.19, 16 (67 M) 2.31 and 2.29;
   // partial, k = 25, 6 (25 M) 0.72 and 0.71; but 256 MiB and 4 (35 M) 1.83 and 1.34
   uint64_t per_sector = 4;
   if (rounds == 1 && filter_bits / 8 == (128ull << 20)) per_sector = k > 31 ? 16 : (o.partial ? 6 : 9);
@@ -201,7 +201,15 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
       // square root). Regions of whole blocks only: a smaller one is named by bits of
       // the second hash too, and two bits of H would be neither in the record nor in
       // its bucket (filters of 2^12 and 2^13 bits)
-      const uint64_t tcap = L.table_slots / R;
+      // A round clears all parts. With less than 16 positions per filter sector the filter
+      // shows few k-mers as candidates that are none, and the parts together take a slot
+      // for every record and no more (an automatic reserve is two to four per position:
+      // 42 M positions with a 2^30-bit filter 1.45 -> 1.37 ms, where the direct passes take
+      // 1.38). A filled filter keeps nearly all k-mers and wants the load low: 340 M
+      // positions of unrelated strings with 2^30 bits took 21.3 ms so, and 16.9 with all
+      // of the reserve.
+      const bool sparse = per_round < 16 * (filter_bits / 256);
+      const uint64_t tcap = (sparse ? std::min(L.table_slots, L.o_rec_cap) : L.table_slots) / R;
       if (k <= 31 && !o.partial && R >= 64 && rw >= 4 && tcap >= 1024 && tcap < (1ull << 32)) {
         L.o_fused = 1;
         L.o_tcap = (uint32_t)tcap;

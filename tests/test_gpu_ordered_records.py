@@ -112,3 +112,21 @@ def test_a_full_reserve_is_reported_and_recovered(n, slots):
     got, st = T().twopaco_build_ex(seqs, 25, 1 << 16, 1, opts)
     _eq(got, O.junctions((bases, off), 25))
     assert st["table_slots"] == 4 * slots and st["ordered_rounds"] == 1
+
+
+@pytest.mark.parametrize("k,rounds", [(25, 1), (31, 1), (28, 4)])
+def test_a_sparse_filter_takes_a_slot_per_record(k, rounds):
+    """With fewer than 16 positions per filter sector the parts of the table take 1.25 slots per
+    position, whatever the reserve (a round clears them all); a filled filter takes it all."""
+    bases, off = G.concat(G.named_set("plain_single", 0.05))
+    m = int(off[-1])
+    want = O.junctions((bases, off), k)
+    for lg, all_of_it in ((26, False), (18, True)):
+        run = T().DeviceBuild(bases, off, k, 1 << lg, rounds,
+                              T().Options(partition_bins=256, table_slots=1 << 22, bucket_inserts=1,
+                                          ordered_first_pass=int(rounds > 1)))
+        run.run()
+        st = run.stats()
+        assert st["ordered_rounds"] == rounds
+        assert st["table_slots"] == 1 << 22 if all_of_it else st["table_slots"] <= 2 * m
+        _eq(run.result(), want)
