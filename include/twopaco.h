@@ -113,23 +113,24 @@ typedef struct twopaco_options {
                               the batched launch). The call reads the string offsets
                               back and synchronises the stream; twopaco_plan_create
                               refuses it. 0 (default): one launch per loop. */
-  int bucket_inserts;      /* one-round runs with a filter beyond L2, which takes random ORs
-                              and probes at DRAM's random-access rate. 0 (default): such a run
-                              (k <= 63, hashes <= 6) takes the passes in filter-region order
-                              that ordered_first_pass describes, in its one round, for filters
-                              of more than 64 MiB with at least 4 positions per 32-byte filter
-                              sector (128 MiB: 9, with partial 6, for k >= 32 16); 1: for any
-                              filter; 2: never; in either case only where the workspace is at
-                              most 8 GiB larger for it. Where those passes
-                              do not go (k > 63, per_string_launches, ordered_first_pass = 2,
-                              the workspace) the ORs
-                              alone go through region buckets: each becomes an 8-byte record
-                              in the bucket of its filter region (32 MiB, or a quarter of a
-                              smaller filter), and the records are applied region by region
-                              while each region sits in L2; the positions go through in chunks
-                              that fill the buckets (records for a round's positions and a
-                              quarter more, at most 2^31) to about 80%, and a full bucket
-                              takes the OR directly -- 0: from 16 ORs of a chunk per filter
+  int bucket_inserts;      /* filters beyond L2, which take random ORs and probes at DRAM's
+                              random-access rate. In one round it chooses the passes in
+                              filter-region order that ordered_first_pass describes (k <= 63,
+                              hashes <= 6): 0 (default) for filters of more than 64 MiB with
+                              at least 4 positions per 32-byte filter sector (128 MiB: 9, with
+                              partial 6, for k >= 32 16); 1: for any filter; 2: never; in any
+                              case only where the workspace is at most 8 GiB larger for it.
+                              Where those passes do not go, in one round (k > 63,
+                              per_string_launches, ordered_first_pass = 2, the workspace) or
+                              in several (the same, or a filter that ordered_first_pass = 0
+                              leaves out), it chooses region buckets for the ORs alone: each
+                              becomes an 8-byte record in the bucket of its filter region (32
+                              MiB, or a quarter of a smaller filter), and the records are
+                              applied region by region while each region sits in L2; the
+                              positions go through in chunks that fill the buckets (records
+                              for a round's positions and a quarter more, at most 2^31) to
+                              about 80%, and a full bucket takes the OR directly -- 0: for
+                              filters of more than 64 MiB from 16 ORs of a chunk per filter
                               sector on; 1: for any filter; 2: never. Same results. Buckets
                               need hashes <= 6 and a filter of at most 2^38 bits (else the ORs
                               are direct). */

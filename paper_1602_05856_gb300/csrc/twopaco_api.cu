@@ -141,9 +141,9 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
   L.cand_cap = o.candidate_records ? o.candidate_records
                                    : (per_round / 2 > (1u << 16) ? per_round / 2 : (1u << 16));
   if (o.partial) L.cand_cap = 0;
-  // region-bucketed first-pass inserts of a one-round run: a filter beyond L2 (over
-  // 64 MiB) with at least 16 ORs of a chunk on every 32-byte filter sector on
-  // average, or any filter when asked
+  // region-bucketed first-pass inserts, where the ordered passes do not go: a filter
+  // beyond L2 (over 64 MiB) with at least 16 ORs of a chunk on every 32-byte filter
+  // sector on average, or any filter when asked
   const bool beyond_l2 = filter_bits / 8 > (64ull << 20);
   const uint64_t per_chunk = std::min<uint64_t>(per_round, 1ull << 31) * 4 / 5;
   const bool want_bkt =

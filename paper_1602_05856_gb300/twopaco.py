@@ -180,7 +180,7 @@ class Options:
     wide_layout: int = 0      # 1/2: the large-input workspace layout at any size (testing)
     partial: bool = False     # omit pass 2: the partially compacted graph's positions
     per_string_launches: bool = False  # every loop launched once per string (a baseline)
-    bucket_inserts: int = 0   # one-round passes in filter-region order or buckets: 0 auto (> 64 MiB), 1 always, 2 never
+    bucket_inserts: int = 0   # one round in filter-region order, else ORs in region buckets: 0 auto (> 64 MiB), 1 always, 2 never
     launch_blocks_per_sm: int = 0  # launch shape of the pass kernels: resident blocks per SM (0: all)
     ordered_first_pass: int = 0    # passes in filter-region order: 0 auto (dense filters > 64 MiB, >= 1 GiB), 1 always, 2 never
 
