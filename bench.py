@@ -212,6 +212,22 @@ def max_over_ranks(x: float, world: int) -> float:
     return float(t.item())
 
 
+def partition_share(m):
+    """Share of the positions whose k-mers the partition pre-pass counts on m bases: of one chunk
+    of 65536 positions in 2^c (at least 2^24 positions walked), one k-mer in 2^s."""
+    c = s = 0
+    while c < 16 and (m >> (c + 1)) >= 1 << 24:
+        c += 1
+    while (m >> c) >= 1 << 23 and s < 8 and (m >> c >> (s + 1)) >= 1 << 21:
+        s += 1
+    return 1 / (1 << (c + s))
+
+
+def slot_bytes(k, on_records):
+    """Bytes of a pass-2 table slot (on_records: pass 2 ran on the ordered records)."""
+    return 8 if k <= 27 or k > 63 or (k <= 31 and on_records) else 16 if k <= 31 else 32
+
+
 # Algorithmic work of every kernel over one step, from the run's own counters:
 # (amount, kind) where kind names the roofline denominator: "rand_or" / "rand_read"
 # are random 64-bit atomic ORs / 8-byte loads into the structure the kernel hits
@@ -250,8 +266,8 @@ def kernel_work(name, st, m, n_seqs, table_bytes, rounds=1):
         return cand, "rand_or"      # one table slot (CAS / OR) per candidate
     if name == "pass2_classify":
         return cand, "rand_read"    # one table slot load per candidate
-    if name == "partition_count":
-        return pos, "rand_read"     # one random filter word test per position
+    if name == "partition_count":  # one random filter word test per counted k-mer
+        return pos * partition_share(m), "rand_read"
     if name == "pack":
         return m + m / 4, "hbm"     # ASCII read + packed write (bytes)
     if name == "class_map":
@@ -477,7 +493,7 @@ def device_leg(T, build, name, genome_len, rounds, args, world, rank, local, dis
     ms = statistics.mean(step_ms)
     ms_max = max_over_ranks(ms, world)
     junctions = int(run.out_offsets[-1].item()) if rank == 0 else st["pass2_marks"]
-    table_bytes = st["table_slots"] * (8 if K <= 27 else 16 if K <= 31 else 32)
+    table_bytes = st["table_slots"] * slot_bytes(K, st["ordered_rounds"] > 0)
     peaks_json = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) \
         if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else {}
     hbm_peak = float(peaks_json.get("hbm_gbs", 6800.0))

@@ -174,7 +174,6 @@ constexpr uint32_t kMaxRegions = 1024;     // filter regions of bucketed inserts
 constexpr uint32_t kMinBuckets = 256;      // buckets of bucketed inserts, at least (sub-buckets per region)
 constexpr uint32_t kMaxBuckets = 1024;
 constexpr int kRegionWordsLog2 = 22;       // 32 MiB regions (words of 8 bytes)
-constexpr uint32_t kCmWindowPositions = 512;  // positions per class-map window (one warp's)
 constexpr unsigned long long kPartMin = 1ull << 17;  // k-mers the partition pre-pass wants to have counted
 constexpr uint64_t kOrdTile = 16384;       // region-ordered first pass: positions per tile
 constexpr uint32_t kOrdMaxRegions = 256;   // buckets (filter regions), at most

@@ -98,8 +98,10 @@ struct Timed {
 // bases) in the first-pass kernels and the partition pre-pass.
 constexpr int kInsertR = 16;
 // Inputs below kInsertSmall positions take fewer per thread, so that all SMs
-// have warps to spare: 16 per thread left 0.2 M positions on 46 blocks (insert
-// 16 -> 10 us); at 3.8 M positions 16 are the better ones (126 us a build to 129).
+// have warps to spare: 16 per thread left 0.2 M positions on 46 blocks. Whole builds at
+// k = 25 and 63, 16 against 4 per thread: 0.2 M positions 71.5 to 66.2 and 85.8 to 78.1 us,
+// 1 M 81.8 to 77.4 and 98.1 to 92.4, 2.1 M 92.2 to 90.2 and 125.1 to 125.2, 4 M 129.1 to 129.1
+// and 225.2 to 232.4, 6 M 187.3 to 188.8 and 444 to 453.
 constexpr int kInsertSmallR = 4;
 constexpr uint64_t kInsertSmall = 1ull << 21;
 constexpr int kProbeR = 8;
@@ -2300,7 +2302,7 @@ __device__ __forceinline__ TileMembers ord_tile(const RunView& v, uint64_t t, in
 // the integer pipe (79% of its peak); reading the tile's packed words through
 // shared memory, which took L1 from 71% to 45%, changed nothing.
 template <int KW, int HB, bool FUSED>
-__global__ void __launch_bounds__(kBlock) ord_scatter_kernel(RunView v, int round) {
+__global__ void __launch_bounds__(kBlock) tile_scatter_kernel(RunView v, int round) {
   __shared__ uint8_t bucket_s[kOrdTile];
   __shared__ unsigned long long delta_s[kOrdMaxRegions];
   __shared__ uint64_t start_s[kOrdMaxRegions];
@@ -2776,7 +2778,7 @@ __device__ __forceinline__ uint32_t ord_tile_positions(const RunView& v, uint64_
 // class takes its decision from its record's slot -- the members of a run read
 // consecutive bits -- and sets its bits of the tile in shared memory; then the
 // tile's words, list entries and counts go out (ord_tile_out).
-__global__ void __launch_bounds__(kBlock) ord_gather_kernel(RunView v, int round) {
+__global__ void __launch_bounds__(kBlock) tile_gather_kernel(RunView v, int round) {
   __shared__ uint8_t bucket_s[kOrdTile];
   __shared__ unsigned long long delta_s[kOrdMaxRegions];
   __shared__ uint64_t start_s[kOrdMaxRegions];
@@ -2954,9 +2956,12 @@ __global__ void __launch_bounds__(1024) table_setup_kernel(RunView v) {
     // candidate list)
     const unsigned long long part = (cap / v.o_regions + 64 + 3) / 4 * 4;
     // worth it where the table is far beyond L2 and the candidates are not a small
-    // share of the members, which all have to be looked at: 62 genomes at k = 63 (65%
-    // of 312 M, 6 GB) 21.2 -> 11.5 ms with the gather, but 800 Mbp at k = 31 (12%, 141
-    // MB) 6.3 -> 12.3 ms
+    // share of the members, which all have to be looked at. Builds at k = 63, list against
+    // parts: a table of 0.5-0.6 GB at shares of 10, 12 and 100% 9.7 to 10.6, 9.9 to 10.7 and
+    // 1.59 to 1.26 ms; 100% at 212 and 304 MB 0.66 to 0.73 and 1.10 to 1.02; 14, 19, 27 and 32%
+    // at 1.0, 1.8, 3.3 and 4.7 GB 11.0 to 11.3, 12.9 to 12.3, 16.0 to 13.9 and 18.5 to 15.3; 57%
+    // at 6 GB 25.5 to 18.5. The two meet near 300 MB and 16%: both lines are on the
+    // list's side of that.
     const bool pays = part * v.o_regions * (32 / SectorOf<TS>::kSlots) > kPartTableBytes && 4 * kept >= v.o_start[v.o_regions];
     if (pays && part * v.o_regions <= v.table_max_slots) {
       h->part_slots = part;
@@ -3846,9 +3851,9 @@ static int ordered_round_impl(const RunView& v, int round, cudaStream_t s, RunVi
   }
   {
     Timed t("tile_scatter", s);
-    auto kern = ord_scatter_kernel<KW, HB, false>;
+    auto kern = tile_scatter_kernel<KW, HB, false>;
     if constexpr (KW == 1)
-      if (fused) kern = ord_scatter_kernel<KW, HB, true>;
+      if (fused) kern = tile_scatter_kernel<KW, HB, true>;
     kern<<<grid_for(kern, kBlock, v.o_tiles * kBlock, v.blocks_per_sm), kBlock, 0, s>>>(v, round);
   }
   {
@@ -3862,7 +3867,7 @@ static int ordered_round_impl(const RunView& v, int round, cudaStream_t s, RunVi
     kern<<<grid_for(kern, kBlock, v.o_tiles * kBlock, v.blocks_per_sm), kBlock, 0, s>>>(v, round);
   }
   // one candidate-list segment per warp of the gather (and of the direct probe)
-  unsigned grid = std::min(grid_for(ord_gather_kernel, kBlock, v.o_tiles * kBlock, v.blocks_per_sm),
+  unsigned grid = std::min(grid_for(tile_gather_kernel, kBlock, v.o_tiles * kBlock, v.blocks_per_sm),
                            grid_for(list_probe_kernel<KW, HB>, kBlock, v.o_tiles * kBlock, v.blocks_per_sm));
   grid = std::min(grid, (unsigned)(kMaxSegments / (kBlock / 32)));
   pv->n_segments = grid * (kBlock / 32);
@@ -3902,7 +3907,7 @@ static int ordered_round_impl(const RunView& v, int round, cudaStream_t s, RunVi
   }
   {
     Timed t("tile_gather", s);
-    ord_gather_kernel<<<grid, kBlock, 0, s>>>(*pv, round);
+    tile_gather_kernel<<<grid, kBlock, 0, s>>>(*pv, round);
   }
   return launched + 1;
 }
