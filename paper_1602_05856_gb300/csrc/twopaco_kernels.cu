@@ -881,6 +881,12 @@ constexpr uint64_t kNoSlot = ~0ull;
 // k-mer mostly costs one round trip. Slot by slot from any start, the longest
 // of a warp's 32 chains -- six to eight slots at a load of 0.4 -- cost one each,
 // and the rest of the warp its instructions. Tables hold whole sectors.
+// That is for tables of up to about twice L2: larger ones (kSectorSlots) are probed slot
+// by slot, from a k-mer's very slot, as the two loads of a sector are two misses in
+// flight for one there. Pass-2 inserts, by sectors and by slots: one-word slots at 195 MB
+// 502 and 545 us, 229 MB 634 and 680, 269 MB 800 and 734, 390 MB 1932 and 1359, 714 MB 4.60
+// and 3.20 ms; 16-byte slots at 243 MB 428 and 437 us, 347 MB 1080 and 817, 1.4 GB 7.07 and
+// 5.12 ms.
 template <int TS>
 struct SectorOf {
   static constexpr int kSlots = TS == 0 || TS == 3 ? 4 : (TS == 2 ? 1 : 2);
@@ -903,12 +909,41 @@ struct SectorOf {
   }
 };
 
-// Insert into the one-word slots T[0 .. cap), probing from the sector at i (a
-// multiple of 4 below cap): the key's slot, or kNoSlot if `tries` slots were tried
+template <int TS>
+constexpr uint64_t kSectorSlots = (256ull << 20) / (TS == 1 ? 16 : 8);
+
+// A table of cap slots is probed by sectors (else slot by slot; kinds 0 and 1 only).
+template <int TS>
+__device__ __forceinline__ bool by_sectors(uint64_t cap) {
+  return (TS != 0 && TS != 1) || cap <= kSectorSlots<TS>;
+}
+
+// Start slot of a k-mer in a pass-2 table of cap slots of kind TS.
+template <int TS>
+__device__ __forceinline__ uint64_t table_start(uint64_t H, uint64_t cap) {
+  const uint64_t i = slot_start<1>(H, cap);
+  return by_sectors<TS>(cap) ? i & ~(uint64_t)(SectorOf<TS>::kSlots - 1) : i;
+}
+
+// Insert into the one-word slots T[0 .. cap), probing from slot i (table_start; by
+// sectors a multiple of 4): the key's slot, or kNoSlot if `tries` slots were tried
 // (all of them: the table is full). Bits already present are not written again. A
 // word is key << 9 | mask bits; never all ones for a key < 2^54.
 __device__ __forceinline__ uint64_t word_insert(unsigned long long* T, uint64_t cap, uint64_t i, uint64_t key,
                                                 uint32_t bits, uint64_t tries) {
+  if (!by_sectors<0>(cap)) {
+    for (uint64_t seen = 0; seen < tries; ++seen, i = i + 1 == cap ? 0 : i + 1) {
+      unsigned long long cur = __ldcg(T + i);
+      if (cur == kEmpty) {
+        cur = atomicCAS(T + i, kEmpty, (key << kMaskBits) | bits);
+        if (cur == kEmpty) return i;
+      }
+      if ((cur >> kMaskBits) != key) continue;
+      if ((cur & bits) != bits) atomicOr(T + i, (unsigned long long)bits);
+      return i;
+    }
+    return kNoSlot;
+  }
   for (uint64_t seen = 0; seen < tries; seen += 4) {
     SectorOf<0> q;
     q.load(T, i);
@@ -942,6 +977,14 @@ __device__ __forceinline__ uint64_t word_insert(unsigned long long* T, uint64_t 
 
 // Mask of key in the one-word slots T[0 .. cap), or -1 if absent.
 __device__ __forceinline__ int word_find(const unsigned long long* T, uint64_t cap, uint64_t i, uint64_t key) {
+  if (!by_sectors<0>(cap)) {
+    for (uint64_t seen = 0; seen < cap; ++seen, i = i + 1 == cap ? 0 : i + 1) {
+      const unsigned long long cur = __ldcg(T + i);
+      if (cur == kEmpty) return -1;
+      if ((cur >> kMaskBits) == key) return (int)(cur & ((1u << kMaskBits) - 1u));
+    }
+    return -1;
+  }
   for (uint64_t seen = 0; seen < cap; seen += 4) {
     SectorOf<0> q;
     q.load(T, i);
@@ -960,8 +1003,7 @@ __device__ __forceinline__ int word_find(const unsigned long long* T, uint64_t c
 }
 
 // Insert (key, bits) into a table of cap TS-kind slots (table_slot_kind),
-// probing from the sector at start (below cap); the key's slot, or kNoSlot if
-// `tries` slots were tried (all of them: the table is full). Bits already present
+// probing from start (table_start); the key's slot, or kNoSlot if `tries` slots were tried (all of them: the table is full). Bits already present
 // are not written again.
 template <int TS>
 __device__ __forceinline__ uint64_t table_insert(const RunView& v, uint64_t cap, const Key& key,
@@ -971,6 +1013,25 @@ __device__ __forceinline__ uint64_t table_insert(const RunView& v, uint64_t cap,
   } else {
     constexpr uint64_t N = SectorOf<TS>::kSlots;
     uint64_t base = start;
+    if constexpr (TS == 1) {
+      if (!by_sectors<1>(cap)) {
+        for (uint64_t seen = 0; seen < tries; ++seen, base = base + 1 == cap ? 0 : base + 1) {
+          Slot1* s = static_cast<Slot1*>(v.table) + base;
+          const ulonglong2 w = __ldcg(reinterpret_cast<const ulonglong2*>(s));
+          unsigned long long cur = w.x;
+          uint32_t have = (uint32_t)w.y;
+          if (cur == kEmpty) {
+            cur = atomicCAS(&s->key, kEmpty, (unsigned long long)key.lo);
+            if (cur == kEmpty) cur = key.lo;
+            have = 0;
+          }
+          if (cur != key.lo) continue;
+          if ((have & bits) != bits) atomicOr(&s->mask, bits);
+          return base;
+        }
+        return kNoSlot;
+      }
+    }
     for (uint64_t seen = 0; seen < tries; seen += N) {
       SectorOf<TS> q;
       if constexpr (TS == 1) q.load(v.table, base);  // TS 2: the CAS itself is the first look
@@ -1010,6 +1071,16 @@ __device__ __forceinline__ int table_find(const RunView& v, uint64_t cap, const 
   } else {
     constexpr uint64_t N = SectorOf<TS>::kSlots;
     uint64_t base = start;
+    if constexpr (TS == 1) {
+      if (!by_sectors<1>(cap)) {
+        for (uint64_t seen = 0; seen < cap; ++seen, base = base + 1 == cap ? 0 : base + 1) {
+          const ulonglong2 w = __ldcg(reinterpret_cast<const ulonglong2*>(static_cast<const Slot1*>(v.table) + base));
+          if (w.x == key.lo) return (int)(uint32_t)w.y;
+          if (w.x == kEmpty) return -1;
+        }
+        return -1;
+      }
+    }
     for (uint64_t seen = 0; seen < cap; seen += N) {
       SectorOf<TS> q;
       q.load(v.table, base);
@@ -1099,7 +1170,7 @@ template <int KW, int TS>
 __device__ __forceinline__ uint64_t insert_occurrence(const RunView& v, uint64_t cap, const OccT<KW>& oc,
                                                       uint64_t g, uint64_t tries) {
   if constexpr (TS == 3) return table_insert_ref(v, cap, oc.key, oc.H, slot_start<4>(oc.H, cap), oc.tbits, g, oc.rc);
-  else return table_insert<TS>(v, cap, oc.key, slot_start<SectorOf<TS>::kSlots>(oc.H, cap), oc.tbits, tries);
+  else return table_insert<TS>(v, cap, oc.key, table_start<TS>(oc.H, cap), oc.tbits, tries);
 }
 
 template <int KW, int TS>
@@ -1111,7 +1182,7 @@ __device__ __forceinline__ uint64_t insert_occurrence(const RunView& v, uint64_t
 template <int KW, int TS>
 __device__ __forceinline__ int find_occurrence(const RunView& v, uint64_t cap, const OccT<KW>& oc) {
   if constexpr (TS == 3) return table_find_ref(v, cap, oc.key, oc.H);
-  else return table_find<TS>(v, cap, oc.key, slot_start<SectorOf<TS>::kSlots>(oc.H, cap));
+  else return table_find<TS>(v, cap, oc.key, table_start<TS>(oc.H, cap));
 }
 
 // Mask held by slot i (a slot that table_insert returned).
