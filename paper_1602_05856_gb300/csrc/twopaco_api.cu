@@ -358,9 +358,11 @@ RunView make_view(const uint8_t* d_bases, const uint64_t* d_offsets, uint64_t n_
   // s <= 8: 32 per bin of the default 65536, a class of ell = 4 to about 0.15%).
   // Every counted k-mer is a random atomic in a filter beyond L2: on 200 M bases
   // counting all of them took 4.2 ms of a 13.6 ms build.
+  // (k <= 8 has at most 2^16 k-mers, and an eighth of them mostly comes short of
+  // kPartMin a class: all are counted)
   int chunk_log2 = 0, sample_log2 = 0;
-  while (chunk_log2 < 16 && (m >> (chunk_log2 + 1)) >= (1ull << 24)) ++chunk_log2;
-  while (sample_log2 < 8 && ((m >> chunk_log2) >> (sample_log2 + 1)) >= (1ull << 21)) ++sample_log2;
+  while (k > 8 && chunk_log2 < 16 && (m >> (chunk_log2 + 1)) >= (1ull << 24)) ++chunk_log2;
+  while (k > 8 && sample_log2 < 8 && ((m >> chunk_log2) >> (sample_log2 + 1)) >= (1ull << 21)) ++sample_log2;
   if ((m >> chunk_log2) < (1ull << 23)) sample_log2 = 0;
   v.part_chunks = (1u << chunk_log2) - 1u;
   v.part_sample = ((1ull << sample_log2) - 1ull) << std::max(16, log2_exact(o.partition_bins));

@@ -84,7 +84,7 @@ struct RunView {
                             // (next to the bin's, from bit 16 up) all zero (0: every k-mer)
   uint32_t part_chunks;     // ... and walks the chunks of 65536 positions whose index has these
                             // bits zero (0: every chunk)
-  uint64_t part_sample_all; // the same two where that sample came short of kPartMin k-mers
+  uint64_t part_sample_all; // the same two where that sample came short of kPartMin k-mers a class
   uint32_t part_chunks_all;
   DevHeader* hdr;
   uint32_t* packed;         // 2-bit packed input, ceil(m/16) + pad words
@@ -174,7 +174,7 @@ constexpr uint32_t kMaxRegions = 1024;     // filter regions of bucketed inserts
 constexpr uint32_t kMinBuckets = 256;      // buckets of bucketed inserts, at least (sub-buckets per region)
 constexpr uint32_t kMaxBuckets = 1024;
 constexpr int kRegionWordsLog2 = 22;       // 32 MiB regions (words of 8 bytes)
-constexpr unsigned long long kPartMin = 1ull << 17;  // k-mers the partition pre-pass wants to have counted
+constexpr unsigned long long kPartMin = 1024;  // k-mers the partition pre-pass wants counted for each class
 constexpr uint64_t kOrdTile = 16384;       // region-ordered first pass: positions per tile
 constexpr uint32_t kOrdMaxRegions = 256;   // buckets (filter regions), at most
 constexpr uint32_t kOrdMaxHist = 4096;     // rounds x regions, at most

@@ -3248,11 +3248,11 @@ __global__ void __launch_bounds__(kBlock) pass2_classify_kernel(RunView v) {
 // count then shrinks by the same factor in expectation, which keeps the cut's balance
 // while the random filter accesses drop by that factor. What balances the cut is
 // the number of k-mers counted, and what a chunk holds is the input's choice: the
-// second launch (all) counts the rest where the sample came short of kPartMin
-// (2^17 k-mers: a class of 4 to 0.5%, of 64 to 2.2%), and returns at once otherwise.
+// second launch (all) counts the rest where the sample came short of kPartMin k-mers
+// a class (1024: a class to 3%), and returns at once otherwise.
 template <int KW, int HB>
 __global__ void __launch_bounds__(kBlock) partition_count_kernel(RunView v, int all) {
-  if (all && __ldcg(&v.hdr->part_counted) >= kPartMin) return;
+  if (all && __ldcg(&v.hdr->part_counted) >= kPartMin * (unsigned long long)v.rounds) return;
   const uint32_t chunks = all ? v.part_chunks_all : v.part_chunks;
   const uint64_t sample = all ? v.part_sample_all : v.part_sample;
   const uint64_t stride = (uint64_t)gridDim.x * kBlock * kR;
