@@ -209,7 +209,8 @@ Layout layout(uint64_t m, uint64_t n_seqs, int k, uint64_t filter_bits, int roun
       // positions of unrelated strings with 2^30 bits took 21.3 ms so, and 16.9 with all
       // of the reserve.
       const bool sparse = per_round < 16 * (filter_bits / 256);
-      const uint64_t tcap = (sparse ? std::min(L.table_slots, L.o_rec_cap) : L.table_slots) / R;
+      uint64_t tcap = L.table_slots / R;
+      if (sparse) tcap = std::min(tcap, std::max<uint64_t>(1024, L.o_rec_cap / R));
       if (k <= 31 && !o.partial && R >= 64 && rw >= 4 && tcap >= 1024 && tcap < (1ull << 32)) {
         L.o_fused = 1;
         L.o_tcap = (uint32_t)tcap;
